@@ -52,7 +52,7 @@ typedef enum {
 } mrc_status;
 
 typedef enum {
-    MRC_FP64 = 0,  /* every stage in IEEE binary64 on the FP64 pipes */
+    MRC_FP64 = 0,  /* binary64 data and accuracy in every stage (its arithmetic partly in 64-bit fixed point) */
     MRC_MIXED = 1  /* FP32 Newton + double-float (FP32-pair) residual refinement */
 } mrc_precision;
 

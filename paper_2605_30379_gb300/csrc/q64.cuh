@@ -1,0 +1,152 @@
+// q64.cuh -- 64-bit fixed-point arithmetic of the FP64 FFT passes.
+//
+// The FP64 pipe of this GPU issues two operations per clock and SM, the
+// integer pipes about thirty times as many (measured: DFMA 2, IMAD.WIDE 60,
+// 32-bit adds 90 per clock and SM), so a pass converts its points to
+// fixed-point numbers with one exponent per CTA and entry column, runs its
+// in-CTA stages in 64-bit integers and converts back on the store.
+//
+// Scaling.  A column's points (the R points of the pass at one entry) are
+// aligned to the largest exponent among them; the inputs of every stage of
+// radix 8 are kept below 2^57 (|re|, |im|; 2^59 in the last one), so that
+// its sums stay below 2^60.5 and fit the next twiddle products.  The shift
+// before a stage is taken from the magnitudes the previous stage left in the
+// column (block floating point): none where the values did not grow.  A
+// stage thus rounds at 2^-57 .. 2^-56 of the column's largest magnitude;
+// against 128-bit references, passes of 512 and 1024 points err 0.4 to 0.8
+// times as much (root mean square) as the same passes in FP64, for random,
+// decaying and constant-plus-decaying columns alike (with fixed divisions by
+// the radix instead of the measured ones: 0.7 to 7 times).
+//
+// Products.  A value a < 2^61 and a twiddle w <= 2^60 are split into a high
+// limb and a 30-bit low limb each (nonnegative for a, balanced for w); the
+// product takes the high and the two middle limb products (32 x 32 -> 64 bit
+// multiply-adds), the low one is below the rounding of the result.
+//
+// Every rounding is unbiased: a constant offset of the points would add up in
+// the zero frequency, which the inverse amplifies by N (e0 - q is singular
+// there).
+#pragma once
+#include "arith.cuh"
+
+struct q64 {
+    long long v;
+};
+// twiddle factor: Q60 limbs of its real and imaginary parts
+struct __align__(16) qtw {
+    int rh, rl, ih, il;
+};
+
+constexpr int Q_TOP = 60;
+constexpr int Q_MASK30 = (1 << 30) - 1;
+
+// biased exponent of a double (0 for zero and subnormals, 2047 for Inf / NaN)
+__device__ __forceinline__ int q_exponent(double x) { return (__double2hiint(x) >> 20) & 0x7ff; }
+
+// x 2^(top + 1022 - ex) rounded to an integer, for |x| < 2^(ex - 1022) and
+// top <= 60: the magnitude is rounded (symmetric in the sign, so that a column
+// of one sign is not shortened); neg flips the sign.
+__device__ __forceinline__ q64 q_decode(double x, int ex, int top, int neg = 0)
+{
+    const unsigned hw = (unsigned)__double2hiint(x), lw = (unsigned)__double2loint(x);
+    const int e = (int)((hw >> 20) & 0x7ffu);
+    const unsigned mh = (hw & 0xfffffu) | (e ? 0x100000u : 0u);
+    const int sh = min(ex - max(e, 1) + (62 - top), 63);
+    const unsigned long long m = (((((unsigned long long)mh << 42) | ((unsigned long long)lw << 10)) >> sh) + 1ull) >> 1;
+    const long long s = (long long)((int)hw >> 31) ^ (long long)neg;
+    return {((long long)m ^ s) - s};
+}
+
+// v 2^(eb - 1086) rounded to a double (flushed to zero below the normal
+// range, infinity above it): a value with leading bit 63 - lz gets the biased
+// exponent eb - lz.
+__device__ __forceinline__ double q_encode(q64 x, int eb, unsigned sgn)
+{
+    const long long s = x.v >> 63;
+    const unsigned long long a = (unsigned long long)((x.v ^ s) - s);
+    const int lz = __clzll((long long)a);
+    const unsigned long long n = a << (lz & 63);
+    const unsigned long long m = (n >> 11) + ((n >> 10) & 1ull);
+    const int e = eb - lz;
+    unsigned hi = (unsigned)(m >> 32) + ((unsigned)(e - 1) << 20), lo = (unsigned)m;
+    const bool tiny = e < 1 || a == 0ull;
+    hi = tiny ? 0u : hi;
+    lo = tiny ? 0u : lo;
+    if (e >= 2047) {
+        hi = a == 0ull ? 0u : 0x7ff00000u;
+        lo = 0u;
+    }
+    hi |= ((unsigned)s ^ sgn) & 0x80000000u;
+    return __hiloint2double((int)hi, (int)lo);
+}
+
+__device__ __forceinline__ long long q_wide(int a, int b, long long c) { return (long long)a * b + c; }
+
+// a w for a real factor w <= 2^60 (Q60)
+__device__ __forceinline__ long long q_mul(long long a, long long w)
+{
+    const int ah = (int)(a >> 30), al = (int)a & Q_MASK30, wh = (int)(w >> 30), wl = (int)w & Q_MASK30;
+    const long long mid = q_wide(al, wh, q_wide(ah, wl, (1ll << 29) + wl / 2));  // + the mean of al wl
+    return q_wide(ah, wh, mid >> 30);
+}
+
+template <>
+struct Ar<q64> {
+    static __device__ __forceinline__ q64 add(q64 a, q64 b) { return {a.v + b.v}; }
+    static __device__ __forceinline__ q64 sub(q64 a, q64 b) { return {a.v - b.v}; }
+    static __device__ __forceinline__ q64 add_nn(q64 a, q64 b) { return {a.v + b.v}; }
+    static __device__ __forceinline__ q64 sub_nn(q64 a, q64 b) { return {a.v - b.v}; }
+    static __device__ __forceinline__ q64 neg(q64 a) { return {-a.v}; }
+    static __device__ __forceinline__ q64 mul(q64 a, q64 w) { return {q_mul(a.v, w.v)}; }
+    static __device__ __forceinline__ q64 norm(q64 a) { return a; }
+    // sqrt(1/2) 2^60
+    static __device__ __forceinline__ q64 rsqrt2() { return {815238614083298888ll}; }
+};
+
+// a w; the middle products start at r0: 2^29 rounds the result, 0 leaves its floor
+__device__ __forceinline__ cx<q64> c_mul(cx<q64> a, qtw w, long long r0 = 1ll << 29)
+{
+    const int arh = (int)(a.re.v >> 30), arl = (int)a.re.v & Q_MASK30;
+    const int aih = (int)(a.im.v >> 30), ail = (int)a.im.v & Q_MASK30;
+    const int nh = -aih, nl = -ail;
+    long long mr = q_wide(arh, w.rl, r0), mi = q_wide(arh, w.il, r0);
+    mr = q_wide(arl, w.rh, mr);
+    mi = q_wide(arl, w.ih, mi);
+    mr = q_wide(nh, w.il, mr);
+    mi = q_wide(aih, w.rl, mi);
+    mr = q_wide(nl, w.ih, mr);
+    mi = q_wide(ail, w.rh, mi);
+    return {{q_wide(nh, w.ih, q_wide(arh, w.rh, mr >> 30))}, {q_wide(aih, w.rh, q_wide(arh, w.ih, mi >> 30))}};
+}
+
+// a / 2^s rounded half to even, s < 32
+__device__ __forceinline__ long long q_shift_even(long long a, int s)
+{
+    const long long h = s ? (1ll << (s - 1)) - 1 + ((a >> s) & 1) : 0;
+    return (a + h) >> s;
+}
+
+// (a + rd) / 2^s, s < 32: with rd = 2^(s-1) unbiased for the floors of numbers
+// whose fractions are spread evenly
+__device__ __forceinline__ cx<q64> q_shift(cx<q64> a, int s, long long rd)
+{
+    const long long r = a.re.v + rd, i = a.im.v + rd;
+    const unsigned rl = __funnelshift_r((unsigned)r, (unsigned)(r >> 32), s), il = __funnelshift_r((unsigned)i, (unsigned)(i >> 32), s);
+    const int rh = (int)(r >> 32) >> s, ih = (int)(i >> 32) >> s;
+    return {{((long long)rh << 32) | rl}, {((long long)ih << 32) | il}};
+}
+
+// the magnitude bits of a value's high word
+__device__ __forceinline__ unsigned q_bits(q64 a)
+{
+    const int h = (int)(a.v >> 32);
+    return (unsigned)(h ^ (h >> 31));
+}
+
+// the limbs of w / 2^s (conjugated if conj)
+__device__ __forceinline__ qtw q_twiddle(cx<double> w, int s, bool conj)
+{
+    const long long r = q_decode(w.re, 1022 + s, Q_TOP).v, i = q_decode(w.im, 1022 + s, Q_TOP, conj ? -1 : 0).v;
+    const int rl = (int)(r << 2) >> 2, il = (int)(i << 2) >> 2;  // balanced 30-bit low limbs
+    return {(int)((r - rl) >> 30), rl, (int)((i - il) >> 30), il};
+}

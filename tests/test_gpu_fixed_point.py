@@ -1,0 +1,86 @@
+"""The FP64 path's fixed-point transforms and digit products at the sizes and
+values where they can go wrong, against the oracle's direct sums."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from paper_2605_30379_gb300 import synth
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def mrc():
+    from paper_2605_30379_gb300 import build
+    build.build()
+    from paper_2605_30379_gb300 import mrc as m
+    m.load()
+    return m
+
+
+def dev(x):
+    return torch.from_numpy(np.ascontiguousarray(x)).to("cuda")
+
+
+def product_bound(A, B, u=2.0 ** -53):
+    """Prop 2.1's forward-error bound of the FFT product (the constants of
+    test_fft_product_within_prop_2_1_bound)."""
+    N, d = A.shape[0], A.shape[1]
+    L = 2 << max(0, (N - 1).bit_length())
+    sig, gam = 7 * u * np.log2(L), np.sqrt(2.0) * (d + 2) * u
+    beta = 2 * sig + sig ** 2 + gam * (1 + sig) ** 2
+    norm = lambda X: np.sqrt((X ** 2).sum())
+    return np.sqrt(L) * norm(A) * norm(B) * (beta + sig * (1 + beta))
+
+
+def integers(rng, N, d):
+    return rng.integers(-8, 9, size=(N, d, d)).astype(np.float64)
+
+
+@pytest.mark.parametrize("d", [1, 3])
+@pytest.mark.parametrize("N", [1, 2, 3, 4, 5, 8, 9, 16, 17, 33, 65, 129, 257, 513, 1024, 1025, 2049, 4097])
+def test_transform_sizes(mrc, N, d):
+    """One transform length per power of two up to two passes, ragged row
+    counts, E = 1 and 9 (partial entry chunks): rho = e0 - A * B on small
+    integers, whose direct sums are exact, within 1 % of Prop 2.1's bound
+    (N >= 2; a few roundings of the entries at N = 1)."""
+    rng = np.random.default_rng(1000 * d + N)
+    A, B = integers(rng, N, d), integers(rng, N, d)
+    ref, _ = oracle.residuals(A, B)
+    got = mrc.residual(dev(A), dev(B), sides=1, prec="fp64")[0].cpu().numpy()
+    assert np.sqrt(((got - ref) ** 2).sum()) <= max(1e-2, 0.2 / N) * product_bound(A, B)
+
+
+@pytest.mark.parametrize("e", [300, -300, 900])
+def test_power_of_two_scaling_is_exact(mrc, e):
+    """The alignment follows each column's exponent: scaling A by 2^e and B by
+    2^-e changes no bit of their product."""
+    rng = np.random.default_rng(5)
+    A, B = rng.standard_normal((300, 3, 3)), rng.standard_normal((300, 3, 3))
+    one = mrc.residual(dev(A), dev(B), sides=1, prec="fp64")[0]
+    two = mrc.residual(dev(np.ldexp(A, e)), dev(np.ldexp(B, -e)), sides=1, prec="fp64")[0]
+    assert torch.equal(one, two)
+
+
+@pytest.mark.parametrize("bad", [np.nan, np.inf, -np.inf])
+def test_non_finite_values_stay_in_their_row(mrc, bad):
+    """A NaN or infinity in A(k)[1][2] reaches row 1 of A * B and no other row;
+    nothing finite comes out of that row's product."""
+    rng = np.random.default_rng(6)
+    A, B = rng.standard_normal((40, 3, 3)), rng.standard_normal((40, 3, 3))
+    ref = mrc.residual(dev(A), dev(B), sides=1, prec="fp64")[0]
+    A[7, 1, 2] = bad
+    got = mrc.residual(dev(A), dev(B), sides=1, prec="fp64")[0]
+    assert not torch.isfinite(got[:, 1]).any()
+    assert torch.equal(got[:, [0, 2]], ref[:, [0, 2]])
+
+
+@pytest.mark.parametrize("d,N,seed", [(3, 2048, 0), (16, 2049, 1), (40, 700, 2)])
+def test_long_tails_and_spikes(mrc, d, N, seed):
+    """A = e0 - q: unit spikes beside entries of 1e-3 that fall off to nothing;
+    the inverse keeps the FP64 tolerance."""
+    q, _ = synth.weibull_model(d, N, seed=seed)
+    A = synth.identity_minus(q)
+    psi = mrc.inverse(dev(A), prec="fp64").cpu().numpy()
+    assert np.abs(psi - oracle.inverse_left(A)).max() <= 1e-12
