@@ -207,17 +207,28 @@ size_t ws_inverse(int d, int64_t N, int prec)
 
 // Product kernel choices: 0..2 and 4 the FP32-pipe tile configurations
 // 16/32/64 and 24 (pairmul_cfg), 3 the tensor-core digit kernel: for square 32 <= d <= 64
-// the pipelined one (pair_tc.cu; double-float or FP32), for double-float
+// (FP64: 17 <= d) the pipelined one (pair_tc.cu), for double-float
 // 64 < d <= 512 the tiled one (ozaki_tc.cu).
 bool tensor_choice_exists(int prec, int r, int m, int c)
 {
+    if (prec == PREC_F64) return mrc_tcp64_supported(r, m, c);
     if (prec == PREC_DD) return mrc_tc_supported(r, m, c);
     return prec == PREC_F32 && mrc_tcp_supported(r, m, c);
+}
+
+// whether the built-in choice for a square product is the tensor-core kernel:
+// double-float always, FP32 from 256 points on (fewer pairs than SMs below),
+// FP64 by mrc_tcp64_default
+bool tensor_default(int prec, int64_t M, int r, int m, int c)
+{
+    if (!tensor_choice_exists(prec, r, m, c)) return false;
+    return prec == PREC_DD || (prec == PREC_F64 ? mrc_tcp64_default(M, r) : M >= 256);
 }
 
 cudaError_t launch_tensor(mrc_ctx *cx, int prec, const void *zx, const void *zy, void *zc, int64_t M, int d,
                           const void *tw, cudaStream_t st)
 {
+    if (prec == PREC_F64) return mrc_pairmul_f64_tcp(zx, zy, zc, M, d, tw, MRC_TW_LOG, cx->cur_status, st);
     if (prec == PREC_F32) return mrc_pairmul_f32_tcp(zx, zy, zc, M, d, tw, MRC_TW_LOG, cx->cur_status, st);
     if (d <= 64) return mrc_pairmul_dd_tcp(zx, zy, zc, M, d, tw, MRC_TW_LOG, cx->cur_status, st);
     return mrc_pairmul_dd_tc(zx, zy, zc, M, d, tw, MRC_TW_LOG, cx->cur_status, st);
@@ -340,16 +351,14 @@ cudaError_t fft_any(mrc_ctx *cx, int prec, const FftSrc &sx, const FftDst &dx, i
 }
 
 // The per-frequency product of one precision: the autotuned choice when the
-// call asked for tuning, else the tensor-core digit kernels for square
-// double-float products with 32 <= d <= 512 and square FP32 products with
-// 32 <= d <= 64 on transforms of at least 256 points (fewer pairs than SMs
-// below that), the FP32-pipe tiles elsewhere.
+// call asked for tuning, else the tensor-core digit kernels where
+// tensor_default says so, the FP32- or FP64-pipe tiles elsewhere.
 cudaError_t pairmul_any(mrc_ctx *cx, int prec, const void *zx, const void *zy, void *zc, int64_t M, int r, int m,
                         int c, const void *tw, cudaStream_t st)
 {
     const int ch = tuned_choice(cx, prec, zx, zy, zc, M, r, m, c, tw, st);
     if (ch >= 0) return launch_choice(cx, prec, ch, zx, zy, zc, M, r, m, c, tw, st);
-    if (tensor_choice_exists(prec, r, m, c) && (prec == PREC_DD || M >= 256))
+    if (tensor_default(prec, M, r, m, c))
         return launch_tensor(cx, prec, zx, zy, zc, M, r, tw, st);
     return OPS[prec].pairmul(zx, zy, zc, M, r, m, c, tw, MRC_TW_LOG, st);
 }
@@ -394,7 +403,7 @@ mrc_status conv_product(mrc_ctx *c, Arena &ar, int prec, const double *X, int64_
         P.nseg = 1;
         P.a[0] = mrc_tcp_args(xpt, bY, bC, Mr, r, tw, MRC_TW_LOG);
         P.a[0].xs = xps;
-        CK(mrc_tcp_seg(1, P, c->cur_status, st));
+        CK(mrc_tcp_seg(PREC_DD, P, c->cur_status, st));
     } else {
         CK(pairmul_any(c, prec, bX, bY, bC, Mr, r, m, cc, tw, st));
     }
@@ -840,7 +849,7 @@ int product_choice(mrc_ctx *cx, int prec, int64_t M, int d)
         auto it = cx->tune.find(tune_key(prec, d, d, d, M));
         if (it != cx->tune.end()) return it->second;
     }
-    if (tensor_choice_exists(prec, d, d, d) && (prec == PREC_DD || M >= 256)) return 3;
+    if (tensor_default(prec, M, d, d, d)) return 3;
     return d <= 16 ? 0 : (d <= 24 ? 4 : (d <= 32 ? 1 : 2));
 }
 
@@ -885,7 +894,7 @@ mrc_status product_stage(mrc_ctx *c, int prec, int64_t M, const std::vector<Pair
                 P->a[q - i0] = mrc_tcp_args(j.zx, j.zy, j.zc, M, j.d, c->tw[prec], MRC_TW_LOG);
                 P->a[q - i0].xs = j.xs;
             }
-            CK(mrc_tcp_seg(prec == PREC_DD, *P, jobs[tcp[g][i0]].status, st));
+            CK(mrc_tcp_seg(prec, *P, jobs[tcp[g][i0]].status, st));
         }
     const int bsz[5] = {16, 32, 64, 0, 24};
     for (int cfg = 0; cfg < 5; ++cfg)

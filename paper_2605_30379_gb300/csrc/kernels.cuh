@@ -344,7 +344,7 @@ __device__ __forceinline__ void fft_stage(const FftArgs &a, cx<typename FftC<T>:
 #pragma unroll
             for (int q = 0; q < r; ++q) {
                 y[u][q] = {q_encode(v[u][q].re, eb, sgn), q_encode(v[u][q].im, eb, sgn)};
-                if (ex >= 2047) {  // an Inf or NaN among the column's points
+                if (ex >= Q_NONFINITE) {  // an Inf or NaN among the column's points
                     y[u][q].re = __longlong_as_double(0x7ff8000000000000ll);
                     y[u][q].im = y[u][q].re;
                 }
@@ -503,7 +503,7 @@ __device__ __forceinline__ void fft_pass_body(const FftArgs &a, int64_t j, int e
         if ((tid & 31) < EC) atomicMax(&sexp[tid & (EC - 1)], m);
         __syncthreads();
         ex = sexp[tid & (EC - 1)];
-        if (ex == 2047) ex = 4096;  // stays above every finite column's
+        if (ex == 2047) ex = Q_NONFINITE;
     }
     const int64_t base_out = (j >> a.logNs << (a.logNs + LOGR)) + jm;
     fft_stage<T, LOGR, EC, 0, INV>(a, sm, stw, spt, e0, ecount, base_out, pre, ex, sor);

@@ -189,9 +189,19 @@ cudaError_t mrc_pairmul_dd_tcp(const void *zx, const void *zy, void *zc, int64_t
                                int *status, cudaStream_t st);
 cudaError_t mrc_pairmul_f32_tcp(const void *zx, const void *zy, void *zc, int64_t M, int d, const void *tw, int tw_log,
                                 int *status, cudaStream_t st);
-// the same over the products of one segmented launch (all of the same M and
-// of the same ceil(d / 16)); a timeout is reported in *status
-cudaError_t mrc_tcp_seg(int dd_prec, const SegParams<PairArgs> &P, int *status, cudaStream_t st);
+// FP64: square 17 <= d <= 64.  The built-in choice takes it for d >= 25 and,
+// below, for M <= 256: the FP64-pipe tiles of 24 and 16 need 28 and 8 us per
+// frequency pair and SM and one pair fills an SM, the digit product about 40
+// us at two K chunks but less where pairs are fewer than SMs (timed per d and
+// M: the digit product is the faster from d = 26 on at every M, for d = 20 and
+// 24 up to M = 256, at d = 16 nowhere).
+bool mrc_tcp64_supported(int r, int m, int c);
+bool mrc_tcp64_default(int64_t M, int d);
+cudaError_t mrc_pairmul_f64_tcp(const void *zx, const void *zy, void *zc, int64_t M, int d, const void *tw, int tw_log,
+                                int *status, cudaStream_t st);
+// the same over the products of one segmented launch (all of the same
+// precision, M and ceil(d / 16)); a timeout is reported in *status
+cudaError_t mrc_tcp_seg(int prec, const SegParams<PairArgs> &P, int *status, cudaStream_t st);
 PairArgs mrc_tcp_args(const void *zx, const void *zy, void *zc, int64_t M, int d, const void *tw, int tw_log);
 // The double-float product with X prepared once (X is the spectrum of A,
 // the same in every residual sweep): mrc_tcp_prep writes, for every product

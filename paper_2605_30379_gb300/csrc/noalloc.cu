@@ -58,10 +58,12 @@ cudaError_t fft_f64(void *, int, const FftSrc &sx, const FftDst &dx, int64_t M, 
     return mrc_fft_f64(sx, dx, M, E, dir, scratch, tw, tw_log, st, -1);
 }
 
-// the level product: the default FP64 product kernel (no autotuning here)
-cudaError_t product_f64(void *, int, const void *zx, const void *zy, void *zc, int64_t M, int d, const void *tw,
+// the level product: the default FP64 product kernels (no autotuning here);
+// status: the word a tensor-core product's bounded wait reports to
+cudaError_t product_f64(void *status, int, const void *zx, const void *zy, void *zc, int64_t M, int d, const void *tw,
                         int tw_log, cudaStream_t st)
 {
+    if (mrc_tcp64_default(M, d)) return mrc_pairmul_f64_tcp(zx, zy, zc, M, d, tw, tw_log, (int *)status, st);
     return mrc_pairmul_f64(zx, zy, zc, M, d, d, d, tw, tw_log, st);
 }
 
@@ -89,7 +91,7 @@ mrc_status setup(int dev, unsigned char **out)
         return MRC_ERR_CUDA;
     }
     unsigned char *base = (unsigned char *)p;
-    if (mrc_init_f64() != cudaSuccess) return MRC_ERR_CUDA;
+    if (mrc_init_f64() != cudaSuccess || mrc_tcp_init() != cudaSuccess) return MRC_ERR_CUDA;
     if (mrc_twiddles_f64(base + kTwOff, kTwLog, 0) != cudaSuccess) return MRC_ERR_CUDA;
     if (cudaStreamSynchronize(0) != cudaSuccess) return MRC_ERR_CUDA;
     g_addr[dev] = base;
@@ -141,7 +143,7 @@ extern "C" mrc_status mrc_inverse_noalloc(int d, int64_t N, const double *A, dou
     const int64_t m0 = mrc_base_size(d, N);
     CKN(mrc_base_case(A, psi, d, m0, st));
     const NewtonBufs nb{b0, b1, b2, bt};
-    if (mrc_newton_levels(PREC_F64, d, N, A, psi, m0, nb, tw, kTwLog, fft_f64, product_f64, nullptr, st, nullptr,
+    if (mrc_newton_levels(PREC_F64, d, N, A, psi, m0, nb, tw, kTwLog, fft_f64, product_f64, status, st, nullptr,
                           nullptr, nullptr, nullptr) != 0)
         return MRC_ERR_CUDA;
     CKN(cudaStreamSynchronize(st));

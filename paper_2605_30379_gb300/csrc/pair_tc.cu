@@ -1,8 +1,16 @@
 // pair_tc.cu -- per-frequency complex matrix products of the FFT-Newton path
 // (Eq. (fft-convolution): C(phi) = X(phi) Y(phi) at every frequency of the
-// half spectrum, square d x d with 32 <= d <= 64) as exact digit products on
-// the tcgen05 tensor cores, for two working precisions:
+// half spectrum, square d x d with d <= 64) as exact digit products on the
+// tcgen05 tensor cores, for three working precisions:
 //
+//   FP64 (17 <= d): eight balanced base-256 digits of 64-bit fixed-point
+//     values, pairs s + t >= 7 (36 pairs in 8 weight groups), about 2^-58
+//     relative to the row and column maxima.  The FP64 pipe gives two
+//     multiply-adds per clock and SM; at d = 64, N = 2^15 the inverse's 28
+//     products take 17 ms here against 138 ms on it (whole inverse 159.6 ->
+//     39.2 ms), with smaller errors (Weibull d = 64, N = 512 against
+//     long double: 7.9e-16 -> 5.5e-16);
+
 //   double-float (the residual product of Proposition 2.6): six balanced
 //     base-256 digits per value, digit pairs of weight s + t >= 5 (21 pairs
 //     in 6 weight groups), about 2^-41 relative to the row and column bounds;
@@ -11,6 +19,11 @@
 //     relative to the row and column bounds.  Three digits (6 pairs, about
 //     2^-21) made the product 1.27x faster at d = 64, N = 2^18 but left
 //     e_rel at 1.7e-9 after the sweep (gate 1e-10).
+//
+// FP64 digits are FP16 integers cut from the bytes of the fixed-point value
+// (a byte permute and one packed subtraction per two digits) and its groups
+// are folded in 64-bit integers; the rest of this comment describes the two
+// FP32-based precisions, whose digits are BF16 numbers kept at their scale.
 //
 // The rows of X are scaled by 2^-sigma_i and the columns of Y by 2^-tau_j
 // (powers of two from bounds over both frequencies of the pair) and every
@@ -68,6 +81,10 @@ template <class T> struct TcP;
 // ahead 41.4 -> 46.4 ms (256 KB per pair and SM crowd L2), so none.
 template <> struct TcP<dd> { static constexpr int S = 6, GMIN = 5, NSLOT = 3, NF = 1, PF = 0; };
 template <> struct TcP<float> { static constexpr int S = 4, GMIN = 3, NSLOT = 2, NF = 2, PF = 2; };
+// FP64: eight digits of a 64-bit fixed-point value, pairs s + t >= 7 (36 pairs
+// in 8 groups: all 512 TMEM columns)
+template <> struct TcP<double> { static constexpr int S = 8, GMIN = 7, NSLOT = 2, NF = 1, PF = 0; };
+template <class T> constexpr bool tc_q = std::is_same<T, double>::value;
 
 constexpr int KC = 16;                // K per chunk: one MMA K step
 constexpr int NCH = 64 / KC;          // chunks per frequency
@@ -82,7 +99,8 @@ constexpr int NTHREADS = 13 * 32;
 constexpr int XLD = 33;               // row length (values) of the epilogue transpose
 constexpr unsigned TMEM_COLS = 512;
 constexpr int BAR_SPLIT = 1, BAR_EPI = 2;
-constexpr unsigned IDESC = idesc_bf16<128, 64>();
+template <class T>
+constexpr unsigned IDESC = tc_q<T> ? idesc_f16<128, 64>() : idesc_bf16<128, 64>();
 
 template <class T>
 struct TcL {
@@ -147,6 +165,14 @@ __device__ __forceinline__ cx<float> ldv_cx<float>(const cx<float> *p)
     return {v.x, v.y};
 }
 
+template <>
+__device__ __forceinline__ cx<double> ldv_cx<double>(const cx<double> *p)
+{
+    double2 v;
+    asm volatile("ld.global.nc.v2.f64 {%0, %1}, [%2];\n" : "=d"(v.x), "=d"(v.y) : "l"(p));
+    return {v.x, v.y};
+}
+
 // High parts of one packed value (re, im): the bounds use them only
 template <class T>
 __device__ __forceinline__ float2 ldg_hi(const cx<T> *p);
@@ -160,6 +186,14 @@ template <>
 __device__ __forceinline__ float2 ldg_hi<float>(const cx<float> *p)
 {
     return __ldg(reinterpret_cast<const float2 *>(p));
+}
+
+// FP64: the bits of the high words (their exponents are the bounds)
+template <>
+__device__ __forceinline__ float2 ldg_hi<double>(const cx<double> *p)
+{
+    const float *q = reinterpret_cast<const float *>(p);
+    return make_float2(__ldg(q + 1), __ldg(q + 3));
 }
 
 // Bounds of a pair: row bounds bx[i] = max_k (|Z_X(f)_ik|_1 + |Z_X(M-f)_ik|_1)
@@ -193,11 +227,24 @@ __device__ __forceinline__ void bnd_issue(BndIn &b, const cx<T> *ZX, const cx<T>
     }
 }
 
+__device__ __forceinline__ unsigned abs_bits(float2 a, float2 b)
+{
+    return max(max(__float_as_uint(a.x) & 0x7fffffffu, __float_as_uint(a.y) & 0x7fffffffu),
+               max(__float_as_uint(b.x) & 0x7fffffffu, __float_as_uint(b.y) & 0x7fffffffu));
+}
+
+template <class T>
 __device__ __forceinline__ void bnd_reduce(const BndIn &b, unsigned *bx, float &my, int t, int n0)
 {
 #pragma unroll
     for (int u = 0; u < 2; ++u) {
         const int i = (t >> 6) + 4 * (n0 + u);  // one row per pair of warps
+        if constexpr (tc_q<T>) {  // the largest high word of a magnitude (as bits: nonnegative floats order like them)
+            my = __uint_as_float(max(__float_as_uint(my), abs_bits(b.ya[u], b.yb[u])));
+            const unsigned wm = __reduce_max_sync(0xffffffffu, abs_bits(b.xa[u], b.xb[u]));
+            if ((t & 31) == 0) atomicMax(&bx[i], wm);
+            continue;
+        }
         const float mx = fabsf(b.xa[u].x) + fabsf(b.xa[u].y) + fabsf(b.xb[u].x) + fabsf(b.xb[u].y);
         my = fmaxf(my, fabsf(b.ya[u].x) + fabsf(b.ya[u].y) + fabsf(b.yb[u].x) + fabsf(b.yb[u].y));
         const unsigned wmx = __reduce_max_sync(0xffffffffu, __float_as_uint(mx));  // nonnegative: bits order
@@ -207,8 +254,18 @@ __device__ __forceinline__ void bnd_reduce(const BndIn &b, unsigned *bx, float &
 
 // The pair's scale factors from its bounds (2 Xh and 2 Yh are split: bound
 // 2 |.|, scaled values <= 1/2)
+template <class T>
 __device__ __forceinline__ void bnd_scales(const unsigned *bx, const unsigned *by, float *sc, int d, int t)
 {
+    if constexpr (tc_q<T>) {
+        // the alignment exponents: every |re|, |im| below 63/64 2^(ex - 1022)
+        // (above every finite one for Inf and NaN)
+        const int ex = t < d ? max(1, (int)((bx[t] + 0x8000u) >> 20)) : 1;
+        const int ey = t < d ? max(1, (int)((by[t] + 0x8000u) >> 20)) : 1;
+        sc[t] = sc[128 + t] = __int_as_float(ex >= 2047 ? Q_NONFINITE : ex);
+        sc[64 + t] = sc[192 + t] = __int_as_float(ey >= 2047 ? Q_NONFINITE : ey);
+        return;
+    }
     const int sx = t < d ? scale_exp(2.0f * __uint_as_float(bx[t])) : 0;
     const int sy = t < d ? scale_exp(2.0f * __uint_as_float(by[t])) : 0;
     sc[t] = t < d ? pow2c(-sx) : 0.0f;
@@ -425,15 +482,80 @@ __device__ __forceinline__ void ydigits(DState<T> (&st)[NFQ][4][2], unsigned cha
     (ydigit<T, NFQ, TcL<T>::S - 1 - s>(st, slot, off), ...);
 }
 
+// FP64: 2 Xh (or 2 Yh) of packed values a = Z(f), b = Z(M - f) as 64-bit
+// fixed-point numbers aligned to the exponent ex: |re|, |im| of the raw
+// values stay below 63/64 2^60, so |2 Xh| <= 2 sqrt(|a|^2 + |b|^2) < 63/64 2^62.
+__device__ __forceinline__ cx<q64> split_q(cx<double> za, cx<double> zb, qtw w, int ex)
+{
+    const cx<q64> a = {q_decode(za.re, ex, Q_TOP), q_decode(za.im, ex, Q_TOP)};
+    const cx<q64> b = {q_decode(zb.re, ex, Q_TOP), q_decode(zb.im, ex, Q_TOP)};
+    // s = a + conj b, t = w (-i) (a - conj b)
+    const cx<q64> t = c_mul(cx<q64>{{a.im.v + b.im.v}, {b.re.v - a.re.v}}, w);
+    return {{a.re.v + b.re.v + t.re.v}, {a.im.v - b.im.v + t.im.v}};
+}
+
+// FP16 pairs of four balanced digits of two values: with every byte offset by
+// 128 digit s is byte s minus 128; 0x6400 makes a byte the FP16 number
+// 1024 + byte
+__device__ __forceinline__ void digits_q(unsigned u0, unsigned u1, unsigned (&q)[4])
+{
+    const unsigned lo = __byte_perm(u0, u1, 0x5410), hi = __byte_perm(u0, u1, 0x7632);
+    const unsigned off = 0x64806480u;  // 1152 = 1024 + 128
+    auto sub = [&](unsigned x) {
+        const unsigned b = (x & 0x00ff00ffu) | 0x64006400u;
+        unsigned r;
+        asm("sub.f16x2 %0, %1, %2;" : "=r"(r) : "r"(b), "r"(off));
+        return r;
+    };
+    q[0] = sub(lo);
+    q[1] = sub(lo >> 8);
+    q[2] = sub(hi);
+    q[3] = sub(hi >> 8);
+}
+
+// The digits of 2 v of four values (below 63/64 2^63: the whole 64 bits are
+// used, which leaves the dropped pairs s + t < 7 at 2^-58 of the row and
+// column maxima), packed as store_x / store_y take them
+__device__ __forceinline__ void pack4_q(const q64 (&v)[4], unsigned (&w)[8][2])
+{
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        const unsigned long long a = ((unsigned long long)v[2 * h].v << 1) + 0x8080808080808080ull;
+        const unsigned long long b = ((unsigned long long)v[2 * h + 1].v << 1) + 0x8080808080808080ull;
+        unsigned q[4];
+        digits_q((unsigned)a, (unsigned)b, q);
+#pragma unroll
+        for (int s = 0; s < 4; ++s) w[s][h] = q[s];
+        digits_q((unsigned)(a >> 32), (unsigned)(b >> 32), q);
+#pragma unroll
+        for (int s = 0; s < 4; ++s) w[4 + s][h] = q[s];
+    }
+}
+
 // The split of one chunk into the slot.  NF == 1: the frequency with
 // twiddle w of the raw rows (ra, rb); NF == 2: f (sub-slot 0) and M - f (1).
 template <class T>
-__device__ __forceinline__ void split_chunk_x(const Raw<T> &r, unsigned char *slot, const float *scx, cx<T> w, int t)
+using TcW = typename std::conditional<tc_q<T>, qtw, cx<T>>::type;  // the split's twiddle
+
+template <class T>
+__device__ __forceinline__ void split_chunk_x(const Raw<T> &r, unsigned char *slot, const float *scx, TcW<T> w, int t)
 {
     using L = TcL<T>;
     constexpr int NF = L::NF;
-    const int k = t & 15, i4 = t >> 4;
-    if constexpr (__is_same(T, dd)) {  // value by value
+    [[maybe_unused]] const int k = t & 15, i4 = t >> 4;
+    if constexpr (tc_q<T>) {
+        q64 vr[4], vi[4];
+#pragma unroll
+        for (int n = 0; n < 4; ++n) {
+            const cx<q64> v = split_q(r.xa[n], r.xb[n], w, __float_as_int(scx[4 * i4 + n]));
+            vr[n] = v.re;
+            vi[n] = v.im;
+        }
+        unsigned wr[8][2], wi[8][2];
+        pack4_q(vr, wr);
+        pack4_q(vi, wi);
+        store_x<8>(slot, wr, wi, t);
+    } else if constexpr (__is_same(T, dd)) {  // value by value
         float sc[4];
 #pragma unroll
         for (int n = 0; n < 4; ++n) sc[n] = scx[4 * i4 + n];
@@ -468,13 +590,25 @@ __device__ __forceinline__ void split_chunk_x(const Raw<T> &r, unsigned char *sl
 }
 
 template <class T>
-__device__ __forceinline__ void split_chunk_y(const Raw<T> &r, unsigned char *slot, const float *scy, cx<T> w, int t)
+__device__ __forceinline__ void split_chunk_y(const Raw<T> &r, unsigned char *slot, const float *scy, TcW<T> w, int t)
 {
     using L = TcL<T>;
     constexpr int NF = L::NF;
-    const int lane = t & 31, j = 8 * (t >> 5) + (lane & 7), k4 = lane >> 3;
+    [[maybe_unused]] const int lane = t & 31, j = 8 * (t >> 5) + (lane & 7), k4 = lane >> 3;
     const float sc = scy[j];
-    if constexpr (__is_same(T, dd)) {  // value by value
+    if constexpr (tc_q<T>) {
+        q64 vr[4], vi[4];
+#pragma unroll
+        for (int n = 0; n < 4; ++n) {
+            const cx<q64> v = split_q(r.ya[n], r.yb[n], w, __float_as_int(sc));
+            vr[n] = v.re;
+            vi[n] = v.im;
+        }
+        unsigned wr[8][2], wi[8][2];
+        pack4_q(vr, wr);
+        pack4_q(vi, wi);
+        store_y<8>(slot, wr, wi, t);
+    } else if constexpr (__is_same(T, dd)) {  // value by value
         const float scv[4] = {sc, sc, sc, sc};
         cx<T> vf[4];
 #pragma unroll
@@ -519,6 +653,27 @@ __device__ __forceinline__ dd add_f(dd a, float v)
 template <class T, int NG>
 __device__ __forceinline__ void fold8(unsigned tbase, T (&out)[8])
 {
+    if constexpr (tc_q<T>) {
+        // exact integers below 2^24: the top four groups and the lower four as
+        // 64-bit sums, rounded once
+        long long H[8], Lw[8];
+#pragma unroll
+        for (int g = NG - 1; g >= 0; --g) {
+            unsigned r[8];
+            ld8(tbase + (unsigned)(g * 64), r);
+#pragma unroll
+            for (int c = 0; c < 8; ++c) {
+                const int v = __float2int_rn(__uint_as_float(r[c]));
+                if (g == 7) H[c] = (long long)v << 24;
+                else if (g >= 4) H[c] = q_wide(v, 1 << (8 * (g - 4)), H[c]);
+                else if (g == 3) Lw[c] = (long long)v << 24;
+                else Lw[c] = q_wide(v, 1 << (8 * g), Lw[c]);
+            }
+        }
+#pragma unroll
+        for (int c = 0; c < 8; ++c) out[c] = q96_to_double(H[c], Lw[c]);
+        return;
+    } else {
     float lo[8];
 #pragma unroll
     for (int g = NG - 1; g >= 0; --g) {
@@ -542,6 +697,7 @@ __device__ __forceinline__ void fold8(unsigned tbase, T (&out)[8])
 #pragma unroll
         for (int c = 0; c < 8; ++c) out[c] = add_f(out[c], lo[c]);
     }
+    }
 }
 
 __device__ __forceinline__ dd mul_f(dd x, float f) { return {x.hi * f, x.lo * f}; }
@@ -549,6 +705,11 @@ __device__ __forceinline__ float mul_f(float x, float f) { return x * f; }
 
 template <class T>
 __device__ __forceinline__ void st_cx(cx<T> *p, cx<T> v);
+template <>
+__device__ __forceinline__ void st_cx<double>(cx<double> *p, cx<double> v)
+{
+    *reinterpret_cast<double2 *>(p) = make_double2(v.re, v.im);
+}
 template <>
 __device__ __forceinline__ void st_cx<dd>(cx<dd> *p, cx<dd> v)
 {
@@ -558,6 +719,52 @@ template <>
 __device__ __forceinline__ void st_cx<float>(cx<float> *p, cx<float> v)
 {
     *reinterpret_cast<float2 *>(p) = make_float2(v.re, v.im);
+}
+
+// FP64 outputs of one round of 32 columns (this thread: column j, sixteen
+// rows): the exponents of the row and column alignments join, then C(f) is
+// stored unmerged (phase 0) or the pair merged with it,
+//   ZC(f) = s + i p, ZC(M - f) = conj s + i conj p,
+//   s = (C(f) + conj C(M - f)) / 2, p = conj w (C(f) - conj C(M - f)) / 2;
+// the factor 1/2 and the split's 2 on both operands are in the exponent.
+__device__ __forceinline__ void epi_q(cx<double> *ZC, const double *xch, const float *fx, int ey, cx<double> wf, int64_t f,
+                                      int64_t gZ, int d, int64_t E, int j, int jl, int et, int phase, bool self, bool two)
+{
+#pragma unroll 1
+    for (int m0 = 0; m0 < 16; m0 += 4) {
+        cx<double> v[4], cf[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int i = (et >> 5) + 4 * (m0 + u);
+            const int ex = __float_as_int(fx[i]), de = ex + ey - 2113;
+            v[u] = {q_scale(xch[i * XLD + jl], de), q_scale(xch[(64 + i) * XLD + jl], de)};
+            if (max(ex, ey) >= Q_NONFINITE) v[u].re = v[u].im = __longlong_as_double(0x7ff8000000000000ll);
+            if (self) cf[u] = v[u];
+            else if (phase == 1 && i < d && j < d) cf[u] = ZC[f * E + (int64_t)i * d + j];  // stored by this thread
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int i = (et >> 5) + 4 * (m0 + u);
+            if (i >= d || j >= d) continue;
+            cx<double> *zf = ZC + f * E + (int64_t)i * d + j;
+            if (!self && phase == 0) {
+                st_cx(zf, v[u]);
+                continue;
+            }
+            const double sr = cf[u].re + v[u].re, si = cf[u].im - v[u].im;
+            const double dr = cf[u].re - v[u].re, di = cf[u].im + v[u].im;
+            const double pr = fma(wf.re, dr, wf.im * di), pi = fma(wf.re, di, -(wf.im * dr));
+            st_cx(zf, cx<double>{sr - pi, si + pr});
+            if (two) st_cx(ZC + gZ * E + (int64_t)i * d + j, cx<double>{sr + pi, pr - si});
+        }
+    }
+}
+
+template <class T>
+__device__ __forceinline__ TcW<T> split_tw(cx<T> w)
+{
+    if constexpr (tc_q<T>) return q_twiddle(w, 0, false);
+    else return w;
 }
 
 // P: the products of one launch, all of M points (a single one, or every
@@ -662,14 +869,14 @@ __global__ void __launch_bounds__(NTHREADS, 1) tcp_kernel(const __grid_constant_
             float my = 0.0f;
             for (int n0 = 0; n0 < 4 * nck; n0 += 2) {
                 bnd_issue(bi, bx_of(s0), zy_of(s0), f, gZ, d_of(s0), t, n0);
-                bnd_reduce(bi, bxy, my, t, n0);
+                bnd_reduce<T>(bi, bxy, my, t, n0);
             }
             atomicMax(&bxy[64 + (t & 63)], __float_as_uint(my));
         }
         bar_sync(BAR_SPLIT, NSPLIT);
         if (t < 64 && blockIdx.x < total) {
             const int s0 = (int)(blockIdx.x / npairs);
-            bnd_scales(bxy, bxy + 64, scb, d_of(s0), t);
+            bnd_scales<T>(bxy, bxy + 64, scb, d_of(s0), t);
             if (XPRE) scb[128 + t] = xs_of(s0)[(int64_t)(blockIdx.x - (unsigned)s0 * npairs) * 128 + 64 + t];
         }
         bar_sync(BAR_SPLIT, NSPLIT);
@@ -677,8 +884,8 @@ __global__ void __launch_bounds__(NTHREADS, 1) tcp_kernel(const __grid_constant_
         for (unsigned gp = blockIdx.x; gp < total; gp += gridDim.x, ++pl) {
             const int sg = (int)(gp / npairs);
             const int64_t p = gp - (unsigned)sg * npairs, f = p, gZ = (M - p) & (M - 1);
-            const cx<T> wf = tw[f << (a.tw_log - a.logM - 1)];
-            const cx<T> wg = c_neg(c_conj(wf));
+            const cx<T> wfc = tw[f << (a.tw_log - a.logM - 1)];
+            const TcW<T> wf = split_tw<T>(wfc), wg = split_tw<T>(c_neg(c_conj(wfc)));
             const float *sc = scb + 4 * 64 * (pl % L::NB);
             const unsigned gpn = gp + gridDim.x;
             const bool next = gpn < total;
@@ -695,7 +902,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) tcp_kernel(const __grid_constant_
             if (!XPRE) load_x(raw, zx_of(sg), f, gZ, d_of(sg), 0, t);
             load_y(raw, zy_of(sg), f, gZ, d_of(sg), 0, t);
             for (int c = 0; c < nch; ++c, ++it) {
-                const cx<T> w = c < nck ? wf : wg;
+                const TcW<T> w = c < nck ? wf : wg;
                 const int slot = it % NSLOT, use = it / NSLOT;
                 unsigned char *sp = smem + slot * L::SLOT;
                 // bound slices of the next pair (in L2 by now): rows n0 .. n0 + ns - 1,
@@ -724,17 +931,17 @@ __global__ void __launch_bounds__(NTHREADS, 1) tcp_kernel(const __grid_constant_
                 }
                 asm volatile("" ::: "memory");  // the loads above stay ahead of the Y digit stores
                 if (gather) {
-                    bnd_reduce(bi, bn, myn, t, n0);
+                    bnd_reduce<T>(bi, bn, myn, t, n0);
                     for (int u = 2; u < ns - 2; u += 2) {
                         bnd_issue(bi, bx_of(sn), zy_of(sn), fn, gn, d_of(sn), t, n0 + u);
-                        bnd_reduce(bi, bn, myn, t, n0 + u);
+                        bnd_reduce<T>(bi, bn, myn, t, n0 + u);
                     }
                     if (ns > 2) bnd_issue(bi, bx_of(sn), zy_of(sn), fn, gn, d_of(sn), t, n0 + ns - 2);
                 }
                 if (!failed) split_chunk_y<T>(raw, sp, sc + 64, w, t);
                 if (cn < nch) load_y(raw, zy_of(sg), na, nb, d_of(sg), kn, t);
                 asm volatile("" ::: "memory");
-                if (gather && ns > 2) bnd_reduce(bi, bn, myn, t, n0 + ns - 2);
+                if (gather && ns > 2) bnd_reduce<T>(bi, bn, myn, t, n0 + ns - 2);
                 if (!failed) {
                     fence_async_smem();  // digit tiles visible to the tensor cores
                     mbar_arrive(smem_u32(&bar_full[slot]));
@@ -744,7 +951,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) tcp_kernel(const __grid_constant_
             if (bar_or(BAR_SPLIT, NSPLIT, failed || abort_flag)) break;  // the next pair's bounds complete
             if (next && t < 64) {
                 float *scn = scb + 4 * 64 * ((pl + 1) % L::NB);
-                bnd_scales(bn, bn + 64, scn, d_of(sn), t);
+                bnd_scales<T>(bn, bn + 64, scn, d_of(sn), t);
                 if (XPRE) scn[128 + t] = xs_of(sn)[pn * 128 + 64 + t];
             }
             if (t < 128) bxy[128 * (pl & 1) + t] = 0u;  // this pair's buffer: free for pair p + 2 grid
@@ -804,7 +1011,12 @@ __global__ void __launch_bounds__(NTHREADS, 1) tcp_kernel(const __grid_constant_
                     }
                     bar_sync(BAR_EPI, NEPI);
                     const int jl = et & 31, j = 32 * r + jl;
-                    const float sj = fy[j];
+                    [[maybe_unused]] const float sj = fy[j];
+                    if constexpr (tc_q<T>) {
+                        epi_q(ZC, xch, fx, __float_as_int(sj), wf, f, gZ, d, E, j, jl, et, phase, self, two);
+                        bar_sync(BAR_EPI, NEPI);
+                        continue;
+                    }
                     // four outputs at a time, their loads first
 #pragma unroll 1
                     for (int m0 = 0; m0 < 16; m0 += 4) {
@@ -875,9 +1087,9 @@ __global__ void __launch_bounds__(NTHREADS, 1) tcp_kernel(const __grid_constant_
                             for (int s = (g - (S - 1) > 0 ? g - (S - 1) : 0); s <= (g < S - 1 ? g : S - 1); ++s) {
                                 const int tt = g - s;
                                 const unsigned as = sa + s * A_TILE;
-                                mma<IDESC>(dcol, desc<SBO>(as + 8 * SBO), desc<SBO>(sbr + tt * B_TILE), acc);
+                                mma<IDESC<T>>(dcol, desc<SBO>(as + 8 * SBO), desc<SBO>(sbr + tt * B_TILE), acc);
                                 acc = 1u;
-                                mma<IDESC>(dcol, desc<SBO>(as), desc<SBO>(sbi + tt * B_TILE), 1u);
+                                mma<IDESC<T>>(dcol, desc<SBO>(as), desc<SBO>(sbi + tt * B_TILE), 1u);
                             }
                         }
                     }
@@ -976,10 +1188,10 @@ __global__ void __launch_bounds__(NSPLIT) tcp_prep_kernel(const __grid_constant_
     float my = 0.0f;
     for (int n0 = 0; n0 < 4 * NCK; n0 += 2) {
         bnd_issue(bi, ZX, ZX, f, gZ, d, t, n0);
-        bnd_reduce(bi, bxy, my, t, n0);
+        bnd_reduce<dd>(bi, bxy, my, t, n0);
     }
     __syncthreads();
-    if (t < 64) bnd_scales(bxy, bxy + 64, scb, d, t);  // bxy + 64: unused column bounds
+    if (t < 64) bnd_scales<dd>(bxy, bxy + 64, scb, d, t);  // bxy + 64: unused column bounds
     __syncthreads();
     if (t < 64) {
         float *xs = reinterpret_cast<float *>(const_cast<void *>(as.xs)) + p * 128;
@@ -1035,6 +1247,10 @@ cudaError_t tcp_run(const void *zx, const void *zy, void *zc, int64_t M, int d, 
 
 } // namespace
 
+bool mrc_tcp64_supported(int r, int m, int c) { return r == m && m == c && r >= 17 && r <= 64; }
+
+bool mrc_tcp64_default(int64_t M, int d) { return mrc_tcp64_supported(d, d, d) && (d >= 25 || M <= 256); }
+
 bool mrc_tcp_supported(int r, int m, int c) { return r == m && m == c && r >= 32 && r <= 64; }
 
 cudaError_t mrc_tcp_init(void)
@@ -1048,6 +1264,11 @@ cudaError_t mrc_tcp_init(void)
         if (e == cudaSuccess)
             e = cudaFuncSetAttribute(tcp_kernel_for<float, false>(k), cudaFuncAttributeMaxDynamicSharedMemorySize,
                                      TcL<float>::SMEM);
+        if (e != cudaSuccess) return e;
+    }
+    for (int k = 2; k <= 4; ++k) {
+        cudaError_t e = cudaFuncSetAttribute(tcp_kernel_for<double, false>(k), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             TcL<double>::SMEM);
         if (e != cudaSuccess) return e;
     }
     return cudaSuccess;
@@ -1093,9 +1314,16 @@ cudaError_t mrc_pairmul_f32_tcp(const void *zx, const void *zy, void *zc, int64_
     return tcp_run<float>(zx, zy, zc, M, d, tw, tw_log, status, st, 5);
 }
 
-cudaError_t mrc_tcp_seg(int dd_prec, const SegParams<PairArgs> &P, int *status, cudaStream_t st)
+cudaError_t mrc_pairmul_f64_tcp(const void *zx, const void *zy, void *zc, int64_t M, int d, const void *tw, int tw_log,
+                                int *status, cudaStream_t st)
 {
-    return dd_prec ? tcp_launch<dd>(P, status, st, 6) : tcp_launch<float>(P, status, st, 5);
+    return tcp_run<double>(zx, zy, zc, M, d, tw, tw_log, status, st, 4);
+}
+
+cudaError_t mrc_tcp_seg(int prec, const SegParams<PairArgs> &P, int *status, cudaStream_t st)
+{
+    if (prec == PREC_F64) return tcp_launch<double>(P, status, st, 4);
+    return prec == PREC_DD ? tcp_launch<dd>(P, status, st, 6) : tcp_launch<float>(P, status, st, 5);
 }
 
 PairArgs mrc_tcp_args(const void *zx, const void *zy, void *zc, int64_t M, int d, const void *tw, int tw_log)

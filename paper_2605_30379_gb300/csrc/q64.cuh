@@ -38,6 +38,7 @@ struct __align__(16) qtw {
 };
 
 constexpr int Q_TOP = 60;
+constexpr int Q_NONFINITE = 4096;  // alignment exponent of a column or row that holds an Inf or NaN
 constexpr int Q_MASK30 = (1 << 30) - 1;
 
 // biased exponent of a double (0 for zero and subnormals, 2047 for Inf / NaN)
@@ -149,4 +150,36 @@ __device__ __forceinline__ qtw q_twiddle(cx<double> w, int s, bool conj)
     const long long r = q_decode(w.re, 1022 + s, Q_TOP).v, i = q_decode(w.im, 1022 + s, Q_TOP, conj ? -1 : 0).v;
     const int rl = (int)(r << 2) >> 2, il = (int)(i << 2) >> 2;  // balanced 30-bit low limbs
     return {(int)((r - rl) >> 30), rl, (int)((i - il) >> 30), il};
+}
+
+// H 2^32 + L rounded to a double (|H| < 2^50, |L| < 2^50): the sum of a
+// product's weight groups, two halves of four
+__device__ __forceinline__ double q96_to_double(long long H, long long L)
+{
+    const long long hi = H + (L >> 32);
+    const unsigned lo = (unsigned)L;
+    const long long s = hi >> 63;
+    const unsigned al = s ? 0u - lo : lo;
+    const unsigned long long ah = (unsigned long long)(s ? ~hi + (lo == 0u ? 1 : 0) : hi);
+    // 2^13 (ah : al) = U : rest, U < 2^63
+    const unsigned long long U = (ah << 13) | (al >> 19);
+    const unsigned rest = al << 13;
+    const bool big = (U >> 31) != 0ull;
+    const unsigned long long W = big ? U : (U << 32) | rest;
+    const int lz = __clzll((long long)W);
+    const unsigned long long n = (W << (lz & 63)) | (big ? ((unsigned long long)rest << lz) >> 32 : 0ull);
+    const unsigned long long m = (n >> 11) + ((n >> 10) & 1ull);
+    const int e = 1023 + 63 - lz + (big ? 19 : -13);  // biased exponent of the leading bit
+    const unsigned long long b = W == 0ull ? 0ull : ((unsigned long long)(unsigned)(e - 1) << 52) + m;
+    return __longlong_as_double((long long)(b | ((unsigned long long)s & 0x8000000000000000ull)));
+}
+
+// x 2^de by its exponent (zero below the normal range, infinity above it)
+__device__ __forceinline__ double q_scale(double x, int de)
+{
+    const int hw = __double2hiint(x), e = ((hw >> 20) & 0x7ff) + de;
+    const bool z = (hw & 0x7ff00000) == 0 || e < 1;
+    const int sg = hw & (int)0x80000000;
+    const int h = z ? sg : (e > 2046 ? sg | 0x7ff00000 : hw + (de << 20));
+    return __hiloint2double(h, z || e > 2046 ? 0 : __double2loint(x));
 }

@@ -32,6 +32,10 @@ __device__ __forceinline__ uint64_t desc(unsigned addr)
 template <int M, int N>
 constexpr unsigned idesc_bf16() { return (1u << 4) | (1u << 7) | (1u << 10) | (1u << 15) | ((unsigned)(N >> 3) << 17) | ((unsigned)(M >> 4) << 24); }
 
+// the same with A and B both FP16 (formats 0)
+template <int M, int N>
+constexpr unsigned idesc_f16() { return (1u << 4) | (1u << 15) | ((unsigned)(N >> 3) << 17) | ((unsigned)(M >> 4) << 24); }
+
 // D (TMEM) (+)= A (smem) . B (smem); acc = 0 overwrites D
 template <unsigned IDESC>
 __device__ __forceinline__ void mma(unsigned dtm, uint64_t ad, uint64_t bd, unsigned acc)

@@ -84,3 +84,47 @@ def test_long_tails_and_spikes(mrc, d, N, seed):
     A = synth.identity_minus(q)
     psi = mrc.inverse(dev(A), prec="fp64").cpu().numpy()
     assert np.abs(psi - oracle.inverse_left(A)).max() <= 1e-12
+
+
+@pytest.mark.parametrize("N", [1, 2, 3, 40])
+@pytest.mark.parametrize("d", [15, 16, 17, 31, 32, 33, 48, 49, 63, 64, 65])
+def test_digit_product_sizes(mrc, d, N):
+    """The FP64 digit product (17 <= d <= 64: two to four K chunks of 16, full
+    and ragged) and the sizes just outside: M = 1 (the self-paired frequency
+    alone), 2, 4 and 64 points, integers with exact direct sums."""
+    rng = np.random.default_rng(100 * d + N)
+    A, B = integers(rng, N, d), integers(rng, N, d)
+    ref, _ = oracle.residuals(A, B)
+    got = mrc.residual(dev(A), dev(B), sides=1, prec="fp64")[0].cpu().numpy()
+    mrc.sync_status()
+    assert np.sqrt(((got - ref) ** 2).sum()) <= max(1e-2, 0.2 / N) * product_bound(A, B)
+
+
+def test_digit_product_row_and_column_scales(mrc):
+    """Rows of A and columns of B scaled by powers of two far apart: row i and
+    column j of the product scale exactly (rows and columns are aligned each by
+    itself)."""
+    rng = np.random.default_rng(8)
+    d, N = 20, 50
+    A, B = rng.standard_normal((N, d, d)), rng.standard_normal((N, d, d))
+    r, c = rng.integers(-200, 201, d), rng.integers(-200, 201, d)
+    A[0] += 3 * np.eye(d)
+    one = -mrc.residual(dev(A), dev(B), sides=1, prec="fp64")[0].cpu().numpy()
+    one[0] += np.eye(d)
+    two = -mrc.residual(dev(np.ldexp(A, r[None, :, None])), dev(np.ldexp(B, c[None, None, :])), sides=1,
+                        prec="fp64")[0].cpu().numpy()
+    two = np.ldexp(two, -r[None, :, None])
+    two = np.ldexp(two, -c[None, None, :])
+    assert np.array_equal(one[1:], two[1:])
+
+
+@pytest.mark.parametrize("bad", [np.nan, np.inf])
+def test_digit_product_non_finite(mrc, bad):
+    rng = np.random.default_rng(9)
+    A, B = rng.standard_normal((40, 20, 20)), rng.standard_normal((40, 20, 20))
+    ref = mrc.residual(dev(A), dev(B), sides=1, prec="fp64")[0]
+    B[3, 5, 7] = bad
+    got = mrc.residual(dev(A), dev(B), sides=1, prec="fp64")[0]
+    assert not torch.isfinite(got[:, :, 7]).any()
+    keep = [j for j in range(20) if j != 7]
+    assert torch.equal(got[:, :, keep], ref[:, :, keep])
