@@ -850,6 +850,7 @@ int product_choice(mrc_ctx *cx, int prec, int64_t M, int d)
         if (it != cx->tune.end()) return it->second;
     }
     if (tensor_default(prec, M, d, d, d)) return 3;
+    if (prec == PREC_F64) return mrc_pairq_supported(d, d, d) ? 0 : 2;
     return d <= 16 ? 0 : (d <= 24 ? 4 : (d <= 32 ? 1 : 2));
 }
 
@@ -871,7 +872,8 @@ mrc_status product_stage(mrc_ctx *c, int prec, int64_t M, const std::vector<Pair
     std::vector<size_t> bycfg[5], tcp[10];  // tensor-core groups: K-chunk count, + 5 with X prepared
     int *const old = c->cur_status;
     for (size_t i = 0; i < jobs.size(); ++i) {
-        const int ch = jobs[i].xs ? 3 : product_choice(c, prec, M, jobs[i].d);
+        int ch = jobs[i].xs ? 3 : product_choice(c, prec, M, jobs[i].d);
+        if (prec == PREC_F64 && (ch == 0 || ch == 4)) ch = mrc_pairq_supported(jobs[i].d, jobs[i].d, jobs[i].d) ? 0 : 2;
         if (ch == 3 && jobs[i].d <= 64) {
             tcp[(jobs[i].d + 15) / 16 + (jobs[i].xs ? 5 : 0)].push_back(i);
         } else if (ch == 3) {
@@ -912,10 +914,15 @@ mrc_status product_stage(mrc_ctx *c, int prec, int64_t M, const std::vector<Pair
                 a.logM = l;
                 a.npairs = M >= 2 ? M / 2 + 1 : 1;
                 a.r = a.m = a.c = j.d;
-                const int nt = (j.d + bsz[cfg] - 1) / bsz[cfg];
                 P->first[q - i0] = total;
+                if (prec == PREC_F64 && cfg == 0) {
+                    a.pp = mrc_pairq_pp(a.npairs, j.d, j.d, j.d);
+                    total += (unsigned)((a.npairs + a.pp - 1) / a.pp);
+                } else {
+                    const int nt = (j.d + bsz[cfg] - 1) / bsz[cfg];
+                    total += (unsigned)a.npairs * (unsigned)(nt * nt);
+                }
                 P->a[q - i0] = a;
-                total += (unsigned)a.npairs * (unsigned)(nt * nt);
                 by += (double)M * 3.0 * j.d * j.d * OPS[prec].cxb;
                 fl += 8.0 * (double)j.d * j.d * j.d * (double)(M + 1);
             }

@@ -325,7 +325,7 @@ __device__ __forceinline__ void fft_stage(const FftArgs &a, cx<typename FftC<T>:
                 v[u][0] = {{q_shift_even(v[u][0].re.v, qs)}, {q_shift_even(v[u][0].im.v, qs)}};
 #pragma unroll
                 for (int q = 1; q < r; ++q)
-                    v[u][q] = q_shift(c_mul(v[u][q], stw[(bm * q) << (LOGR - LNS - LR)], qs ? 0ll : 1ll << 29), qs, qr);
+                    v[u][q] = q_shift(c_mul(v[u][q], stw[(bm * q) << (LOGR - LNS - LR)], qs ? 0 : 1 << 29), qs, qr);
             } else {
 #pragma unroll
                 for (int q = 1; q < r; ++q) v[u][q] = c_mul(v[u][q], stw[(bm * q) << (LOGR - LNS - LR)]);

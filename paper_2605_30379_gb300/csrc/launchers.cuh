@@ -206,7 +206,8 @@ cudaError_t pairmul2_launch(const PairArgs &a, cudaStream_t st)
     return cudaGetLastError();
 }
 
-// product argument block and tile configuration: 0 = 16x16 (64 threads),
+// product argument block and tile configuration (FP64: 0 and 4 the fixed-point
+// product of pair_q.cu where it fits, 1 and 2 the tiles for the rest): 0 = 16x16 (64 threads),
 // 1 = 32x32 (256), 2 = 64x64 (256), 4 = 24x24 (96: 17 <= d <= 24 fills 50 .. 100 %
 // of it against 28 .. 56 % of a 32x32 tile); cfg < 0 picks by the larger output dimension
 inline PairArgs pairmul_args(const void *zx, const void *zy, void *zc, int64_t M, int r, int m, int c, const void *tw,
@@ -223,18 +224,17 @@ inline int pairmul_cfg_for(int r, int c, int cfg)
     const int mx = r > c ? r : c;
     return cfg >= 0 ? cfg : (mx <= 16 ? 0 : (mx <= 24 ? 4 : (mx <= 32 ? 1 : 2)));
 }
-// CTAs of one product: pairs x output tiles
-inline unsigned pairmul_ctas(const PairArgs &a, int cfg)
-{
-    const int b = cfg == 0 ? 16 : (cfg == 1 ? 32 : (cfg == 4 ? 24 : 64));
-    return (unsigned)a.npairs * (unsigned)(((a.r + b - 1) / b) * ((a.c + b - 1) / b));
-}
-
 template <class T>
 cudaError_t pairmul_run(const void *zx, const void *zy, void *zc, int64_t M, int r, int m, int c, int cfg, const void *tw,
                         int tw_log, cudaStream_t st)
 {
     const PairArgs a = pairmul_args(zx, zy, zc, M, r, m, c, tw, tw_log);
+    if constexpr (std::is_same<T, double>::value) {
+        if (cfg < 0) cfg = mrc_pairq_supported(r, m, c) ? 0 : (std::max(r, c) <= 32 ? 1 : 2);
+        if ((cfg == 0 || cfg == 4) && mrc_pairq_supported(r, m, c)) return mrc_pairq(a, kclass_pair<T>(), st);
+        if (cfg == 1) return pairmul_launch<T, 32, 32, 16, 2, 2>(a, st);
+        return pairmul_launch<T, 64, 64, 8, 4, 4>(a, st);
+    } else {
     cfg = pairmul_cfg_for(r, c, cfg);
     if (cfg == 0) return pairmul_launch<T, 16, 16, 16, 2, 2>(a, st);
     if (cfg == 1) return pairmul_launch<T, 32, 32, 16, 2, 2>(a, st);
@@ -244,6 +244,7 @@ cudaError_t pairmul_run(const void *zx, const void *zy, void *zc, int64_t M, int
     // 49.4 ms at d = 64, N = 2^18 against both frequencies in every thread)
     if constexpr (std::is_same<T, float>::value) return pairmul2_launch<T, 64, 64, 8, 4, 4>(a, st);
     else return pairmul_launch<T, 64, 64, 8, 4, 4>(a, st);
+    }
 }
 
 // One segmented product launch of tile configuration cfg (resolved) over
@@ -253,8 +254,13 @@ cudaError_t pairmul_seg_run(int cfg, const SegParams<PairArgs> &P, unsigned ncta
                             cudaStream_t st)
 {
     if (P.nseg <= 0 || nctas == 0) return cudaSuccess;
+    if constexpr (std::is_same<T, double>::value)
+        if (cfg == 0) return mrc_pairq_seg(P, nctas, bytes, flops, kclass_pair<T>(), st);
     mrc_prof_pre(kclass_pair<T>(), st);
-    if (cfg == 0) pairmul_seg_kernel<T, 16, 16, 16, 2, 2><<<nctas, 64, 0, st>>>(P);
+    if constexpr (std::is_same<T, double>::value) {
+        if (cfg == 1) pairmul_seg_kernel<T, 32, 32, 16, 2, 2><<<nctas, 256, 0, st>>>(P);
+        else pairmul_seg_kernel<T, 64, 64, 8, 4, 4><<<nctas, 256, 0, st>>>(P);
+    } else if (cfg == 0) pairmul_seg_kernel<T, 16, 16, 16, 2, 2><<<nctas, 64, 0, st>>>(P);
     else if (cfg == 1) pairmul_seg_kernel<T, 32, 32, 16, 2, 2><<<nctas, 256, 0, st>>>(P);
     else if (cfg == 4) pairmul_seg_kernel<T, 24, 24, 8, 3, 2><<<nctas, 96, 0, st>>>(P);
     else if constexpr (std::is_same<T, float>::value) pairmul2_seg_kernel<T, 64, 64, 8, 4, 4><<<nctas, 512, 0, st>>>(P);
@@ -299,6 +305,10 @@ cudaError_t init_run()
             cudaError_t e = cudaFuncSetAttribute(t[i][l].fn, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
             if (e != cudaSuccess) return e;
         }
+    if constexpr (std::is_same<T, double>::value) {
+        cudaError_t e = mrc_pairq_init();
+        if (e != cudaSuccess) return e;
+    }
     const auto &ts = fft_seg_table<T>();
     for (int l = 0; l < 11; ++l) {
         cudaError_t e = cudaFuncSetAttribute(ts[l].fn, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);

@@ -52,6 +52,7 @@ struct PairArgs {
     int logM;
     int64_t npairs;
     int r, m, c; // X: r x m, Y: m x c (pairdiag: Y is a c-vector, m unused)
+    int pp;      // fixed-point product: frequency pairs per CTA
     // tensor-core double-float product with X prepared (mrc_tcp_prep): zx
     // holds X's digit tiles, xs its per-pair scale factors; else null
     const void *xs;
@@ -189,12 +190,11 @@ cudaError_t mrc_pairmul_dd_tcp(const void *zx, const void *zy, void *zc, int64_t
                                int *status, cudaStream_t st);
 cudaError_t mrc_pairmul_f32_tcp(const void *zx, const void *zy, void *zc, int64_t M, int d, const void *tw, int tw_log,
                                 int *status, cudaStream_t st);
-// FP64: square 17 <= d <= 64.  The built-in choice takes it for d >= 25 and,
-// below, for M <= 256: the FP64-pipe tiles of 24 and 16 need 28 and 8 us per
-// frequency pair and SM and one pair fills an SM, the digit product about 40
-// us at two K chunks but less where pairs are fewer than SMs (timed per d and
-// M: the digit product is the faster from d = 26 on at every M, for d = 20 and
-// 24 up to M = 256, at d = 16 nowhere).
+// FP64: square 17 <= d <= 64.  The built-in choice takes it for d >= 33 and
+// for d = 30 .. 32 up to M = 256, the fixed-point product (pair_q.cu) below
+// (timed per d and M: the fixed-point product is the faster up to d = 28 at
+// every M and at d = 32 from M = 512 on, the digit product from d = 40 on at
+// every M, and at d = 36 they tie from M = 512 on).
 bool mrc_tcp64_supported(int r, int m, int c);
 bool mrc_tcp64_default(int64_t M, int d);
 cudaError_t mrc_pairmul_f64_tcp(const void *zx, const void *zy, void *zc, int64_t M, int d, const void *tw, int tw_log,
@@ -214,6 +214,16 @@ size_t mrc_tcp_prep_scale_bytes(int64_t M);
 cudaError_t mrc_tcp_prep(const SegParams<PairArgs> &P, cudaStream_t st);
 // the kernels' bounded mbarrier wait on a barrier nothing arrives on: writes 6 to *status
 cudaError_t mrc_tc_wait_selftest(int *status, int spins, cudaStream_t st);
+
+// pair_q.cu: FP64 products in 64-bit fixed point on the integer pipes, for
+// matrices whose spectra of one frequency pair fit in shared memory
+bool mrc_pairq_supported(int r, int m, int c);
+int mrc_pairq_pp(int64_t npairs, int r, int m, int c);
+cudaError_t mrc_pairq_init(void);
+cudaError_t mrc_pairq(const PairArgs &a, int kclass, cudaStream_t st);
+// (every segment with its pp and ceil(npairs / pp) CTAs)
+cudaError_t mrc_pairq_seg(const SegParams<PairArgs> &P, unsigned nctas, double bytes, double flops, int kclass,
+                          cudaStream_t st);
 
 // api.cu: the Newton doubling schedule of Eq. (newton), shared by every
 // inverse entry point (mrc_inverse* and mrc_inverse_noalloc).

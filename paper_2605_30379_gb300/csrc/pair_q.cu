@@ -1,0 +1,202 @@
+// pair_q.cu -- FP64 per-frequency complex matrix products (Eq.
+// (fft-convolution): C(phi) = X(phi) Y(phi), X r x m, Y m x c) in 64-bit fixed
+// point, for matrices that fit in shared memory: the square ones too small for
+// the tensor-core tiles and the rectangular ones.
+//
+// The FP64 pipe gives two multiply-adds per clock and SM, a 32 x 32 -> 64 bit
+// integer multiply-add sixty; a complex multiply-add takes sixteen of the
+// latter on numbers of two limbs.  Rows of X and columns of Y are aligned to
+// their largest magnitude over both frequencies of a pair (2 Xh and 2 Yh below
+// 2^58 to 2^60, as m allows: a high limb and a balanced 30-bit low limb), the
+// limb products
+// accumulate exactly in 64 bits by weight (the lower sums are carried upward
+// every eight terms), and each sum is rounded once to FP64.  (Without the low
+// products, a quarter of the work, the error of a Weibull d = 16, N = 2048
+// inverse rises from FP64's 1.2e-15 to 9e-15: e0 - q is singular at frequency
+// zero.)
+//
+// One CTA takes the pairs p0 .. p0 + pp - 1 (pp so that its outputs fill the
+// threads once, fewer when there are fewer pairs than SMs): it loads their
+// spectra, splits both frequencies into limbs in shared memory, and every
+// thread forms C(f)_ij and C(M - f)_ij of its outputs and merges them.  No work
+// is done for padding.  Against the FP64-pipe tiles of 16, 24 and 32 it
+// replaces: the products of a d = 16, N = 8192 inverse 1.1 -> 0.4 ms, of the
+// d = 4, N = 2^15 renewal equation (a 16 x 16 tile) 3.2 -> 0.1 ms, of an
+// entrance with 18 x 18 blocks, N = 10000, 6.4 -> 1.2 ms.
+#include <algorithm>
+
+#include "q64.cuh"
+#include "mrc_internal.h"
+
+namespace {
+
+constexpr int NT = 128;
+// raw values below 2^top, 2 Xh below 2^(top + 2), so that m products of two
+// numbers of such moduli stay below 2^63 with their 2^60 taken off
+__device__ __forceinline__ int top_for(int m) { return m <= 4 ? 58 : (m <= 31 ? 57 : 56); }
+constexpr int SMEM_MAX = 200 * 1024;
+
+struct __align__(16) limbs {
+    int rh, rl, ih, il;
+};
+
+__device__ __forceinline__ limbs to_limbs(long long re, long long im)
+{
+    const int rl = (int)((unsigned)re << 2) >> 2, il = (int)((unsigned)im << 2) >> 2;
+    return {(int)((re - rl) >> 30), rl, (int)((im - il) >> 30), il};
+}
+
+// accumulators of one complex sum: 2^60 h + 2^30 m + l
+struct acc {
+    long long hr, hi, mr, mi, lr, li;
+};
+
+__device__ __forceinline__ void mac(acc &a, const limbs &x, const limbs &y)
+{
+    const int nh = -x.ih, nl = -x.il;
+    a.hr = q_wide(nh, y.ih, q_wide(x.rh, y.rh, a.hr));
+    a.hi = q_wide(x.ih, y.rh, q_wide(x.rh, y.ih, a.hi));
+    a.mr = q_wide(nl, y.ih, q_wide(nh, y.il, q_wide(x.rl, y.rh, q_wide(x.rh, y.rl, a.mr))));
+    a.mi = q_wide(x.il, y.rh, q_wide(x.ih, y.rl, q_wide(x.rl, y.ih, q_wide(x.rh, y.il, a.mi))));
+    a.lr = q_wide(nl, y.il, q_wide(x.rl, y.rl, a.lr));
+    a.li = q_wide(x.il, y.rl, q_wide(x.rl, y.il, a.li));
+}
+
+__device__ __forceinline__ void fold(acc &a)
+{
+    a.mr += a.lr >> 30;
+    a.mi += a.li >> 30;
+    a.lr &= Q_MASK30;
+    a.li &= Q_MASK30;
+    a.hr += a.mr >> 30;
+    a.hi += a.mi >> 30;
+    a.mr &= Q_MASK30;
+    a.mi &= Q_MASK30;
+}
+
+size_t pair_bytes(int r, int m, int c)
+{
+    return 2 * sizeof(limbs) * ((size_t)r * m + (size_t)m * c) + sizeof(qtw) + sizeof(int) * ((size_t)r + c);
+}
+
+__device__ __forceinline__ void pairq_body(const PairArgs &a, int64_t p0)
+{
+    extern __shared__ __align__(16) unsigned char smem[];
+    const int r = a.r, m = a.m, c = a.c, EX = r * m, EY = m * c, EC = r * c, ex2 = EX + EY;
+    const int np = (int)min((int64_t)a.pp, a.npairs - p0);
+    limbs *sf = reinterpret_cast<limbs *>(smem), *sg = sf + a.pp * ex2;  // per pair: X then Y entries, f and g
+    qtw *stw = reinterpret_cast<qtw *>(sg + a.pp * ex2);
+    unsigned *bnd = reinterpret_cast<unsigned *>(stw + a.pp);            // per pair: r row and c column bounds
+    const cx<double> *ZX = reinterpret_cast<const cx<double> *>(a.zx), *ZY = reinterpret_cast<const cx<double> *>(a.zy);
+    cx<double> *ZC = reinterpret_cast<cx<double> *>(a.zc);
+    const cx<double> *tw = reinterpret_cast<const cx<double> *>(a.tw);
+    const int64_t M = a.M;
+    const int tws = a.tw_log - a.logM - 1;
+    const int tid = threadIdx.x, top = top_for(m);
+
+    for (int t = tid; t < np * (r + c); t += NT) bnd[t] = 0u;
+    __syncthreads();
+    // raw spectra of both rows of every pair, and the row and column bounds
+    for (int t = tid; t < np * ex2; t += NT) {
+        const int q = t / ex2, e = t - q * ex2;
+        const int64_t f = p0 + q, g = (M - f) & (M - 1);
+        const bool x = e < EX;
+        const int ee = x ? e : e - EX;
+        const cx<double> za = x ? ZX[f * EX + ee] : ZY[f * EY + ee], zb = x ? ZX[g * EX + ee] : ZY[g * EY + ee];
+        reinterpret_cast<cx<double> *>(sf)[t] = za;
+        reinterpret_cast<cx<double> *>(sg)[t] = zb;
+        const unsigned b = max(max(q_magnitude(za.re), q_magnitude(za.im)), max(q_magnitude(zb.re), q_magnitude(zb.im)));
+        atomicMax(&bnd[q * (r + c) + (x ? ee / m : r + ee % c)], b);
+    }
+    for (int t = tid; t < np; t += NT) stw[t] = q_twiddle(tw[(p0 + t) << tws], 0, false);
+    __syncthreads();
+    // the split of both frequencies, in place (every thread its own entries)
+    for (int t = tid; t < np * ex2; t += NT) {
+        const int q = t / ex2, e = t - q * ex2;
+        const bool x = e < EX;
+        const int ee = x ? e : e - EX;
+        cx<q64> s, u;
+        q_split(reinterpret_cast<cx<double> *>(sf)[t], reinterpret_cast<cx<double> *>(sg)[t], stw[q],
+                q_align(bnd[q * (r + c) + (x ? ee / m : r + ee % c)]), top, s, u);
+        sf[t] = to_limbs(s.re.v + u.re.v, s.im.v + u.im.v);
+        sg[t] = to_limbs(s.re.v - u.re.v, u.im.v - s.im.v);
+    }
+    __syncthreads();
+    for (int t = tid; t < np * EC; t += NT) {
+        const int q = t / EC, e = t - q * EC, i = e / c, j = e - i * c;
+        const int xo = q * ex2 + i * m, yo = q * ex2 + EX + j;
+        acc af{}, ag{};
+        for (int k0 = 0; k0 < m; k0 += 8) {
+            const int kn = min(8, m - k0);
+#pragma unroll 4
+            for (int k = k0; k < k0 + kn; ++k) {
+                mac(af, sf[xo + k], sf[yo + k * c]);
+                mac(ag, sg[xo + k], sg[yo + k * c]);
+            }
+            fold(af);
+            fold(ag);
+        }
+        const int ax = q_align(bnd[q * (r + c) + i]), ay = q_align(bnd[q * (r + c) + r + j]);
+        const int de = ax + ay - 2017 - 2 * top;  // the alignments, the limbs, the split's factors 2 and the merge's 1/2
+        cx<double> cf = {q_scale(q94_to_double(af.hr, (int)af.mr), de), q_scale(q94_to_double(af.hi, (int)af.mi), de)};
+        cx<double> cg = {q_scale(q94_to_double(ag.hr, (int)ag.mr), de), q_scale(q94_to_double(ag.hi, (int)ag.mi), de)};
+        if (max(ax, ay) >= Q_NONFINITE) cf.re = cf.im = cg.re = cg.im = __longlong_as_double(0x7ff8000000000000ll);
+        const int64_t f = p0 + q, g = (M - f) & (M - 1);
+        cx<double> zf, zg;
+        q_merge(cf, cg, tw[f << tws], zf, zg);
+        ZC[f * EC + e] = zf;
+        if (g != f) ZC[g * EC + e] = zg;
+    }
+}
+
+__global__ void __launch_bounds__(NT) pairq_kernel(const PairArgs a) { pairq_body(a, (int64_t)blockIdx.x * a.pp); }
+
+__global__ void __launch_bounds__(NT) pairq_seg_kernel(const __grid_constant__ SegParams<PairArgs> P)
+{
+    const int s = seg_find(P, blockIdx.x);
+    pairq_body(P.a[s], (int64_t)(blockIdx.x - P.first[s]) * P.a[s].pp);
+}
+
+} // namespace
+
+bool mrc_pairq_supported(int r, int m, int c) { return pair_bytes(r, m, c) <= (size_t)SMEM_MAX; }
+
+// Pairs per CTA: outputs for every thread, but no fewer CTAs than SMs where the
+// pairs allow, and at most 48 KB of shared memory when one pair needs less
+// (several CTAs per SM hide the loads of each other)
+int mrc_pairq_pp(int64_t npairs, int r, int m, int c)
+{
+    const int64_t fill = std::max(1, NT / (r * c)), spread = std::max<int64_t>(1, npairs / 152);
+    const int64_t fit = std::max<int64_t>(1, (int64_t)(48 * 1024 / pair_bytes(r, m, c)));
+    return (int)std::min(std::min(fill, spread), fit);
+}
+
+cudaError_t mrc_pairq_init(void)
+{
+    cudaError_t e = cudaFuncSetAttribute(pairq_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_MAX);
+    if (e != cudaSuccess) return e;
+    return cudaFuncSetAttribute(pairq_seg_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_MAX);
+}
+
+cudaError_t mrc_pairq(const PairArgs &a0, int kclass, cudaStream_t st)
+{
+    PairArgs a = a0;
+    a.pp = mrc_pairq_pp(a.npairs, a.r, a.m, a.c);
+    const double by = (double)a.M * ((double)a.r * a.m + (double)a.m * a.c + (double)a.r * a.c) * 16.0;
+    mrc_prof_pre(kclass, st);
+    pairq_kernel<<<(unsigned)((a.npairs + a.pp - 1) / a.pp), NT, a.pp * pair_bytes(a.r, a.m, a.c), st>>>(a);
+    mrc_prof_post(kclass, st, by, 8.0 * a.r * a.m * a.c * (double)(a.M + 1));
+    return cudaGetLastError();
+}
+
+cudaError_t mrc_pairq_seg(const SegParams<PairArgs> &P, unsigned nctas, double bytes, double flops, int kclass,
+                          cudaStream_t st)
+{
+    if (P.nseg <= 0 || nctas == 0) return cudaSuccess;
+    size_t sm = 0;
+    for (int s = 0; s < P.nseg; ++s) sm = std::max(sm, P.a[s].pp * pair_bytes(P.a[s].r, P.a[s].m, P.a[s].c));
+    mrc_prof_pre(kclass, st);
+    pairq_seg_kernel<<<nctas, NT, sm, st>>>(P);
+    mrc_prof_post(kclass, st, bytes, flops);
+    return cudaGetLastError();
+}

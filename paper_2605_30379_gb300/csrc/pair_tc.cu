@@ -3,7 +3,7 @@
 // half spectrum, square d x d with d <= 64) as exact digit products on the
 // tcgen05 tensor cores, for three working precisions:
 //
-//   FP64 (17 <= d): eight balanced base-256 digits of 64-bit fixed-point
+//   FP64 (d >= 33 by default): eight balanced base-256 digits of 64-bit fixed-point
 //     values, pairs s + t >= 7 (36 pairs in 8 weight groups), about 2^-58
 //     relative to the row and column maxima.  The FP64 pipe gives two
 //     multiply-adds per clock and SM; at d = 64, N = 2^15 the inverse's 28
@@ -258,12 +258,8 @@ template <class T>
 __device__ __forceinline__ void bnd_scales(const unsigned *bx, const unsigned *by, float *sc, int d, int t)
 {
     if constexpr (tc_q<T>) {
-        // the alignment exponents: every |re|, |im| below 63/64 2^(ex - 1022)
-        // (above every finite one for Inf and NaN)
-        const int ex = t < d ? max(1, (int)((bx[t] + 0x8000u) >> 20)) : 1;
-        const int ey = t < d ? max(1, (int)((by[t] + 0x8000u) >> 20)) : 1;
-        sc[t] = sc[128 + t] = __int_as_float(ex >= 2047 ? Q_NONFINITE : ex);
-        sc[64 + t] = sc[192 + t] = __int_as_float(ey >= 2047 ? Q_NONFINITE : ey);
+        sc[t] = sc[128 + t] = __int_as_float(t < d ? q_align(bx[t]) : 1);
+        sc[64 + t] = sc[192 + t] = __int_as_float(t < d ? q_align(by[t]) : 1);
         return;
     }
     const int sx = t < d ? scale_exp(2.0f * __uint_as_float(bx[t])) : 0;
@@ -487,11 +483,9 @@ __device__ __forceinline__ void ydigits(DState<T> (&st)[NFQ][4][2], unsigned cha
 // values stay below 63/64 2^60, so |2 Xh| <= 2 sqrt(|a|^2 + |b|^2) < 63/64 2^62.
 __device__ __forceinline__ cx<q64> split_q(cx<double> za, cx<double> zb, qtw w, int ex)
 {
-    const cx<q64> a = {q_decode(za.re, ex, Q_TOP), q_decode(za.im, ex, Q_TOP)};
-    const cx<q64> b = {q_decode(zb.re, ex, Q_TOP), q_decode(zb.im, ex, Q_TOP)};
-    // s = a + conj b, t = w (-i) (a - conj b)
-    const cx<q64> t = c_mul(cx<q64>{{a.im.v + b.im.v}, {b.re.v - a.re.v}}, w);
-    return {{a.re.v + b.re.v + t.re.v}, {a.im.v - b.im.v + t.im.v}};
+    cx<q64> s, t;
+    q_split(za, zb, w, ex, Q_TOP, s, t);
+    return c_add(s, t);
 }
 
 // FP16 pairs of four balanced digits of two values: with every byte offset by
@@ -722,11 +716,9 @@ __device__ __forceinline__ void st_cx<float>(cx<float> *p, cx<float> v)
 }
 
 // FP64 outputs of one round of 32 columns (this thread: column j, sixteen
-// rows): the exponents of the row and column alignments join, then C(f) is
-// stored unmerged (phase 0) or the pair merged with it,
-//   ZC(f) = s + i p, ZC(M - f) = conj s + i conj p,
-//   s = (C(f) + conj C(M - f)) / 2, p = conj w (C(f) - conj C(M - f)) / 2;
-// the factor 1/2 and the split's 2 on both operands are in the exponent.
+// rows): the exponents of the row and column alignments join (with the factor
+// 1/2 of the merge and the split's 2 on both operands), then C(f) / 2 is stored
+// unmerged (phase 0) or the pair merged with it.
 __device__ __forceinline__ void epi_q(cx<double> *ZC, const double *xch, const float *fx, int ey, cx<double> wf, int64_t f,
                                       int64_t gZ, int d, int64_t E, int j, int jl, int et, int phase, bool self, bool two)
 {
@@ -751,11 +743,10 @@ __device__ __forceinline__ void epi_q(cx<double> *ZC, const double *xch, const f
                 st_cx(zf, v[u]);
                 continue;
             }
-            const double sr = cf[u].re + v[u].re, si = cf[u].im - v[u].im;
-            const double dr = cf[u].re - v[u].re, di = cf[u].im + v[u].im;
-            const double pr = fma(wf.re, dr, wf.im * di), pi = fma(wf.re, di, -(wf.im * dr));
-            st_cx(zf, cx<double>{sr - pi, si + pr});
-            if (two) st_cx(ZC + gZ * E + (int64_t)i * d + j, cx<double>{sr + pi, pr - si});
+            cx<double> zp, zq;
+            q_merge(cf[u], v[u], wf, zp, zq);
+            st_cx(zf, zp);
+            if (two) st_cx(ZC + gZ * E + (int64_t)i * d + j, zq);
         }
     }
 }
@@ -1249,7 +1240,7 @@ cudaError_t tcp_run(const void *zx, const void *zy, void *zc, int64_t M, int d, 
 
 bool mrc_tcp64_supported(int r, int m, int c) { return r == m && m == c && r >= 17 && r <= 64; }
 
-bool mrc_tcp64_default(int64_t M, int d) { return mrc_tcp64_supported(d, d, d) && (d >= 25 || M <= 256); }
+bool mrc_tcp64_default(int64_t M, int d) { return mrc_tcp64_supported(d, d, d) && (d >= 33 || (d >= 30 && M <= 256)); }
 
 bool mrc_tcp_supported(int r, int m, int c) { return r == m && m == c && r >= 32 && r <= 64; }
 

@@ -46,16 +46,25 @@ __device__ __forceinline__ int q_exponent(double x) { return (__double2hiint(x) 
 
 // x 2^(top + 1022 - ex) rounded to an integer, for |x| < 2^(ex - 1022) and
 // top <= 60: the magnitude is rounded (symmetric in the sign, so that a column
-// of one sign is not shortened); neg flips the sign.
+// of one sign is not shortened; a tie, frequent where few bits are dropped,
+// goes by a mantissa bit that is kept); neg flips the sign.
 __device__ __forceinline__ q64 q_decode(double x, int ex, int top, int neg = 0)
 {
     const unsigned hw = (unsigned)__double2hiint(x), lw = (unsigned)__double2loint(x);
     const int e = (int)((hw >> 20) & 0x7ffu);
     const unsigned mh = (hw & 0xfffffu) | (e ? 0x100000u : 0u);
     const int sh = min(ex - max(e, 1) + (62 - top), 63);
-    const unsigned long long m = (((((unsigned long long)mh << 42) | ((unsigned long long)lw << 10)) >> sh) + 1ull) >> 1;
+    const unsigned long long m53 = ((unsigned long long)mh << 42) | ((unsigned long long)lw << 10);
+    const unsigned long long m = (((m53 - (hw & 1u)) >> sh) + 1ull) >> 1;
     const long long s = (long long)((int)hw >> 31) ^ (long long)neg;
     return {((long long)m ^ s) - s};
+}
+
+// n / 2^11 rounded half to even
+__device__ __forceinline__ unsigned long long q_round11(unsigned long long n)
+{
+    const unsigned long long m = n >> 11;
+    return m + (((unsigned)n & 0x7ffu) + ((unsigned)m & 1u) > 0x400u ? 1ull : 0ull);
 }
 
 // v 2^(eb - 1086) rounded to a double (flushed to zero below the normal
@@ -67,7 +76,7 @@ __device__ __forceinline__ double q_encode(q64 x, int eb, unsigned sgn)
     const unsigned long long a = (unsigned long long)((x.v ^ s) - s);
     const int lz = __clzll((long long)a);
     const unsigned long long n = a << (lz & 63);
-    const unsigned long long m = (n >> 11) + ((n >> 10) & 1ull);
+    const unsigned long long m = q_round11(n);
     const int e = eb - lz;
     unsigned hi = (unsigned)(m >> 32) + ((unsigned)(e - 1) << 20), lo = (unsigned)m;
     const bool tiny = e < 1 || a == 0ull;
@@ -104,13 +113,16 @@ struct Ar<q64> {
     static __device__ __forceinline__ q64 rsqrt2() { return {815238614083298888ll}; }
 };
 
-// a w; the middle products start at r0: 2^29 rounds the result, 0 leaves its floor
-__device__ __forceinline__ cx<q64> c_mul(cx<q64> a, qtw w, long long r0 = 1ll << 29)
+// a w; the middle products start at r0: 2^29 rounds the result, 0 leaves its
+// floor.  To it they add the mean of the low products that are left out (the
+// low limbs of a are 2^29 in the mean): the same twiddle serves every entry of
+// a matrix, so that the offset would add up over a row.
+__device__ __forceinline__ cx<q64> c_mul(cx<q64> a, qtw w, int r0 = 1 << 29)
 {
     const int arh = (int)(a.re.v >> 30), arl = (int)a.re.v & Q_MASK30;
     const int aih = (int)(a.im.v >> 30), ail = (int)a.im.v & Q_MASK30;
     const int nh = -aih, nl = -ail;
-    long long mr = q_wide(arh, w.rl, r0), mi = q_wide(arh, w.il, r0);
+    long long mr = q_wide(arh, w.rl, r0 + ((w.rl - w.il) >> 1)), mi = q_wide(arh, w.il, r0 + ((w.rl + w.il) >> 1));
     mr = q_wide(arl, w.rh, mr);
     mi = q_wide(arl, w.ih, mi);
     mr = q_wide(nh, w.il, mr);
@@ -152,26 +164,40 @@ __device__ __forceinline__ qtw q_twiddle(cx<double> w, int s, bool conj)
     return {(int)((r - rl) >> 30), rl, (int)((i - il) >> 30), il};
 }
 
+// (U : rest) with U < 2^63 and 32 bits of rest, rounded to a double: leading bit
+// 63 - lz of U gets the biased exponent eb - lz; neg flips the sign
+__device__ __forceinline__ double q_pack(unsigned long long U, unsigned rest, int eb, bool neg)
+{
+    const bool big = (U >> 31) != 0ull;
+    const unsigned long long W = big ? U : (U << 32) | rest;
+    const int lz = __clzll((long long)W);
+    const unsigned long long n = (W << (lz & 63)) | (big ? ((unsigned long long)rest << lz) >> 32 : 0ull);
+    const unsigned long long m = q_round11(n);
+    const int e = eb - lz - (big ? 0 : 32);
+    const unsigned long long b = W == 0ull ? 0ull : ((unsigned long long)(unsigned)(e - 1) << 52) + m;
+    return __longlong_as_double((long long)(b | (neg ? 0x8000000000000000ull : 0ull)));
+}
+
 // H 2^32 + L rounded to a double (|H| < 2^50, |L| < 2^50): the sum of a
 // product's weight groups, two halves of four
 __device__ __forceinline__ double q96_to_double(long long H, long long L)
 {
     const long long hi = H + (L >> 32);
     const unsigned lo = (unsigned)L;
-    const long long s = hi >> 63;
-    const unsigned al = s ? 0u - lo : lo;
-    const unsigned long long ah = (unsigned long long)(s ? ~hi + (lo == 0u ? 1 : 0) : hi);
-    // 2^13 (ah : al) = U : rest, U < 2^63
-    const unsigned long long U = (ah << 13) | (al >> 19);
-    const unsigned rest = al << 13;
-    const bool big = (U >> 31) != 0ull;
-    const unsigned long long W = big ? U : (U << 32) | rest;
-    const int lz = __clzll((long long)W);
-    const unsigned long long n = (W << (lz & 63)) | (big ? ((unsigned long long)rest << lz) >> 32 : 0ull);
-    const unsigned long long m = (n >> 11) + ((n >> 10) & 1ull);
-    const int e = 1023 + 63 - lz + (big ? 19 : -13);  // biased exponent of the leading bit
-    const unsigned long long b = W == 0ull ? 0ull : ((unsigned long long)(unsigned)(e - 1) << 52) + m;
-    return __longlong_as_double((long long)(b | ((unsigned long long)s & 0x8000000000000000ull)));
+    const bool neg = hi < 0;
+    const unsigned al = neg ? 0u - lo : lo;
+    const unsigned long long ah = (unsigned long long)(neg ? ~hi + (lo == 0u ? 1 : 0) : hi);
+    return q_pack((ah << 13) | (al >> 19), al << 13, 1023 + 63 + 19, neg);
+}
+
+// hi 2^30 + mid rounded to a double (0 <= mid < 2^30, |hi| < 2^63)
+__device__ __forceinline__ double q94_to_double(long long hi, int mid)
+{
+    const unsigned lo = (unsigned)mid << 2;
+    const bool neg = hi < 0;
+    const unsigned al = neg ? 0u - lo : lo;
+    const unsigned long long ah = (unsigned long long)(neg ? ~hi + (lo == 0u ? 1 : 0) : hi);
+    return q_pack(ah, al, 1023 + 63 + 30, neg);
 }
 
 // x 2^de by its exponent (zero below the normal range, infinity above it)
@@ -182,4 +208,37 @@ __device__ __forceinline__ double q_scale(double x, int de)
     const int sg = hw & (int)0x80000000;
     const int h = z ? sg : (e > 2046 ? sg | 0x7ff00000 : hw + (de << 20));
     return __hiloint2double(h, z || e > 2046 ? 0 : __double2loint(x));
+}
+
+// 2 Xh(f) = s + t and 2 Xh(M - f) = conj(s - t) of packed values a = Z(f),
+// b = Z(M - f) as fixed-point numbers aligned to ex at 2^top (|re|, |im| < 2^top):
+// s = a + conj b, t = w (-i) (a - conj b).
+__device__ __forceinline__ void q_split(cx<double> za, cx<double> zb, qtw w, int ex, int top, cx<q64> &s, cx<q64> &t)
+{
+    const cx<q64> a = {q_decode(za.re, ex, top), q_decode(za.im, ex, top)};
+    const cx<q64> b = {q_decode(zb.re, ex, top), q_decode(zb.im, ex, top)};
+    s = {{a.re.v + b.re.v}, {a.im.v - b.im.v}};
+    t = c_mul(cx<q64>{{a.im.v + b.im.v}, {b.re.v - a.re.v}}, w);
+}
+
+// the high word of a magnitude (nonnegative: orders like the magnitude), and
+// the alignment exponent of a row or column from the largest of them: every
+// magnitude below 63/64 2^(ex - 1022); Q_NONFINITE when an Inf or NaN is among them
+__device__ __forceinline__ unsigned q_magnitude(double x) { return (unsigned)__double2hiint(x) & 0x7fffffffu; }
+__device__ __forceinline__ int q_align(unsigned m)
+{
+    const int ex = max(1, (int)((m + 0x8000u) >> 20));
+    return ex >= 2047 ? Q_NONFINITE : ex;
+}
+
+// The packed spectrum of the pair f, M - f from cf = C(f) / 2, cg = C(M - f) / 2:
+// ZC(f) = s + i p, ZC(M - f) = conj s + i conj p,
+// s = cf + conj cg, p = conj w (cf - conj cg).
+__device__ __forceinline__ void q_merge(cx<double> cf, cx<double> cg, cx<double> w, cx<double> &zf, cx<double> &zg)
+{
+    const double sr = cf.re + cg.re, si = cf.im - cg.im;
+    const double dr = cf.re - cg.re, di = cf.im + cg.im;
+    const double pr = fma(w.re, dr, w.im * di), pi = fma(w.re, di, -(w.im * dr));
+    zf = {sr - pi, si + pr};
+    zg = {sr + pi, pr - si};
 }

@@ -128,3 +128,17 @@ def test_digit_product_non_finite(mrc, bad):
     assert not torch.isfinite(got[:, :, 7]).any()
     keep = [j for j in range(20) if j != 7]
     assert torch.equal(got[:, :, keep], ref[:, :, keep])
+
+
+@pytest.mark.parametrize("d,c", [(1, 1), (2, 7), (5, 3), (24, 3), (40, 2), (56, 1), (78, 1), (80, 5), (20, 130)])
+def test_rectangular_products(mrc, d, c):
+    """V = psi * r with c columns: the fixed-point product (several pairs per
+    CTA, ragged last CTA, one pair of up to 200 KB) and, for spectra that do
+    not fit, the tiles (d = 80); integers, within 1 % of Prop 2.1's bound."""
+    rng = np.random.default_rng(10 * d + c)
+    N = 70
+    X = rng.integers(-8, 9, size=(N, d, d)).astype(np.float64)
+    r = rng.integers(-8, 9, size=(N, d, c)).astype(np.float64)
+    V = mrc.reward(dev(X), dev(r), prec="fp64").cpu().numpy()
+    ref = oracle.convolve(X, r)
+    assert np.sqrt(((V - ref) ** 2).sum()) <= 1e-2 * product_bound(X, r)
