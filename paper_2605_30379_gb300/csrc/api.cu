@@ -1598,13 +1598,12 @@ mrc_status mrc_transition(mrc_ctx *c, int d, int64_t N, const double *psi, const
     mrc_status s;
     if ((s = ensure_tw(c, p, st)) != MRC_OK) return s;
     const size_t E = (size_t)d * d;
-    const int64_t nch = (N + 1023) / 1024;
-    size_t need = align_up(sizeof(double) * N * d) + align_up(sizeof(double) * nch * d) +
+    size_t need = align_up(sizeof(double) * N * d) + align_up(mrc_scan_bytes(N, d)) +
                   ws_product(pow2ceil(N), E, d, E, p);
     if ((s = ensure_ws(c, need)) != MRC_OK) return s;
     Arena ar{(char *)c->ws};
     double *h = (double *)ar.take(sizeof(double) * N * d);
-    double *work = (double *)ar.take(sizeof(double) * nch * d);
+    void *work = ar.take(mrc_scan_bytes(N, d));
     CK(mrc_row_sums(q, h, d, N, st));
     CK(mrc_scan_cols(h, d, N, work, -1.0, 1.0, st));  // Hbar_j(k) = 1 - sum_{l<=k} sum_j' q_jj'(l)
     return conv_product(c, ar, p, psi, N, h, N, d, 1, d, N, P, 1.0, 0, 0, true, st);
@@ -1634,7 +1633,7 @@ mrc_status mrc_first_entrance(mrc_ctx *c, int d, int64_t N, const double *q, con
     if ((s = ensure_tw(c, pc, st)) != MRC_OK) return s;
     const size_t ECC = (size_t)nC * nC, ECD = (size_t)nC * nD;
     size_t fixed = align_up(sizeof(double) * N * ECC) * 2 + align_up(sizeof(double) * N * ECD) * 2 +
-                   align_up(sizeof(double) * N) * 2 + align_up(sizeof(double) * ((N + 1023) / 1024));
+                   align_up(sizeof(double) * N) * 2 + align_up(mrc_scan_bytes(N, 1));
     size_t need = fixed + std::max(ws_inverse(nC, N, prec), ws_product(pow2ceil(N), ECC, ECD, ECD, pc));
     if ((s = ensure_ws(c, need)) != MRC_OK) return s;
     Arena ar{(char *)c->ws};
@@ -1644,7 +1643,7 @@ mrc_status mrc_first_entrance(mrc_ctx *c, int d, int64_t N, const double *q, con
     double *gw = (double *)ar.take(sizeof(double) * N * ECD);
     double *Fw = (double *)ar.take(sizeof(double) * N);
     double *fk = (double *)ar.take(sizeof(double) * N);
-    double *work = (double *)ar.take(sizeof(double) * ((N + 1023) / 1024));
+    void *work = ar.take(mrc_scan_bytes(N, 1));
     CK(mrc_gather_blocks(q, d, N, Ci.data(), nC, Di.data(), nD, ACC, QCD, st));
     const size_t mark = ar.off;
     s = inverse_impl(c, ar, nC, N, ACC, psiC, prec, sweeps, nullptr, st);
@@ -1753,12 +1752,11 @@ mrc_status mrc_renewal_visits(mrc_ctx *c, int d, int64_t N, const double *psi, c
     }
     cudaStream_t st = (cudaStream_t)stream;
     cudaSetDevice(c->device);
-    const int64_t nch = (N + 1023) / 1024;
     mrc_status s;
-    if ((s = ensure_ws(c, align_up(sizeof(double) * nch))) != MRC_OK) return s;
+    if ((s = ensure_ws(c, align_up(mrc_scan_bytes(N, 1)))) != MRC_OK) return s;
     // alpha psi(k) 1_B per k, then the running sum over k (Eq. (renewal-visits))
     CK(mrc_occupation_k(psi, d, N, alpha, inB.data(), out, st));
-    CK(mrc_scan_cols(out, 1, N, (double *)c->ws, 1.0, 0.0, st));
+    CK(mrc_scan_cols(out, 1, N, c->ws, 1.0, 0.0, st));
     return MRC_OK;
 }
 

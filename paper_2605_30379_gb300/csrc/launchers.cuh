@@ -277,6 +277,8 @@ cudaError_t pairdiag_run(const void *zx, const void *zy, void *zc, int64_t M, in
     a.zx = zx; a.zy = zy; a.zc = zc; a.tw = tw; a.tw_log = tw_log; a.M = M; a.logM = ilog2_i64(M);
     a.npairs = M >= 2 ? M / 2 + 1 : 1;
     a.r = r; a.m = 0; a.c = c;
+    if constexpr (std::is_same<T, double>::value) return mrc_pairdiagq(a, kclass_pair<T>(), st);
+    else {
     const int64_t total = a.npairs * (int64_t)r * c;
     int64_t blocks = (total + 255) / 256;
     if (blocks > 152 * 32) blocks = 152 * 32;
@@ -285,6 +287,7 @@ cudaError_t pairdiag_run(const void *zx, const void *zy, void *zc, int64_t M, in
     pairdiag_kernel<T><<<(unsigned)blocks, 256, 0, st>>>(a);
     mrc_prof_post(kclass_pair<T>(), st, bytes, 6.0 * r * c * (double)(M + 1));
     return cudaGetLastError();
+    }
 }
 
 template <class T>

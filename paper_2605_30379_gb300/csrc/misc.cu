@@ -165,47 +165,116 @@ __global__ void row_sums_kernel(const double *__restrict__ q, double *__restrict
     }
 }
 
-constexpr int SCAN_CH = 1024;
+// Inclusive running sums down the rows of x [N][ncol], in three launches: the
+// sum of every chunk of SCAN_CH rows, the running sums of those, and each
+// chunk's rows from its start.  A CTA covers one chunk of up to 32 columns:
+// TX columns x TY threads of SCAN_CH / TY consecutive rows each, so that the
+// loads of a warp are consecutive whatever the column count; one thread per
+// chunk and column took 430 us for N = 2^14, ncol = 32 and 90 us for ncol = 1,
+// in chains of 1024 dependent loads.
+constexpr int SCAN_CH = 256;
 
-__global__ void scan_chunk_sums(const double *__restrict__ x, int ncol, int64_t N, double *__restrict__ work)
+struct ScanShape {
+    int tx, ty, rows;  // columns, row groups, rows per thread of a CTA of 256
+};
+__host__ __device__ inline ScanShape scan_shape(int ncol)
 {
-    const int64_t nch = (N + SCAN_CH - 1) / SCAN_CH;
-    for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < nch * ncol; t += (int64_t)gridDim.x * blockDim.x) {
-        int64_t ch = t / ncol;
-        int c = (int)(t - ch * ncol);
-        int64_t k1 = min(N, (ch + 1) * SCAN_CH);
-        double s = 0.0;
-        for (int64_t k = ch * SCAN_CH; k < k1; ++k) s += x[k * ncol + c];
-        work[t] = s;
+    int tx = 1;
+    while (tx < 32 && tx < ncol) tx <<= 1;
+    return {tx, 256 / tx, SCAN_CH / (256 / tx)};
+}
+
+// Sums as unevaluated pairs h + l (Knuth's TwoSum): the survival function 1 -
+// sum has to vanish in the tail, where the transition function adds its error
+// up over the horizon.
+struct Sum2 {
+    double h, l;
+};
+__device__ __forceinline__ Sum2 sum2(Sum2 a, double b)
+{
+    const double s = a.h + b, t = s - a.h;
+    return {s, a.l + ((a.h - (s - t)) + (b - t))};
+}
+__device__ __forceinline__ Sum2 sum2(Sum2 a, Sum2 b)
+{
+    Sum2 s = sum2(a, b.h);
+    s.l += b.l;
+    return s;
+}
+
+__global__ void __launch_bounds__(256) scan_chunk_sums(const double *__restrict__ x, int ncol, int64_t N,
+                                                       Sum2 *__restrict__ work)
+{
+    __shared__ Sum2 part[256];
+    const ScanShape sh = scan_shape(ncol);
+    const int cx = threadIdx.x % sh.tx, ry = threadIdx.x / sh.tx, c = blockIdx.y * sh.tx + cx;
+    const int64_t k0 = (int64_t)blockIdx.x * SCAN_CH + (int64_t)ry * sh.rows;
+    Sum2 s = {0.0, 0.0};
+    if (c < ncol)
+        for (int k = 0; k < sh.rows; ++k)
+            if (k0 + k < N) s = sum2(s, x[(k0 + k) * ncol + c]);
+    part[threadIdx.x] = s;
+    __syncthreads();
+    for (int o = sh.ty / 2; o > 0; o >>= 1) {
+        if (ry < o) part[threadIdx.x] = sum2(part[threadIdx.x], part[threadIdx.x + o * sh.tx]);
+        __syncthreads();
+    }
+    if (ry == 0 && c < ncol) work[(int64_t)blockIdx.x * ncol + c] = part[threadIdx.x];
+}
+
+// the sums of the row groups before this thread's, per column; part keeps the
+// inclusive sums
+__device__ __forceinline__ Sum2 scan_groups(Sum2 v, Sum2 *part, const ScanShape &sh, int ry)
+{
+    part[threadIdx.x] = v;
+    __syncthreads();
+    for (int o = 1; o < sh.ty; o <<= 1) {
+        const Sum2 w = ry >= o ? part[threadIdx.x - o * sh.tx] : Sum2{0.0, 0.0};
+        __syncthreads();
+        part[threadIdx.x] = sum2(w, part[threadIdx.x]);
+        __syncthreads();
+    }
+    return ry > 0 ? part[threadIdx.x - sh.tx] : Sum2{0.0, 0.0};
+}
+
+// the chunk sums' exclusive running sums (one CTA per column tile)
+__global__ void __launch_bounds__(256) scan_chunk_offsets(Sum2 *work, int ncol, int64_t nch)
+{
+    __shared__ Sum2 part[256];
+    const ScanShape sh = scan_shape(ncol);
+    const int cx = threadIdx.x % sh.tx, ry = threadIdx.x / sh.tx, c = blockIdx.x * sh.tx + cx;
+    Sum2 run = {0.0, 0.0};
+    for (int64_t c0 = 0; c0 < nch; c0 += sh.ty) {
+        const bool in = c < ncol && c0 + ry < nch;
+        const Sum2 before = scan_groups(in ? work[(c0 + ry) * ncol + c] : Sum2{0.0, 0.0}, part, sh, ry);
+        if (in) work[(c0 + ry) * ncol + c] = sum2(run, before);
+        run = sum2(run, part[(sh.ty - 1) * sh.tx + cx]);
+        __syncthreads();
     }
 }
 
-__global__ void scan_chunk_offsets(double *work, int ncol, int64_t nch)
+__global__ void __launch_bounds__(256) scan_apply(double *__restrict__ x, int ncol, int64_t N,
+                                                  const Sum2 *__restrict__ work, double scale, double offset)
 {
-    for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < ncol; c += gridDim.x * blockDim.x) {
-        double run = 0.0;
-        for (int64_t ch = 0; ch < nch; ++ch) {
-            double v = work[ch * ncol + c];
-            work[ch * ncol + c] = run;
-            run += v;
+    __shared__ Sum2 part[256];
+    const ScanShape sh = scan_shape(ncol);
+    const int cx = threadIdx.x % sh.tx, ry = threadIdx.x / sh.tx, c = blockIdx.y * sh.tx + cx;
+    const int64_t k0 = (int64_t)blockIdx.x * SCAN_CH + (int64_t)ry * sh.rows;
+    const bool col = c < ncol;
+    Sum2 s = {0.0, 0.0};
+    if (col)
+        for (int k = 0; k < sh.rows; ++k)
+            if (k0 + k < N) s = sum2(s, x[(k0 + k) * ncol + c]);
+    const Sum2 before = scan_groups(s, part, sh, ry);
+    if (!col) return;
+    Sum2 run = sum2(work[(int64_t)blockIdx.x * ncol + c], before);
+    for (int k = 0; k < sh.rows; ++k)
+        if (k0 + k < N) {
+            run = sum2(run, x[(k0 + k) * ncol + c]);
+            // offset + scale (h + l), scale = +-1
+            const Sum2 y = sum2(Sum2{scale * run.h, scale * run.l}, offset);
+            x[(k0 + k) * ncol + c] = y.h + y.l;
         }
-    }
-}
-
-__global__ void scan_apply(double *__restrict__ x, int ncol, int64_t N, const double *__restrict__ work, double scale,
-                           double offset)
-{
-    const int64_t nch = (N + SCAN_CH - 1) / SCAN_CH;
-    for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < nch * ncol; t += (int64_t)gridDim.x * blockDim.x) {
-        int64_t ch = t / ncol;
-        int c = (int)(t - ch * ncol);
-        int64_t k1 = min(N, (ch + 1) * SCAN_CH);
-        double run = work[t];
-        for (int64_t k = ch * SCAN_CH; k < k1; ++k) {
-            run += x[k * ncol + c];
-            x[k * ncol + c] = offset + scale * run;
-        }
-    }
 }
 
 // acc[0] += sum_k ||rho(k)||_F ; acc[1] = max |rho| (as ordered bits of a nonnegative double)
@@ -258,33 +327,42 @@ __global__ void gather_blocks_kernel(const double *__restrict__ q, int d, int64_
     }
 }
 
-// out[k] = sum_{a,b} alpha[a] g[k][a][b]
-__global__ void weighted_rowsum_kernel(const double *__restrict__ g, int nC, int nD, int64_t N,
-                                       const double *__restrict__ alpha, double *__restrict__ out)
+// out[k] = sum_{i,j} alpha[i] P[k][i][j] over the columns j of B (every column
+// if B is null): one warp per k, consecutive entries across the lanes (one
+// thread per k, striding by a whole matrix, took 117 us at d = 32, N = 2^14
+// where the read takes 20).
+template <bool SET>
+__global__ void __launch_bounds__(256) weighted_sum_kernel(const double *__restrict__ P, int r, int c, int64_t N,
+                                                           const double *__restrict__ alpha, const IdxList B,
+                                                           double *__restrict__ out)
 {
-    for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < N; k += (int64_t)gridDim.x * blockDim.x) {
-        double s = 0.0;
-        for (int a = 0; a < nC; ++a) {
-            double r = 0.0;
-            for (int b = 0; b < nD; ++b) r += g[k * nC * nD + (int64_t)a * nD + b];
-            s = fma(alpha[a], r, s);
-        }
-        out[k] = s;
+    __shared__ double al[512];
+    __shared__ unsigned char in[512];
+    for (int i = threadIdx.x; i < r; i += blockDim.x) al[i] = alpha[i];
+    if (SET) {
+        for (int j = threadIdx.x; j < c; j += blockDim.x) in[j] = 0;
+        __syncthreads();
+        for (int b = threadIdx.x; b < B.n; b += blockDim.x) in[B.idx[b]] = 1;
     }
-}
-
-// out[k] = alpha P(k) 1_B
-__global__ void occupation_kernel(const double *__restrict__ P, int d, int64_t N, const double *__restrict__ alpha,
-                                  IdxList B, double *__restrict__ out)
-{
-    for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < N; k += (int64_t)gridDim.x * blockDim.x) {
+    __syncthreads();
+    const int lane = threadIdx.x & 31, E = r * c;
+    const int di = 32 / c, dj = 32 - di * c;  // a step of 32 entries
+    const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    for (int64_t k = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; k < N; k += nw) {
+        const double *p = P + k * E;
         double s = 0.0;
-        for (int i = 0; i < d; ++i) {
-            double r = 0.0;
-            for (int b = 0; b < B.n; ++b) r += P[k * d * d + (int64_t)i * d + B.idx[b]];
-            s = fma(alpha[i], r, s);
+        int i = lane / c, j = lane - (lane / c) * c;
+        for (int e = lane; e < E; e += 32) {
+            if (!SET || in[j]) s = fma(al[i], p[e], s);
+            i += di;
+            j += dj;
+            if (j >= c) {
+                j -= c;
+                ++i;
+            }
         }
-        out[k] = s;
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+        if (lane == 0) out[k] = s;
     }
 }
 
@@ -452,17 +530,21 @@ cudaError_t mrc_row_sums(const double *q, double *rs, int d, int64_t N, cudaStre
     return cudaGetLastError();
 }
 
-cudaError_t mrc_scan_cols(double *x, int ncol, int64_t N, double *work, double scale, double offset, cudaStream_t st)
+size_t mrc_scan_bytes(int64_t N, int ncol) { return sizeof(Sum2) * (size_t)((N + SCAN_CH - 1) / SCAN_CH) * ncol; }
+
+cudaError_t mrc_scan_cols(double *x, int ncol, int64_t N, void *wk, double scale, double offset, cudaStream_t st)
 {
+    Sum2 *work = (Sum2 *)wk;
     const int64_t nch = (N + SCAN_CH - 1) / SCAN_CH;
     mrc_prof_pre(7, st);
-    scan_chunk_sums<<<grid_for(nch * ncol), 256, 0, st>>>(x, ncol, N, work);
+    const int nt = (ncol + scan_shape(ncol).tx - 1) / scan_shape(ncol).tx;
+    scan_chunk_sums<<<dim3((unsigned)nch, nt), 256, 0, st>>>(x, ncol, N, work);
     mrc_prof_post(7, st, 0, 0);
     mrc_prof_pre(7, st);
-    scan_chunk_offsets<<<grid_for(ncol), 256, 0, st>>>(work, ncol, nch);
+    scan_chunk_offsets<<<nt, 256, 0, st>>>(work, ncol, nch);
     mrc_prof_post(7, st, 0, 0);
     mrc_prof_pre(7, st);
-    scan_apply<<<grid_for(nch * ncol), 256, 0, st>>>(x, ncol, N, work, scale, offset);
+    scan_apply<<<dim3((unsigned)nch, nt), 256, 0, st>>>(x, ncol, N, work, scale, offset);
     mrc_prof_post(7, st, 0, 0);
     return cudaGetLastError();
 }
@@ -495,7 +577,7 @@ cudaError_t mrc_weighted_rowsum(const double *g, int nC, int nD, int64_t N, cons
                                 cudaStream_t st)
 {
     mrc_prof_pre(7, st);
-    weighted_rowsum_kernel<<<grid_for(N), 256, 0, st>>>(g, nC, nD, N, alpha, out);
+    weighted_sum_kernel<false><<<grid_for(N * 32), 256, 0, st>>>(g, nC, nD, N, alpha, IdxList{}, out);
     mrc_prof_post(7, st, 0, 0);
     return cudaGetLastError();
 }
@@ -508,7 +590,7 @@ cudaError_t mrc_occupation_k(const double *P, int d, int64_t N, const double *al
     for (int j = 0; j < d; ++j)
         if (inB[j]) B.idx[B.n++] = j;
     mrc_prof_pre(7, st);
-    occupation_kernel<<<grid_for(N), 256, 0, st>>>(P, d, N, alpha, B, out);
+    weighted_sum_kernel<true><<<grid_for(N * 32), 256, 0, st>>>(P, d, d, N, alpha, B, out);
     mrc_prof_post(7, st, 0, 0);
     return cudaGetLastError();
 }

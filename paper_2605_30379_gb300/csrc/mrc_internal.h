@@ -221,6 +221,8 @@ bool mrc_pairq_supported(int r, int m, int c);
 int mrc_pairq_pp(int64_t npairs, int r, int m, int c);
 cudaError_t mrc_pairq_init(void);
 cudaError_t mrc_pairq(const PairArgs &a, int kclass, cudaStream_t st);
+// C(f)_ij = X(f)_ij Y(f)_j
+cudaError_t mrc_pairdiagq(const PairArgs &a, int kclass, cudaStream_t st);
 // (every segment with its pp and ceil(npairs / pp) CTAs)
 cudaError_t mrc_pairq_seg(const SegParams<PairArgs> &P, unsigned nctas, double bytes, double flops, int kclass,
                           cudaStream_t st);
@@ -273,8 +275,10 @@ int mrc_newton_levels(int prec, int d, int64_t N, const double *A, double *psi, 
 cudaError_t mrc_gauss_jordan(const double *A0, double *out, double *work, int d, int *status, cudaStream_t st);
 cudaError_t mrc_base_case(const double *A, double *psi, int d, int64_t m0, cudaStream_t st);
 cudaError_t mrc_row_sums(const double *q, double *rs, int d, int64_t N, cudaStream_t st);
-cudaError_t mrc_scan_cols(double *x, int ncol, int64_t N, double *work, double scale, double offset,
-                          cudaStream_t st);
+// x(k) <- offset + scale sum_{l <= k} x(l) down the rows (scale = +-1);
+// work: mrc_scan_bytes(N, ncol)
+size_t mrc_scan_bytes(int64_t N, int ncol);
+cudaError_t mrc_scan_cols(double *x, int ncol, int64_t N, void *work, double scale, double offset, cudaStream_t st);
 cudaError_t mrc_norms(const double *rho, int E, int64_t N, double *acc, cudaStream_t st);
 cudaError_t mrc_gather_blocks(const double *q, int d, int64_t N, const int *Cidx, int nC, const int *Didx,
                               int nD, double *ACC, double *QCD, cudaStream_t st);

@@ -36,22 +36,12 @@ constexpr int NT = 128;
 __device__ __forceinline__ int top_for(int m) { return m <= 4 ? 58 : (m <= 31 ? 57 : 56); }
 constexpr int SMEM_MAX = 200 * 1024;
 
-struct __align__(16) limbs {
-    int rh, rl, ih, il;
-};
-
-__device__ __forceinline__ limbs to_limbs(long long re, long long im)
-{
-    const int rl = (int)((unsigned)re << 2) >> 2, il = (int)((unsigned)im << 2) >> 2;
-    return {(int)((re - rl) >> 30), rl, (int)((im - il) >> 30), il};
-}
-
 // accumulators of one complex sum: 2^60 h + 2^30 m + l
 struct acc {
     long long hr, hi, mr, mi, lr, li;
 };
 
-__device__ __forceinline__ void mac(acc &a, const limbs &x, const limbs &y)
+__device__ __forceinline__ void mac(acc &a, const qtw &x, const qtw &y)
 {
     const int nh = -x.ih, nl = -x.il;
     a.hr = q_wide(nh, y.ih, q_wide(x.rh, y.rh, a.hr));
@@ -76,7 +66,7 @@ __device__ __forceinline__ void fold(acc &a)
 
 size_t pair_bytes(int r, int m, int c)
 {
-    return 2 * sizeof(limbs) * ((size_t)r * m + (size_t)m * c) + sizeof(qtw) + sizeof(int) * ((size_t)r + c);
+    return 2 * sizeof(qtw) * ((size_t)r * m + (size_t)m * c) + sizeof(qtw) + sizeof(int) * ((size_t)r + c);
 }
 
 __device__ __forceinline__ void pairq_body(const PairArgs &a, int64_t p0)
@@ -84,7 +74,7 @@ __device__ __forceinline__ void pairq_body(const PairArgs &a, int64_t p0)
     extern __shared__ __align__(16) unsigned char smem[];
     const int r = a.r, m = a.m, c = a.c, EX = r * m, EY = m * c, EC = r * c, ex2 = EX + EY;
     const int np = (int)min((int64_t)a.pp, a.npairs - p0);
-    limbs *sf = reinterpret_cast<limbs *>(smem), *sg = sf + a.pp * ex2;  // per pair: X then Y entries, f and g
+    qtw *sf = reinterpret_cast<qtw *>(smem), *sg = sf + a.pp * ex2;  // per pair: X then Y entries, f and g
     qtw *stw = reinterpret_cast<qtw *>(sg + a.pp * ex2);
     unsigned *bnd = reinterpret_cast<unsigned *>(stw + a.pp);            // per pair: r row and c column bounds
     const cx<double> *ZX = reinterpret_cast<const cx<double> *>(a.zx), *ZY = reinterpret_cast<const cx<double> *>(a.zy);
@@ -118,8 +108,8 @@ __device__ __forceinline__ void pairq_body(const PairArgs &a, int64_t p0)
         cx<q64> s, u;
         q_split(reinterpret_cast<cx<double> *>(sf)[t], reinterpret_cast<cx<double> *>(sg)[t], stw[q],
                 q_align(bnd[q * (r + c) + (x ? ee / m : r + ee % c)]), top, s, u);
-        sf[t] = to_limbs(s.re.v + u.re.v, s.im.v + u.im.v);
-        sg[t] = to_limbs(s.re.v - u.re.v, u.im.v - s.im.v);
+        sf[t] = q_limbs(c_add(s, u));
+        sg[t] = q_limbs({{s.re.v - u.re.v}, {u.im.v - s.im.v}});
     }
     __syncthreads();
     for (int t = tid; t < np * EC; t += NT) {
@@ -146,6 +136,68 @@ __device__ __forceinline__ void pairq_body(const PairArgs &a, int64_t p0)
         q_merge(cf, cg, tw[f << tws], zf, zg);
         ZC[f * EC + e] = zf;
         if (g != f) ZC[g * EC + e] = zg;
+    }
+}
+
+// Product with a diagonal right factor, C(f)_ij = X(f)_ij Y(f)_j: a complex
+// product per entry, with each pair of packed values aligned by itself and
+// merged in fixed point.  The 56 FP64 operations per pair of entries were what
+// bound it (1.1 ms at d = 32, M = 2^14, where its bytes take 0.08 ms).  CTA:
+// the pairs p0 .. p0 + pp - 1; Y's factors once per column.
+__global__ void __launch_bounds__(NT) pairdiagq_kernel(const PairArgs a)
+{
+    extern __shared__ __align__(16) unsigned char smem[];
+    const int r = a.r, c = a.c, E = r * c;
+    const int64_t p0 = (int64_t)blockIdx.x * a.pp, M = a.M;
+    const int np = (int)min((int64_t)a.pp, a.npairs - p0), tws = a.tw_log - a.logM - 1, tid = threadIdx.x;
+    qtw *yf = reinterpret_cast<qtw *>(smem), *yg = yf + a.pp * c, *stw = yg + a.pp * c;
+    int *yex = reinterpret_cast<int *>(stw + a.pp);
+    const cx<double> *ZX = reinterpret_cast<const cx<double> *>(a.zx), *ZY = reinterpret_cast<const cx<double> *>(a.zy);
+    cx<double> *ZC = reinterpret_cast<cx<double> *>(a.zc);
+    const cx<double> *tw = reinterpret_cast<const cx<double> *>(a.tw);
+    auto align = [](cx<double> za, cx<double> zb) {
+        return q_align(max(max(q_magnitude(za.re), q_magnitude(za.im)), max(q_magnitude(zb.re), q_magnitude(zb.im))));
+    };
+    // 2 Xh(f) and 2 Xh(M - f), moduli below 2^60
+    auto split = [](cx<double> za, cx<double> zb, qtw w, int ex, cx<q64> &xf, cx<q64> &xg) {
+        cx<q64> s, t;
+        q_split(za, zb, w, ex, Q_TOP - 2, s, t);
+        xf = c_add(s, t);
+        xg = {{s.re.v - t.re.v}, {t.im.v - s.im.v}};
+    };
+    for (int t = tid; t < np * c; t += NT) {
+        const int q = t / c, j = t - q * c;
+        const int64_t f = p0 + q, g = (M - f) & (M - 1);
+        const qtw w = q_twiddle(tw[f << tws], 0, false);
+        if (j == 0) stw[q] = q_twiddle(c_conj(tw[f << tws]), 0, false);
+        const cx<double> za = ZY[f * c + j], zb = ZY[g * c + j];
+        const int ex = align(za, zb);
+        cx<q64> vf, vg;
+        split(za, zb, w, ex, vf, vg);
+        yf[t] = q_limbs(vf);
+        yg[t] = q_limbs(vg);
+        yex[t] = ex;
+    }
+    __syncthreads();
+    for (int t = tid; t < np * E; t += NT) {
+        const int q = t / E, e = t - q * E, j = e % c;
+        const int64_t f = p0 + q, g = (M - f) & (M - 1);
+        const cx<double> za = ZX[f * E + e], zb = ZX[g * E + e];
+        const int ex = align(za, zb), ey = yex[q * c + j];
+        const qtw wc = stw[q];  // conj w
+        cx<q64> xf, xg;
+        split(za, zb, qtw{wc.rh, wc.rl, -wc.ih, -wc.il}, ex, xf, xg);
+        const cx<q64> cf = c_mul(xf, yf[q * c + j]), cg = c_mul(xg, yg[q * c + j]);
+        // s = cf + conj cg, p = conj w (cf - conj cg); ZC(f) = s + i p, ZC(M - f) = conj s + i conj p
+        const cx<q64> s = {{cf.re.v + cg.re.v}, {cf.im.v - cg.im.v}};
+        const cx<q64> p = c_mul(cx<q64>{{cf.re.v - cg.re.v}, {cf.im.v + cg.im.v}}, wc);
+        // cf = 4 C(f) 2^(2 1080 - 60 - ex - ey); the merge halves
+        const int eb = ex + ey - 2 * (Q_TOP - 2 + 1022) + Q_TOP - 3 + 1086;
+        cx<double> zf = {q_encode({s.re.v - p.im.v}, eb, 0u), q_encode({s.im.v + p.re.v}, eb, 0u)};
+        cx<double> zg = {q_encode({s.re.v + p.im.v}, eb, 0u), q_encode({p.re.v - s.im.v}, eb, 0u)};
+        if (max(ex, ey) >= Q_NONFINITE) zf.re = zf.im = zg.re = zg.im = __longlong_as_double(0x7ff8000000000000ll);
+        ZC[f * E + e] = zf;
+        if (g != f) ZC[g * E + e] = zg;
     }
 }
 
@@ -186,6 +238,18 @@ cudaError_t mrc_pairq(const PairArgs &a0, int kclass, cudaStream_t st)
     mrc_prof_pre(kclass, st);
     pairq_kernel<<<(unsigned)((a.npairs + a.pp - 1) / a.pp), NT, a.pp * pair_bytes(a.r, a.m, a.c), st>>>(a);
     mrc_prof_post(kclass, st, by, 8.0 * a.r * a.m * a.c * (double)(a.M + 1));
+    return cudaGetLastError();
+}
+
+cudaError_t mrc_pairdiagq(const PairArgs &a0, int kclass, cudaStream_t st)
+{
+    PairArgs a = a0;
+    const int64_t fill = std::max(1, 2 * NT / (a.r * a.c)), spread = std::max<int64_t>(1, a.npairs / 304);
+    a.pp = (int)std::min(fill, spread);
+    const size_t sm = a.pp * (2 * sizeof(qtw) * a.c + sizeof(qtw) + sizeof(int) * a.c);
+    mrc_prof_pre(kclass, st);
+    pairdiagq_kernel<<<(unsigned)((a.npairs + a.pp - 1) / a.pp), NT, sm, st>>>(a);
+    mrc_prof_post(kclass, st, (double)a.M * (2.0 * a.r * a.c + a.c) * 16.0, 6.0 * a.r * a.c * (double)(a.M + 1));
     return cudaGetLastError();
 }
 

@@ -156,12 +156,18 @@ __device__ __forceinline__ unsigned q_bits(q64 a)
     return (unsigned)(h ^ (h >> 31));
 }
 
+// limbs with balanced 30-bit low parts
+__device__ __forceinline__ qtw q_limbs(cx<q64> v)
+{
+    const int rl = (int)((unsigned)v.re.v << 2) >> 2, il = (int)((unsigned)v.im.v << 2) >> 2;
+    return {(int)((v.re.v - rl) >> 30), rl, (int)((v.im.v - il) >> 30), il};
+}
+
 // the limbs of w / 2^s (conjugated if conj)
 __device__ __forceinline__ qtw q_twiddle(cx<double> w, int s, bool conj)
 {
     const long long r = q_decode(w.re, 1022 + s, Q_TOP).v, i = q_decode(w.im, 1022 + s, Q_TOP, conj ? -1 : 0).v;
-    const int rl = (int)(r << 2) >> 2, il = (int)(i << 2) >> 2;  // balanced 30-bit low limbs
-    return {(int)((r - rl) >> 30), rl, (int)((i - il) >> 30), il};
+    return q_limbs({{r}, {i}});
 }
 
 // (U : rest) with U < 2^63 and 32 bits of rest, rounded to a double: leading bit

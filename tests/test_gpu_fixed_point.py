@@ -142,3 +142,38 @@ def test_rectangular_products(mrc, d, c):
     V = mrc.reward(dev(X), dev(r), prec="fp64").cpu().numpy()
     ref = oracle.convolve(X, r)
     assert np.sqrt(((V - ref) ** 2).sum()) <= 1e-2 * product_bound(X, r)
+
+
+@pytest.mark.parametrize("d,N", [(2, 1), (3, 255), (31, 256), (32, 257), (33, 700), (7, 70000)])
+def test_functionals_sizes(mrc, d, N):
+    """Running sums over one, full, ragged and many chunks and 1 to 33 columns,
+    weighted sums of matrices narrower and wider than a warp, and the diagonal
+    product: visits, occupation and transition against numpy sums (transition:
+    rows add up to one for psi = the inverse, checked on the horizon the
+    oracle reaches)."""
+    rng = np.random.default_rng(d)
+    psi, alpha = rng.uniform(0, 1, (N, d, d)), rng.uniform(0, 1, d)
+    B = sorted(rng.choice(d, max(1, d // 2), replace=False).tolist())
+    occ = np.einsum("i,kij->k", alpha, psi[:, :, B])
+    got = mrc.occupation(dev(psi), torch.tensor(alpha), B).cpu().numpy()
+    assert np.abs(got - occ).max() <= 1e-15 * d * d
+    vis = mrc.renewal_visits(dev(psi), torch.tensor(alpha), B).cpu().numpy()
+    ref = np.cumsum(occ.astype(np.longdouble)).astype(float)
+    assert np.abs(vis - ref).max() <= 1e-15 * (d * d + np.log2(N + 1)) * max(1.0, ref.max())
+    n = min(N, 1500)
+    q, _ = synth.weibull_model(d, n, seed=d)
+    x = oracle.inverse_left(synth.identity_minus(q))
+    P = mrc.transition(dev(x), dev(q), prec="fp64").cpu().numpy()
+    assert np.abs(P - oracle.transition(x, q)).max() <= 1e-13
+    assert np.abs(P.sum(axis=2) - 1.0).max() <= 1e-12
+
+
+def test_diagonal_product_non_finite(mrc):
+    q, _ = synth.weibull_model(5, 40, seed=1)
+    psi = torch.rand(40, 5, 5, dtype=torch.float64, device="cuda")
+    ref = mrc.transition(psi, dev(q))
+    psi[3, 2, 1] = float("inf")
+    got = mrc.transition(psi, dev(q))
+    assert not torch.isfinite(got[:, 2, 1]).any()
+    got[:, 2, 1] = ref[:, 2, 1]
+    assert torch.equal(got, ref)
