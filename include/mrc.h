@@ -71,7 +71,7 @@ typedef struct {
     double res_left_l1;   /* sum_k ||rho_L(k)||_F over k < N (Frobenius form of ||.||_{1,N}) */
     double res_right_l1;  /* same for rho_R, when computed; else -1 */
     double res_max_abs;   /* max_{k,i,j} |rho_L(k)_{ij}| (or of rho_R when only R was asked) */
-    int levels;           /* Newton doubling levels run */
+    int levels;           /* Newton doubling levels run (beyond the first 32, 8 or 2 coefficients for d <= 8, d <= 32, above) */
     int sweeps;           /* refinement sweeps run */
     double ms;            /* device time of the call (CUDA events) */
 } mrc_report;
@@ -300,7 +300,7 @@ mrc_status mrc_renewal_visits(mrc_ctx *ctx, int d, int64_t N, const double *psi,
  * agree with mrc_inverse's to rounding.
  *   d, N, A, psi, stream : as mrc_inverse with prec = MRC_FP64.
  * Scratch: one fixed 64 MiB device array inside the library.  The call uses
- * 256 B + 512 KiB (twiddles) + 16 d^2 + 4 * 16 d^2 * M bytes of it, M being
+ * 256 B + 512 KiB (twiddles) + 4 * 16 d^2 * M bytes of it, M being
  * the largest Newton level (< N); N must be <= 2^14.  Larger requests return
  * MRC_ERR_NO_MEMORY at once, with the limit printed to stderr.
  * No cudaMalloc/cudaFree or allocating library routine is called.

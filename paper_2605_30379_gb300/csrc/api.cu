@@ -153,15 +153,16 @@ mrc_status ensure_ws(mrc_ctx *c, size_t need)
 
 // ---------------------------------------------------------------------------
 // Workspace plans
-int64_t base_size(int d, int64_t N) { return mrc_base_size(d, N); }
-int64_t newton_maxM(int d, int64_t N) { return mrc_newton_maxM(d, N); }
+// (of the Newton levels' working precision: FP64 or FP32)
+int64_t base_size(int d, int64_t N, int prec) { return mrc_base_size(d, N, prec == PREC_F32); }
+int64_t newton_maxM(int d, int64_t N, int prec) { return mrc_newton_maxM(d, N, prec == PREC_F32); }
+int level_prec(int prec) { return prec == MRC_FP64 ? PREC_F64 : PREC_F32; }
 
 size_t ws_newton(int d, int64_t N, int prec)
 {
     const size_t E = (size_t)d * d;
-    size_t b = align_up(sizeof(double) * 2 * E);  // Gauss-Jordan work
-    const int64_t M = newton_maxM(d, N);
-    b += 3 * align_up((size_t)M * E * OPS[prec].cxb) + align_up(mrc_fft_scratch_elems(M, (int)E) * OPS[prec].cxb);
+    const int64_t M = newton_maxM(d, N, prec);
+    size_t b = 3 * align_up((size_t)M * E * OPS[prec].cxb) + align_up(mrc_fft_scratch_elems(M, (int)E) * OPS[prec].cxb);
     return b;
 }
 
@@ -173,7 +174,7 @@ size_t ws_product(int64_t Mr, size_t EX, size_t EY, size_t EC, int prec)
            align_up(mrc_fft_scratch_elems(Mr, (int)emax) * cxb);
 }
 
-// Mixed inverse layout: [Gauss-Jordan work | double-float spectrum of A |
+// Mixed inverse layout: [double-float spectrum of A |
 // its FFT scratch | psi_0 in binary32 | then either A in binary32 and the
 // FP32 Newton buffers or, afterwards, rho_L (binary32) followed by the
 // residual's two other double-float spectra or the FP32 correction's
@@ -187,12 +188,11 @@ size_t ws_inverse(int d, int64_t N, int prec)
     const size_t E = (size_t)d * d;
     if (prec == MRC_FP64) return ws_newton(d, N, PREC_F64);
     const int64_t Mr = pow2ceil(N);
-    const size_t gj = align_up(sizeof(double) * 2 * E);
     const size_t ahat = align_up((size_t)Mr * E * 16) + align_up(mrc_fft_scratch_elems(Mr, (int)E) * 16);
     // psi_0 in binary32 (the FP32 Newton levels' output), kept to the end
     const size_t psi32 = align_up((size_t)N * E * sizeof(float));
     // the FP32 Newton levels: their binary32 copy of A and their buffers
-    const size_t newton = align_up((size_t)N * E * sizeof(float)) + ws_newton(d, N, PREC_F32) - gj;
+    const size_t newton = align_up((size_t)N * E * sizeof(float)) + ws_newton(d, N, PREC_F32);
     // rho_L (binary32), the FP32 spectrum of psi_0 (hi parts of its
     // double-float one), then the residual's spectra of psi_0 and of the
     // product (double-float) or the correction's FP32 spectrum of rho,
@@ -202,7 +202,7 @@ size_t ws_inverse(int d, int64_t N, int prec)
                                    2 * align_up((size_t)Mr * E * 8) + align_up(mrc_fft_scratch_elems(Mr, (int)E) * 8));
     // the residual product's prepared X (digit tiles and scales of A's spectrum)
     const size_t xpre = xpre_used(d) ? align_up(mrc_tcp_prep_bytes(Mr, d)) + align_up(mrc_tcp_prep_scale_bytes(Mr)) : 0;
-    return gj + ahat + xpre + psi32 + std::max(newton, refine);
+    return ahat + xpre + psi32 + std::max(newton, refine);
 }
 
 // Product kernel choices: 0..2 and 4 the FP32-pipe tile configurations
@@ -430,13 +430,12 @@ cudaError_t level_product(void *user, int prec, const void *zx, const void *zy, 
 // Newton doubling levels in working precision `prec` over buffers taken
 // from the context workspace (the schedule itself is mrc_newton_levels).
 mrc_status newton_levels(mrc_ctx *c, Arena &ar, int prec, int d, int64_t N, const double *A, double *psi,
-                         int64_t m0, int *levels, cudaStream_t st, const RowWait *rw = nullptr,
+                         int64_t m0, cudaStream_t st, const RowWait *rw = nullptr,
                          float *A32 = nullptr, float *psi32 = nullptr, int64_t a32_rows = 0)
 {
     const PrecOps &op = OPS[prec];
     const int E = d * d;
-    const int64_t Mmax = newton_maxM(d, N);
-    if (levels) *levels = 0;
+    const int64_t Mmax = newton_maxM(d, N, prec);
     if (Mmax == 0) return MRC_OK;
     NewtonBufs b;
     b.b0 = ar.take((size_t)Mmax * E * op.cxb);
@@ -444,10 +443,35 @@ mrc_status newton_levels(mrc_ctx *c, Arena &ar, int prec, int d, int64_t N, cons
     b.b2 = ar.take((size_t)Mmax * E * op.cxb);
     b.bt = ar.take(mrc_fft_scratch_elems(Mmax, E) * op.cxb);
     return (mrc_status)mrc_newton_levels(prec, d, N, A, psi, m0, b, c->tw[prec], MRC_TW_LOG, level_fft,
-                                         level_product, c, st, rw, A32, psi32, levels, a32_rows);
+                                         level_product, c, st, rw, A32, psi32, a32_rows);
 }
 
 bool valid_dN(int d, int64_t N) { return d >= 1 && d <= 512 && N >= 1 && N <= ((int64_t)1 << 20); }
+
+// mrc_report::levels: the doublings beyond the first 32 (d <= 8), 8 (d <= 32) or
+// 2 coefficients, whether by FFT or by direct sums
+int report_levels(int d, int64_t N)
+{
+    int lv = 0;
+    for (int64_t m = d <= 8 ? 32 : (d <= 32 ? 8 : 2); m < N; m <<= 1) ++lv;
+    return lv;
+}
+
+// psi(0 .. m0-1) on `st` (and its binary32 copy); launched before the mixed
+// path's side stream gets its first kernel: a cluster of 16 CTAs waits for SMs
+// while another kernel still has CTAs to place
+mrc_status seed_one(mrc_ctx *c, int d, const double *A, double *psi, int64_t m0, int *status, float *psi32,
+                    const RowWait *rw, cudaStream_t st)
+{
+    if (rw) CK(rw->wait(st, m0));
+    auto P = std::make_unique<SegParams<SeedArgs>>();
+    P->nseg = 1;
+    P->a[0] = SeedArgs{A, psi, d, (int)m0, status ? status : c->d_status};
+    CK(mrc_seed(*P, st));
+    if (d > MRC_SEED_DMAX) CK(mrc_base_case(A, psi, d, m0, st));
+    if (psi32) CK(mrc_f64_to_f32(psi, psi32, m0 * (int64_t)d * d, st));
+    return MRC_OK;
+}
 
 // Mixed precision: the double-float spectrum of A that every residual sweep
 // uses, and the residual product's prepared X, depend on A alone.  With
@@ -460,7 +484,7 @@ bool valid_dN(int d, int64_t N) { return d >= 1 && d <= 512 && N >= 1 && N <= ((
 // `st` waits for both before the first residual.  Without `split` everything
 // runs on `st`.
 mrc_status inverse_impl(mrc_ctx *c, Arena &ar, int d, int64_t N, const double *A, double *psi, int prec, int sweeps,
-                        int *levels, cudaStream_t st, int *status = nullptr, bool split = false,
+                        cudaStream_t st, int *status = nullptr, bool split = false,
                         const RowWait *rw = nullptr)
 {
     const size_t E = (size_t)d * d;
@@ -470,11 +494,12 @@ mrc_status inverse_impl(mrc_ctx *c, Arena &ar, int d, int64_t N, const double *A
         ~StatusScope() { c->cur_status = old; }
     } sscope{c, c->cur_status};
     c->cur_status = status ? status : c->d_status;
-    double *gjw = (double *)ar.take(sizeof(double) * 2 * E);
     void *ahat = nullptr, *ascr = nullptr, *xpt = nullptr, *xps = nullptr;
     float *psi32 = nullptr, *A32 = nullptr;
     size_t mark = 0;
     int64_t a32_rows = 0;
+    const int64_t m0 = base_size(d, N, level_prec(prec));
+    mrc_status s;
     cudaStream_t sn = st;  // Newton levels
     if (prec == MRC_MIXED) {
         const int64_t Mr = pow2ceil(N);
@@ -504,6 +529,7 @@ mrc_status inverse_impl(mrc_ctx *c, Arena &ar, int d, int64_t N, const double *A
             sa = c->aux;
             sn = c->lvl;
         }
+        if ((s = seed_one(c, d, A, psi, m0, status, psi32, rw, sn)) != MRC_OK) return s;
         if (rw) CK(rw->wait(sa, N));
         FftSrc sx{SRC_REAL64, A, 0, N, (int)E, 0};
         FftDst dx{DST_CPLX, ahat, (int)E, 0, 0, 0, 1.0, 0};
@@ -517,14 +543,11 @@ mrc_status inverse_impl(mrc_ctx *c, Arena &ar, int d, int64_t N, const double *A
         }
         if (split) CK(cudaEventRecord(c->ev_join, c->aux));
     }
-    const int64_t m0 = base_size(d, N);
-    if (rw) CK(rw->wait(sn, m0));
-    CK(mrc_gauss_jordan(A, psi, gjw, d, status ? status : c->d_status, sn));
-    CK(mrc_base_case(A, psi, d, m0, sn));
-    if (psi32) CK(mrc_f64_to_f32(psi, psi32, m0 * (int64_t)E, sn));
-    if (!psi32) mark = ar.off;
-    mrc_status s = newton_levels(c, ar, prec == MRC_FP64 ? PREC_F64 : PREC_F32, d, N, A, psi, m0, levels, sn, rw,
-                                 A32, psi32, a32_rows);
+    if (!psi32) {
+        if ((s = seed_one(c, d, A, psi, m0, status, nullptr, rw, st)) != MRC_OK) return s;
+        mark = ar.off;
+    }
+    s = newton_levels(c, ar, prec == MRC_FP64 ? PREC_F64 : PREC_F32, d, N, A, psi, m0, sn, rw, A32, psi32, a32_rows);
     if (s != MRC_OK) return s;
     ar.off = mark;
     if (prec == MRC_MIXED) {
@@ -598,7 +621,7 @@ mrc_status gj_series_impl(mrc_ctx *c, Arena &ar, int d, int64_t N, const double 
         CK(mrc_gjs_pivot(A, W, d, N, col, flags, u, cv, flags + 1, c->cur_status, st));
         // v = u^(-1) mod x^N (scalar Newton; its own workspace above this call's)
         const size_t mark = ar.off;
-        mrc_status s = inverse_impl(c, ar, 1, N, u, v, MRC_FP64, 0, nullptr, st);
+        mrc_status s = inverse_impl(c, ar, 1, N, u, v, MRC_FP64, 0, st);
         if (s != MRC_OK) return s;
         ar.off = mark;
         // normalise: row <- v * row mod x^N
@@ -699,7 +722,7 @@ void pretune_model(mrc_ctx *cx, int prec, int d, int64_t N, char *buf, size_t by
         tuned_choice(cx, p, buf, buf + sz, buf + 2 * sz, M, d, d, d, cx->tw[p], st);
     };
     const int pl = prec == MRC_FP64 ? PREC_F64 : PREC_F32;
-    for (int64_t m = base_size(d, N); m < N; m <<= 1) one(pl, m);
+    for (int64_t m = base_size(d, N, pl); m < N; m <<= 1) one(pl, m);
     if (prec == MRC_MIXED) {
         one(PREC_DD, pow2ceil(N));
         one(PREC_F32, pow2ceil(N));
@@ -760,7 +783,6 @@ struct BModel {
     int *status = nullptr;
     double cost = 0;
     size_t ws = 0;
-    double *gjw = nullptr;
     float *A32 = nullptr, *psi32 = nullptr, *rho32 = nullptr;
     void *b0 = nullptr, *b1 = nullptr, *b2 = nullptr, *bt = nullptr;  // Newton level spectra and scratch
     void *ahat = nullptr, *ascr = nullptr;                              // double-float spectrum of A, scratch
@@ -774,7 +796,6 @@ void bmodel_layout(BModel &m, int prec, char *base)
 {
     const size_t E = (size_t)m.E, Mr = (size_t)m.Mr, Mm = (size_t)m.Mmax, N = (size_t)m.N;
     Arena ar{base};
-    m.gjw = (double *)ar.take(sizeof(double) * 2 * E);
     if (prec == MRC_FP64) {
         m.b0 = ar.take(Mm * E * 16);
         m.b1 = ar.take(Mm * E * 16);
@@ -944,20 +965,20 @@ mrc_status batch_wave(mrc_ctx *c, std::vector<BModel> &W, int prec, int sweeps, 
         if (m.m0 < m.N) mmin = std::min(mmin, m.m0);
         nmax = std::max(nmax, m.N);
     }
-    // psi(0) = A(0)^(-1) and the direct recursion for psi(1 .. m0-1)
+    // psi(0 .. m0-1)
     {
-        auto G = std::make_unique<SegParams<GjArgs>>();
+        auto G = std::make_unique<SegParams<SeedArgs>>();
         auto B = std::make_unique<SegParams<BaseArgs>>();
         for (size_t i0 = 0; i0 < n; i0 += MRC_SEG_MAX) {
             const size_t i1 = std::min(n, i0 + (size_t)MRC_SEG_MAX);
             G->nseg = B->nseg = (int)(i1 - i0);
             for (size_t i = i0; i < i1; ++i) {
                 G->first[i - i0] = B->first[i - i0] = (unsigned)(i - i0);
-                G->a[i - i0] = GjArgs{W[i].A, W[i].psi, W[i].gjw, W[i].d, W[i].status};
-                B->a[i - i0] = BaseArgs{W[i].A, W[i].psi, W[i].d, (int)W[i].m0};
+                G->a[i - i0] = SeedArgs{W[i].A, W[i].psi, W[i].d, (int)W[i].m0, W[i].status};
+                B->a[i - i0] = BaseArgs{W[i].A, W[i].psi, W[i].d, W[i].d > MRC_SEED_DMAX ? (int)W[i].m0 : 0};
             }
-            CK(mrc_gauss_jordan_batch(*G, dmax, st));
-            CK(mrc_base_case_batch(*B, dmax, st));
+            CK(mrc_seed(*G, st));
+            if (dmax > MRC_SEED_DMAX) CK(mrc_base_case_batch(*B, dmax, st));
         }
     }
     if (f32) {
@@ -1095,15 +1116,9 @@ mrc_status batch_wave(mrc_ctx *c, std::vector<BModel> &W, int prec, int sweeps, 
 
 // ===========================================================================
 // The Newton schedule shared by the inverse entry points.
-int64_t mrc_base_size(int d, int64_t N)
+int64_t mrc_newton_maxM(int d, int64_t N, bool f32)
 {
-    int64_t m0 = d <= 8 ? 32 : (d <= 32 ? 8 : 2);
-    return std::min<int64_t>(m0, N);
-}
-
-int64_t mrc_newton_maxM(int d, int64_t N)
-{
-    int64_t m0 = mrc_base_size(d, N), M = 0;
+    int64_t m0 = mrc_base_size(d, N, f32), M = 0;
     for (int64_t m = m0; m < N; m <<= 1) M = m;
     return M;
 }
@@ -1112,13 +1127,12 @@ int64_t mrc_newton_maxM(int d, int64_t N)
 // (L = 2m): E = A*B (cyclic), R = -E[m, 2m), B[m, 2m) = (B*R)[0, m).
 int mrc_newton_levels(int prec, int d, int64_t N, const double *A, double *psi, int64_t m0, const NewtonBufs &b,
                       const void *tw, int tw_log, mrc_level_fft_fn fft, mrc_level_product_fn product, void *user,
-                      cudaStream_t st, const RowWait *rw, float *A32, float *psi32, int *levels, int64_t a32_rows)
+                      cudaStream_t st, const RowWait *rw, float *A32, float *psi32, int64_t a32_rows)
 {
     const int E = d * d;
     const bool f32 = A32 && psi32;
     int64_t conv = a32_rows;  // rows of A32 converted so far
-    int lv = 0;
-    for (int64_t m = m0; m < N; m <<= 1, ++lv) {
+    for (int64_t m = m0; m < N; m <<= 1) {
         const int64_t M = m, m2 = std::min<int64_t>(2 * m, N);
         if (rw) CK(rw->wait(st, m2));  // this level reads A[0, 2m)
         if (f32 && conv < m2) {
@@ -1143,7 +1157,6 @@ int mrc_newton_levels(int prec, int d, int64_t N, const double *A, double *psi, 
         FftDst toP{f32 ? DST_REAL32 : DST_REAL64, f32 ? (void *)psi32 : psi, E, 0, m2 - m, m, 1.0 / (double)M, 0};
         CK(fft(user, prec, s0, toP, M, E, +1, b.bt, tw, tw_log, st));        // B[m, m2)
     }
-    if (levels) *levels = lv;
     return MRC_OK;
 }
 
@@ -1188,7 +1201,7 @@ mrc_status mrc_create(mrc_ctx **out, int device, size_t max_workspace_bytes)
     if (cudaSetDevice(device) != cudaSuccess) return MRC_ERR_CUDA;
     for (int p = 0; p < 3; ++p)
         if (OPS[p].init() != cudaSuccess) return MRC_ERR_CUDA;
-    if (mrc_tc_init() != cudaSuccess || mrc_tcp_init() != cudaSuccess) return MRC_ERR_CUDA;
+    if (mrc_tc_init() != cudaSuccess || mrc_tcp_init() != cudaSuccess || mrc_seed_init() != cudaSuccess) return MRC_ERR_CUDA;
     mrc_ctx *c = new mrc_ctx();
     c->device = device;
     c->cap = max_workspace_bytes;
@@ -1270,16 +1283,15 @@ mrc_status mrc_inverse(mrc_ctx *c, int d, int64_t N, const double *A, double *ps
     if (check) need = std::max(need, ws_residual(d, N, MRC_MIXED, true));
     if ((s = ensure_ws(c, need)) != MRC_OK) return s;
     Arena ar{(char *)c->ws};
-    int levels = 0;
     if (report) CK(cudaEventRecord(c->ev0, st));
     if (prec == MRC_MIXED && (s = ensure_split_streams(c)) != MRC_OK) return s;
-    s = inverse_impl(c, ar, d, N, A, psi, prec, sweeps, &levels, st, nullptr, prec == MRC_MIXED);
+    s = inverse_impl(c, ar, d, N, A, psi, prec, sweeps, st, nullptr, prec == MRC_MIXED);
     if (s != MRC_OK) return s;
     if (report) {
         CK(cudaEventRecord(c->ev1, st));
         memset(report, 0, sizeof(*report));
         report->res_left_l1 = report->res_right_l1 = report->res_max_abs = -1.0;
-        report->levels = levels;
+        report->levels = report_levels(d, N);
         report->sweeps = prec == MRC_MIXED ? sweeps : 0;
         s = read_status(c, st);
         float ms = 0.f;
@@ -1357,7 +1369,7 @@ mrc_status mrc_inverse_host(mrc_ctx *c, int d, int64_t N, const double *A_host, 
     CK(cudaEventRecord(c->ev_cpy_fork, st));  // earlier work on st may still use the workspace
     CK(cudaStreamWaitEvent(c->cpy, c->ev_cpy_fork, 0));
     RowWait rw;
-    int64_t r0 = 0, r1 = std::min<int64_t>(2 * base_size(d, N), N);
+    int64_t r0 = 0, r1 = std::min<int64_t>(2 * base_size(d, N, level_prec(prec)), N);
     while (r0 < N && rw.n < 32) {
         if (rw.n == 31) r1 = N;
         CK(cudaMemcpyAsync(dA + r0 * E, A_host + r0 * E, (size_t)(r1 - r0) * E * sizeof(double),
@@ -1370,8 +1382,7 @@ mrc_status mrc_inverse_host(mrc_ctx *c, int d, int64_t N, const double *A_host, 
         r1 = std::min<int64_t>(2 * r1, N);
     }
     Arena ar{(char *)c->ws + 2 * seq};
-    int levels = 0;
-    s = inverse_impl(c, ar, d, N, dA, dpsi, prec, sweeps, &levels, st, nullptr, prec == MRC_MIXED, &rw);
+    s = inverse_impl(c, ar, d, N, dA, dpsi, prec, sweeps, st, nullptr, prec == MRC_MIXED, &rw);
     if (s != MRC_OK) return s;
     CK(rw.wait(st, N));
     CK(cudaMemcpyAsync(psi_host, dpsi, bytes, cudaMemcpyDeviceToHost, st));
@@ -1379,7 +1390,7 @@ mrc_status mrc_inverse_host(mrc_ctx *c, int d, int64_t N, const double *A_host, 
         CK(cudaEventRecord(c->ev1, st));
         memset(report, 0, sizeof(*report));
         report->res_left_l1 = report->res_right_l1 = report->res_max_abs = -1.0;
-        report->levels = levels;
+        report->levels = report_levels(d, N);
         report->sweeps = prec == MRC_MIXED ? sweeps : 0;
         s = read_status(c, st);
         float ms = 0.f;
@@ -1427,9 +1438,9 @@ mrc_status mrc_inverse_batched(mrc_ctx *c, int nmodels, const int *d, const int6
         m.d = d[b];
         m.E = d[b] * d[b];
         m.N = N[b];
-        m.m0 = base_size(d[b], N[b]);
+        m.m0 = base_size(d[b], N[b], level_prec(prec));
         m.Mr = pow2ceil(N[b]);
-        m.Mmax = newton_maxM(d[b], N[b]);
+        m.Mmax = newton_maxM(d[b], N[b], level_prec(prec));
         m.A = A[b];
         m.psi = psi[b];
         double lg = 1.0;
@@ -1557,9 +1568,7 @@ mrc_status mrc_inverse_batched(mrc_ctx *c, int nmodels, const int *d, const int6
         mrc_report &r = report[b];
         memset(&r, 0, sizeof(r));
         r.res_left_l1 = r.res_right_l1 = r.res_max_abs = -1.0;
-        int lv = 0;
-        for (int64_t m = base_size(d[b], N[b]); m < N[b]; m <<= 1) ++lv;
-        r.levels = lv;
+        r.levels = report_levels(d[b], N[b]);
         r.sweeps = sweeps;
         r.ms = ms;
         if (hs[b] && first == MRC_OK) first = (mrc_status)hs[b];
@@ -1646,7 +1655,7 @@ mrc_status mrc_first_entrance(mrc_ctx *c, int d, int64_t N, const double *q, con
     void *work = ar.take(mrc_scan_bytes(N, 1));
     CK(mrc_gather_blocks(q, d, N, Ci.data(), nC, Di.data(), nD, ACC, QCD, st));
     const size_t mark = ar.off;
-    s = inverse_impl(c, ar, nC, N, ACC, psiC, prec, sweeps, nullptr, st);
+    s = inverse_impl(c, ar, nC, N, ACC, psiC, prec, sweeps, st);
     if (s != MRC_OK) return s;
     ar.off = mark;
     double *gout = g ? g : gw;
@@ -1721,7 +1730,7 @@ mrc_status mrc_mre_solve(mrc_ctx *c, int d, int cc, int64_t N, const double *Q, 
     const size_t mark = ar.off;
     // e0 - Qbar_h (or e0 - Delta Q_h) and its inverse
     CK(mrc_mre_operator(Q, A, d, N, scheme, st));
-    s = inverse_impl(c, ar, d, N, A, psi, prec, sweeps, nullptr, st);
+    s = inverse_impl(c, ar, d, N, A, psi, prec, sweeps, st);
     if (s != MRC_OK) return s;
     ar.off = mark;
     // right-hand side: L_h - (1/2) Delta+ Q_h L_h(0) (mean-value rule) or L_h, then K = psi * R

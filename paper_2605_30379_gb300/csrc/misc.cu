@@ -1,5 +1,5 @@
-// misc.cu -- FP64 kernels around the FFT-Newton core: Gauss-Jordan inverse of
-// A(0), the direct recursion for the first m0 coefficients, survival
+// misc.cu -- FP64 kernels around the FFT-Newton core: the direct recursion for
+// the first coefficients of large matrices, survival
 // diagonal scans, residual norms, block gathers for first-entrance kernels and
 // the occupation / first-entrance reductions.
 #include <math.h>
@@ -38,78 +38,7 @@ __device__ void block_argmax(double &v, int &i, double *sv, int *si)
     __syncthreads();
 }
 
-// Gauss-Jordan with partial pivoting on [A0 | I] (d x 2d, row-major in W).
-// One CTA.  A pivot with |p| <= d 2^-52 max|A0| marks A0 singular: the
-// status word is set, `out` is filled with NaN and the kernel returns.
-__device__ __forceinline__ void gj_run(const double *__restrict__ A0, double *__restrict__ out,
-                                       double *__restrict__ W, int d, int *status)
-{
-    __shared__ double sv[32];
-    __shared__ int si[32];
-    extern __shared__ double fac[];  // [d]
-    const int n2 = 2 * d, tid = threadIdx.x, nt = blockDim.x;
-    double amax = 0.0;
-    for (int t = tid; t < d * n2; t += nt) {
-        int i = t / n2, j = t - i * n2;
-        double v = j < d ? A0[i * d + j] : ((j - d) == i ? 1.0 : 0.0);
-        W[t] = v;
-        if (j < d) amax = fmax(amax, fabs(v));
-    }
-    int dummy = 0;
-    block_argmax(amax, dummy, sv, si);
-    const double tol = (double)d * 0x1p-52 * amax;
-    for (int col = 0; col < d; ++col) {
-        double best = -1.0;
-        int piv = 0x7fffffff;
-        for (int i = col + tid; i < d; i += nt) {
-            double v = fabs(W[i * n2 + col]);
-            if (v > best || (v == best && i < piv)) { best = v; piv = i; }
-        }
-        block_argmax(best, piv, sv, si);
-        if (!(best > tol)) {
-            if (tid == 0) atomicExch(status, MRC_ST_SINGULAR);
-            for (int t = tid; t < d * d; t += nt) out[t] = __longlong_as_double(0x7ff8000000000000ll);
-            return;
-        }
-        if (piv != col)
-            for (int j = tid; j < n2; j += nt) {
-                double t = W[col * n2 + j];
-                W[col * n2 + j] = W[piv * n2 + j];
-                W[piv * n2 + j] = t;
-            }
-        __syncthreads();
-        const double p = W[col * n2 + col];
-        __syncthreads();
-        for (int j = tid; j < n2; j += nt) W[col * n2 + j] /= p;
-        __syncthreads();
-        for (int i = tid; i < d; i += nt) fac[i] = W[i * n2 + col];
-        __syncthreads();
-        for (int t = tid; t < d * n2; t += nt) {
-            int i = t / n2, j = t - i * n2;
-            if (i != col) W[t] = fma(-fac[i], W[col * n2 + j], W[t]);
-        }
-        __syncthreads();
-    }
-    for (int t = tid; t < d * d; t += nt) {
-        int i = t / d, j = t - i * d;
-        out[t] = W[i * n2 + d + j];
-    }
-}
-
-__global__ void __launch_bounds__(1024) gj_kernel(const double *__restrict__ A0, double *__restrict__ out,
-                                                  double *__restrict__ W, int d, int *status)
-{
-    gj_run(A0, out, W, d, status);
-}
-
-// one CTA per model of a batch
-__global__ void __launch_bounds__(1024) gj_batch_kernel(const __grid_constant__ SegParams<GjArgs> P)
-{
-    const GjArgs &g = P.a[blockIdx.x];
-    gj_run(g.A0, g.out, g.W, g.d, g.status);
-}
-
-// Direct recursion for the first m0 coefficients (left form, Theorem 2.2):
+// Direct recursion for psi(1 .. m0-1), d > 32 (left form, Theorem 2.2):
 //   psi(k) = A(0)^{-1} [ - sum_{l=1..k} A(l) psi(k-l) ],  k = 1..m0-1,
 // with psi(0) = A(0)^{-1} already in place.  CTA j owns column j (columns
 // are independent in the left recursion), thread i owns row i.
@@ -504,14 +433,6 @@ inline unsigned grid_for(int64_t n, int bs = 256)
 
 } // namespace
 
-cudaError_t mrc_gauss_jordan(const double *A0, double *out, double *work, int d, int *status, cudaStream_t st)
-{
-    mrc_prof_pre(7, st);
-    gj_kernel<<<1, 1024, sizeof(double) * d, st>>>(A0, out, work, d, status);
-    mrc_prof_post(7, st, 0, 0);
-    return cudaGetLastError();
-}
-
 cudaError_t mrc_base_case(const double *A, double *psi, int d, int64_t m0, cudaStream_t st)
 {
     if (m0 <= 1) return cudaSuccess;
@@ -636,15 +557,6 @@ __global__ void f64_to_f32_batch_kernel(const __grid_constant__ SegParams<CvtArg
     const int64_t e0 = (int64_t)(blockIdx.x - P.first[s]) * MRC_CVT_CHUNK;
     const int64_t e1 = min(g.n, e0 + MRC_CVT_CHUNK);
     for (int64_t i = e0 + threadIdx.x; i < e1; i += blockDim.x) g.y[i] = f64_to_f32_rn(g.x[i]);
-}
-
-cudaError_t mrc_gauss_jordan_batch(const SegParams<GjArgs> &P, int dmax, cudaStream_t st)
-{
-    if (P.nseg <= 0) return cudaSuccess;
-    mrc_prof_pre(7, st);
-    gj_batch_kernel<<<P.nseg, 1024, sizeof(double) * dmax, st>>>(P);
-    mrc_prof_post(7, st, 0, 0);
-    return cudaGetLastError();
 }
 
 cudaError_t mrc_base_case_batch(const SegParams<BaseArgs> &P, int dmax, cudaStream_t st)

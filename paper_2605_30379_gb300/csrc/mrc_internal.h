@@ -103,11 +103,11 @@ __device__ __forceinline__ int seg_find(const SegParams<A> &P, unsigned b)
     return lo;
 }
 
-// argument blocks of the batched Gauss-Jordan, base-case and conversion kernels
-struct GjArgs {
-    const double *A0;
-    double *out, *W;
-    int d;
+// argument blocks of the seed, base-case and conversion kernels
+struct SeedArgs {
+    const double *A;  // its first m0 coefficients are read
+    double *psi;
+    int d, m0;
     int *status;
 };
 struct BaseArgs {
@@ -229,10 +229,11 @@ cudaError_t mrc_pairq_seg(const SegParams<PairArgs> &P, unsigned nctas, double b
 
 // api.cu: the Newton doubling schedule of Eq. (newton), shared by every
 // inverse entry point (mrc_inverse* and mrc_inverse_noalloc).
-//   mrc_base_size: the first m0 coefficients come from the direct recursion;
+//   mrc_base_size: the first m0 coefficients come from direct sums (seed.cu);
 //   mrc_newton_maxM: the largest level m (its transforms have M = m points).
-int64_t mrc_base_size(int d, int64_t N);
-int64_t mrc_newton_maxM(int d, int64_t N);
+// (f32: of the mixed path's FP32 levels)
+int64_t mrc_base_size(int d, int64_t N, bool f32);
+int64_t mrc_newton_maxM(int d, int64_t N, bool f32);
 // Row ranges of A still being uploaded (mrc_inverse_host): rows
 // [end[i-1], end[i]) complete at ev[i]; wait(s, rows) makes stream s wait
 // until rows [0, rows) are on the device.  n == 0: everything is there.
@@ -255,7 +256,7 @@ typedef cudaError_t (*mrc_level_fft_fn)(void *user, int prec, const FftSrc &src,
 typedef cudaError_t (*mrc_level_product_fn)(void *user, int prec, const void *zx, const void *zy, void *zc,
                                             int64_t M, int d, const void *tw, int tw_log, cudaStream_t st);
 // Buffers of the levels: three spectra and the FFT scratch, each
-// mrc_newton_maxM(d, N) * d^2 complex values of the working precision.
+// mrc_newton_maxM * d^2 complex values of the working precision.
 struct NewtonBufs {
     void *b0, *b1, *b2, *bt;
 };
@@ -263,16 +264,21 @@ struct NewtonBufs {
 // psi32 (FP32 levels of the mixed path) A is read from its binary32 copy,
 // converted here row range by row range, and psi is read and written in
 // binary32.  rw (nullable) delays each level until its rows of A arrived.
-// Returns 0 or 4 (a CUDA error, printed); *levels (nullable) = levels run.
+// Returns 0 or 4 (a CUDA error, printed).
 // a32_rows: rows of A32 already converted by the caller (the rest are
 // converted level by level, as each level first reads them)
 int mrc_newton_levels(int prec, int d, int64_t N, const double *A, double *psi, int64_t m0, const NewtonBufs &b,
                       const void *tw, int tw_log, mrc_level_fft_fn fft, mrc_level_product_fn product, void *user,
-                      cudaStream_t st, const RowWait *rw, float *A32, float *psi32, int *levels,
-                      int64_t a32_rows = 0);
+                      cudaStream_t st, const RowWait *rw, float *A32, float *psi32, int64_t a32_rows = 0);
+
+// seed.cu: per model psi(0) = A(0)^(-1) (a singular A(0): NaN, and 2 in
+// *status) and, for d <= MRC_SEED_DMAX, psi(1 .. m0-1); larger models take
+// psi(1) from mrc_base_case
+#define MRC_SEED_DMAX 32
+cudaError_t mrc_seed_init(void);
+cudaError_t mrc_seed(const SegParams<SeedArgs> &P, cudaStream_t st);
 
 // misc.cu
-cudaError_t mrc_gauss_jordan(const double *A0, double *out, double *work, int d, int *status, cudaStream_t st);
 cudaError_t mrc_base_case(const double *A, double *psi, int d, int64_t m0, cudaStream_t st);
 cudaError_t mrc_row_sums(const double *q, double *rs, int d, int64_t N, cudaStream_t st);
 // x(k) <- offset + scale sum_{l <= k} x(l) down the rows (scale = +-1);
@@ -288,10 +294,8 @@ cudaError_t mrc_occupation_k(const double *P, int d, int64_t N, const double *al
                              cudaStream_t st);
 cudaError_t mrc_one_minus(const double *x, double *y, int64_t n, cudaStream_t st);
 cudaError_t mrc_f64_to_f32(const double *x, float *y, int64_t n, cudaStream_t st);
-// batched: Gauss-Jordan of every segment's A(0) (one CTA each, dmax the
-// largest d), the direct recursion (dmax x nseg CTAs), and conversions
+// batched: the direct recursion (dmax x nseg CTAs) and conversions
 // (P.first: CTA starts in MRC_CVT_CHUNK elements; nctas in all)
-cudaError_t mrc_gauss_jordan_batch(const SegParams<GjArgs> &P, int dmax, cudaStream_t st);
 cudaError_t mrc_base_case_batch(const SegParams<BaseArgs> &P, int dmax, cudaStream_t st);
 cudaError_t mrc_f64_to_f32_batch(const SegParams<CvtArgs> &P, unsigned nctas, cudaStream_t st);
 // series Gauss-Jordan on W = [P_A | I] ([N][d][2d]): build W (clearing the

@@ -48,7 +48,7 @@ constexpr size_t kTwOff = 256;
 constexpr size_t kTwBytes = (size_t)16 << kTwLog;
 constexpr size_t kWorkOff = kTwOff + kTwBytes;
 
-int64_t max_level(int d, int64_t N) { return mrc_newton_maxM(d, N); }
+int64_t max_level(int d, int64_t N) { return mrc_newton_maxM(d, N, false); }
 
 // the level transforms and products: the built-in FFT plans and the default
 // FP64 product kernel (no autotuning here)
@@ -70,7 +70,7 @@ cudaError_t product_f64(void *status, int, const void *zx, const void *zy, void 
 size_t need_bytes(int d, int64_t N)
 {
     const size_t E = (size_t)d * d;
-    return kWorkOff + up256(sizeof(double) * 2 * E) + 3 * up256((size_t)max_level(d, N) * E * 16) +
+    return kWorkOff + 3 * up256((size_t)max_level(d, N) * E * 16) +
            up256(mrc_fft_scratch_elems(max_level(d, N), (int)E) * 16);
 }
 
@@ -91,7 +91,8 @@ mrc_status setup(int dev, unsigned char **out)
         return MRC_ERR_CUDA;
     }
     unsigned char *base = (unsigned char *)p;
-    if (mrc_init_f64() != cudaSuccess || mrc_tcp_init() != cudaSuccess) return MRC_ERR_CUDA;
+    if (mrc_init_f64() != cudaSuccess || mrc_tcp_init() != cudaSuccess || mrc_seed_init() != cudaSuccess)
+        return MRC_ERR_CUDA;
     if (mrc_twiddles_f64(base + kTwOff, kTwLog, 0) != cudaSuccess) return MRC_ERR_CUDA;
     if (cudaStreamSynchronize(0) != cudaSuccess) return MRC_ERR_CUDA;
     g_addr[dev] = base;
@@ -131,20 +132,22 @@ extern "C" mrc_status mrc_inverse_noalloc(int d, int64_t N, const double *A, dou
     const int E = d * d;
     int *status = (int *)(base + kStatusOff);
     const void *tw = base + kTwOff;
-    double *gjw = (double *)(base + kWorkOff);
-    unsigned char *spec = base + kWorkOff + up256(sizeof(double) * 2 * E);
+    unsigned char *spec = base + kWorkOff;
     const int64_t Mmax = max_level(d, N);
     const size_t sb = up256((size_t)Mmax * E * 16);
     void *b0 = spec, *b1 = spec + sb, *b2 = spec + 2 * sb, *bt = spec + 3 * sb;
 
     // the status word keeps the previous call's value: clear it first
     CKN(cudaMemsetAsync(status, 0, sizeof(int), st));
-    CKN(mrc_gauss_jordan(A, psi, gjw, d, status, st));
-    const int64_t m0 = mrc_base_size(d, N);
-    CKN(mrc_base_case(A, psi, d, m0, st));
+    const int64_t m0 = mrc_base_size(d, N, false);
+    SegParams<SeedArgs> sp{};
+    sp.nseg = 1;
+    sp.a[0] = SeedArgs{A, psi, d, (int)m0, status};
+    CKN(mrc_seed(sp, st));
+    if (d > MRC_SEED_DMAX) CKN(mrc_base_case(A, psi, d, m0, st));
     const NewtonBufs nb{b0, b1, b2, bt};
     if (mrc_newton_levels(PREC_F64, d, N, A, psi, m0, nb, tw, kTwLog, fft_f64, product_f64, status, st, nullptr,
-                          nullptr, nullptr, nullptr) != 0)
+                          nullptr, nullptr) != 0)
         return MRC_ERR_CUDA;
     CKN(cudaStreamSynchronize(st));
     int h = 0;

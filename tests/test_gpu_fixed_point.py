@@ -177,3 +177,34 @@ def test_diagonal_product_non_finite(mrc):
     assert not torch.isfinite(got[:, 2, 1]).any()
     got[:, 2, 1] = ref[:, 2, 1]
     assert torch.equal(got, ref)
+
+
+@pytest.mark.parametrize("d", [1, 2, 4, 10, 16, 25, 26, 32, 33, 47, 48, 64, 100, 256])
+def test_seed_sizes(mrc, d):
+    """The start of the doubling on one cluster: A(0) with a zero diagonal (every
+    pivot from another row) and dense signed coefficients, horizons below, at
+    and beyond the direct levels (256 coefficients at d <= 4 down to 2 for
+    d > 32), rows spread evenly and unevenly over the 16 CTAs."""
+    rng = np.random.default_rng(d)
+    for N in ([1, 2, 3, 7, 255, 256, 300] if d <= 4 else [1, 2, 5, 33] if d <= 64 else [1, 3]):
+        A = rng.standard_normal((N, d, d)) * (0.5 ** np.arange(N))[:, None, None] * 0.2 / d
+        A[0] += np.roll(np.diag(2.0 + np.arange(d)), 1, axis=1)
+        ref = oracle.inverse_left(A)
+        psi = mrc.inverse(dev(A), prec="fp64", report=True)[0].cpu().numpy()
+        assert np.abs(psi - ref).max() <= 1e-12 * max(1.0, np.abs(ref).max())
+
+
+@pytest.mark.parametrize("d", [3, 32, 33, 100, 512])
+def test_seed_singular(mrc, d):
+    rng = np.random.default_rng(d)
+    A = np.zeros((4, d, d))
+    A[0] = rng.standard_normal((d, d))
+    A[0, :, d - 1] = 0.0
+    with pytest.raises(mrc.MrcError) as ei:
+        mrc.inverse(dev(A), prec="fp64", report=True)
+    assert ei.value.status == 2
+    assert torch.isnan(mrc.inverse(dev(A), prec="fp64")[0]).all()
+    with pytest.raises(mrc.MrcError):
+        mrc.sync_status()
+    eye = torch.eye(d, dtype=torch.float64, device="cuda")[None]
+    assert torch.equal(mrc.inverse(eye, report=True)[0], eye)
