@@ -309,10 +309,10 @@ __device__ __forceinline__ void fft_stage(const FftArgs &a, cx<typename FftC<T>:
     // FP64: the shift that leaves this stage its growth (|re|, |im| of its inputs
     // below 2^57, 2^59 in the last stage, whose outputs meet no more products)
     [[maybe_unused]] int qs = 0;
-    [[maybe_unused]] long long qr = 0;
+    [[maybe_unused]] long long qc = 0;
     if constexpr (!FIRST && QF) {
         qs = max(0, 64 - __clz((int)sor[(S - 1) * EC + (tid & (EC - 1))]) - (LAST ? Q_TOP - 1 : Q_TOP - 3));
-        qr = qs ? 1ll << (qs - 1) : 0ll;
+        qc = q_round_start(qs);
         ex += qs;
     }
     if (!FIRST) __syncthreads();  // every read of sm done before the in-place writes
@@ -325,7 +325,7 @@ __device__ __forceinline__ void fft_stage(const FftArgs &a, cx<typename FftC<T>:
                 v[u][0] = {{q_shift_even(v[u][0].re.v, qs)}, {q_shift_even(v[u][0].im.v, qs)}};
 #pragma unroll
                 for (int q = 1; q < r; ++q)
-                    v[u][q] = q_shift(c_mul(v[u][q], stw[(bm * q) << (LOGR - LNS - LR)], qs ? 0 : 1 << 29), qs, qr);
+                    v[u][q] = q_shift(c_mul(v[u][q], stw[(bm * q) << (LOGR - LNS - LR)], qc), qs);
             } else {
 #pragma unroll
                 for (int q = 1; q < r; ++q) v[u][q] = c_mul(v[u][q], stw[(bm * q) << (LOGR - LNS - LR)]);
@@ -475,7 +475,7 @@ __device__ __forceinline__ void fft_pass_body(const FftArgs &a, int64_t j, int e
     if constexpr (QF)
         for (int t = tid; t < 3 * EC; t += P::NT) {
             sor[t] = 0u;
-            if (t < EC) sexp[t] = 1;
+            if (t < EC) sexp[t] = Q_EXMIN;
         }
     // table entry of w (fixed point: divided by 2^s, the radix of the stage that applies it)
     auto table = [&](cx<T> w, [[maybe_unused]] int s) -> W {
@@ -493,7 +493,7 @@ __device__ __forceinline__ void fft_pass_body(const FftArgs &a, int64_t j, int e
     if constexpr (QF) {
         // the entry's largest exponent over the CTA's R points (a thread's points
         // share their entry: NT is a multiple of EC or the CTA one unit per thread)
-        int m = 1;
+        int m = 0;
 #pragma unroll
         for (int q = 0; q < P::EPT; ++q) m = max(m, max(q_exponent(pre[q].re), q_exponent(pre[q].im)));
         constexpr int NL = P::NT < 32 ? P::NT : 32;  // lanes of a warp in use

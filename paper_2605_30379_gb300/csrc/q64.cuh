@@ -41,23 +41,51 @@ constexpr int Q_TOP = 60;
 constexpr int Q_NONFINITE = 4096;  // alignment exponent of a column or row that holds an Inf or NaN
 constexpr int Q_MASK30 = (1 << 30) - 1;
 
+// 64-bit values in two registers, with the instructions written out: from C++
+// expressions the compiler made twice as many of them (a complex product 63
+// instructions, with these 29)
+__device__ __forceinline__ long long q_wide(int a, int b, long long c)
+{
+    long long r;
+    asm("mad.wide.s32 %0, %1, %2, %3;" : "=l"(r) : "r"(a), "r"(b), "l"(c));
+    return r;
+}
+__device__ __forceinline__ int q_lo(long long a) { return (int)a; }
+__device__ __forceinline__ int q_hi(long long a) { return (int)(a >> 32); }
+__device__ __forceinline__ long long q_join(int lo, int hi)
+{
+    long long r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "r"(lo), "r"(hi));
+    return r;
+}
+// a >> 30, as a 32-bit number and as a 64-bit one
+__device__ __forceinline__ int q_top30(long long a)
+{
+    int r;
+    asm("shf.l.clamp.b32 %0, %1, %2, 2;" : "=r"(r) : "r"(q_lo(a)), "r"(q_hi(a)));
+    return r;
+}
+__device__ __forceinline__ long long q_sar30(long long a) { return q_join(q_top30(a), q_hi(a) >> 30); }
+
 // biased exponent of a double (0 for zero and subnormals, 2047 for Inf / NaN)
 __device__ __forceinline__ int q_exponent(double x) { return (__double2hiint(x) >> 20) & 0x7ff; }
 
-// x 2^(top + 1022 - ex) rounded to an integer, for |x| < 2^(ex - 1022) and
-// top <= 60: the magnitude is rounded (symmetric in the sign, so that a column
-// of one sign is not shortened; a tie, frequent where few bits are dropped,
-// goes by a mantissa bit that is kept); neg flips the sign.
+// x 2^(top + 1022 - ex) rounded to an integer, for |x| < 2^(ex - 1022), ex >=
+// Q_EXMIN and top <= 60: the magnitude is rounded (symmetric in the sign, so that
+// a column of one sign is not shortened; a tie, frequent where few bits are
+// dropped, goes by a mantissa bit that is kept); neg (0 or -1) flips the sign.
+// Q_EXMIN shifts zeros (and subnormals) out altogether.
+constexpr int Q_EXMIN = 64;
 __device__ __forceinline__ q64 q_decode(double x, int ex, int top, int neg = 0)
 {
     const unsigned hw = (unsigned)__double2hiint(x), lw = (unsigned)__double2loint(x);
-    const int e = (int)((hw >> 20) & 0x7ffu);
-    const unsigned mh = (hw & 0xfffffu) | (e ? 0x100000u : 0u);
-    const int sh = min(ex - max(e, 1) + (62 - top), 63);
-    const unsigned long long m53 = ((unsigned long long)mh << 42) | ((unsigned long long)lw << 10);
-    const unsigned long long m = (((m53 - (hw & 1u)) >> sh) + 1ull) >> 1;
-    const long long s = (long long)((int)hw >> 31) ^ (long long)neg;
-    return {((long long)m ^ s) - s};
+    const int sh = min(ex + (62 - top) - (int)((hw >> 20) & 0x7ffu), 63);
+    const unsigned mh = (hw & 0xfffffu) | 0x100000u;
+    const long long m = q_join((int)(lw << 10), (int)__funnelshift_l(lw, mh, 10)) - (long long)(hw & 1u);
+    const unsigned long long w = ((unsigned long long)m >> sh) + 1ull;
+    const int s = ((int)hw >> 31) ^ neg;
+    const long long r = (long long)(w >> 1);
+    return {q_join(q_lo(r) ^ s, q_hi(r) ^ s) - (long long)s};
 }
 
 // n / 2^11 rounded half to even
@@ -68,36 +96,39 @@ __device__ __forceinline__ unsigned long long q_round11(unsigned long long n)
 }
 
 // v 2^(eb - 1086) rounded to a double (flushed to zero below the normal
-// range, infinity above it): a value with leading bit 63 - lz gets the biased
-// exponent eb - lz.
+// range, infinity above it), |v| < 2^63: a value with leading bit 63 - lz gets
+// the biased exponent eb - lz.
 __device__ __forceinline__ double q_encode(q64 x, int eb, unsigned sgn)
 {
-    const long long s = x.v >> 63;
-    const unsigned long long a = (unsigned long long)((x.v ^ s) - s);
-    const int lz = __clzll((long long)a);
-    const unsigned long long n = a << (lz & 63);
-    const unsigned long long m = q_round11(n);
+    const int s = q_hi(x.v) >> 31;
+    const long long a = q_join(q_lo(x.v) ^ s, q_hi(x.v) ^ s) - (long long)s;
+    const unsigned sg = ((unsigned)s ^ sgn) & 0x80000000u;
+    int lz = __clz(q_hi(a)) - 1;  // leading bit to 62
+    // the common case: the value's high word is not zero and no exponent between
+    // eb - 63 and eb leaves the range
+    if (q_hi(a) != 0 && (unsigned)(eb - 64) < 2047u - 64u) {
+        const unsigned hi = __funnelshift_l((unsigned)q_lo(a), (unsigned)q_hi(a), lz);
+        const unsigned long long n = (unsigned long long)q_join(q_lo(a) << lz, (int)hi) + 0x200ull;
+        return __hiloint2double((int)((unsigned)(n >> 42) + ((unsigned)(eb - 2 - lz) << 20) | sg), (int)(n >> 10));
+    }
+    lz = __clzll(a);
+    const unsigned long long m = q_round11((unsigned long long)a << (lz & 63));
     const int e = eb - lz;
     unsigned hi = (unsigned)(m >> 32) + ((unsigned)(e - 1) << 20), lo = (unsigned)m;
-    const bool tiny = e < 1 || a == 0ull;
-    hi = tiny ? 0u : hi;
-    lo = tiny ? 0u : lo;
+    if (e < 1 || a == 0) hi = lo = 0u;
     if (e >= 2047) {
-        hi = a == 0ull ? 0u : 0x7ff00000u;
+        hi = a == 0 ? 0u : 0x7ff00000u;
         lo = 0u;
     }
-    hi |= ((unsigned)s ^ sgn) & 0x80000000u;
-    return __hiloint2double((int)hi, (int)lo);
+    return __hiloint2double((int)(hi | sg), (int)lo);
 }
-
-__device__ __forceinline__ long long q_wide(int a, int b, long long c) { return (long long)a * b + c; }
 
 // a w for a real factor w <= 2^60 (Q60)
 __device__ __forceinline__ long long q_mul(long long a, long long w)
 {
-    const int ah = (int)(a >> 30), al = (int)a & Q_MASK30, wh = (int)(w >> 30), wl = (int)w & Q_MASK30;
+    const int ah = q_top30(a), al = q_lo(a) & Q_MASK30, wh = (int)(w >> 30), wl = (int)w & Q_MASK30;
     const long long mid = q_wide(al, wh, q_wide(ah, wl, (1ll << 29) + wl / 2));  // + the mean of al wl
-    return q_wide(ah, wh, mid >> 30);
+    return q_wide(ah, wh, q_sar30(mid));
 }
 
 template <>
@@ -113,23 +144,27 @@ struct Ar<q64> {
     static __device__ __forceinline__ q64 rsqrt2() { return {815238614083298888ll}; }
 };
 
-// a w; the middle products start at r0: 2^29 rounds the result, 0 leaves its
-// floor.  To it they add the mean of the low products that are left out (the
-// low limbs of a are 2^29 in the mean): the same twiddle serves every entry of
-// a matrix, so that the offset would add up over a row.
-__device__ __forceinline__ cx<q64> c_mul(cx<q64> a, qtw w, int r0 = 1 << 29)
+// a w / 2^s without its last shift: high + middle products as a 64-bit number
+// of weight 2^-s, to be shifted right by s.  c is the middle products' start:
+// q_round_start(s) rounds the result.  To it they add the mean of the low
+// products that are left out (the low limbs of a are 2^29 in the mean): the same
+// twiddle serves every entry of a matrix, so that the offset would add up over a
+// row.
+__device__ __forceinline__ long long q_round_start(int s) { return 1ll << (29 + s); }
+__device__ __forceinline__ cx<q64> c_mul(cx<q64> a, qtw w, long long c = 1ll << 29)
 {
-    const int arh = (int)(a.re.v >> 30), arl = (int)a.re.v & Q_MASK30;
-    const int aih = (int)(a.im.v >> 30), ail = (int)a.im.v & Q_MASK30;
+    const int arh = q_top30(a.re.v), arl = q_lo(a.re.v) & Q_MASK30;
+    const int aih = q_top30(a.im.v), ail = q_lo(a.im.v) & Q_MASK30;
     const int nh = -aih, nl = -ail;
-    long long mr = q_wide(arh, w.rl, r0 + ((w.rl - w.il) >> 1)), mi = q_wide(arh, w.il, r0 + ((w.rl + w.il) >> 1));
+    long long mr = q_wide(arh, w.rl, c + (long long)((w.rl - w.il) >> 1));
+    long long mi = q_wide(arh, w.il, c + (long long)((w.rl + w.il) >> 1));
     mr = q_wide(arl, w.rh, mr);
     mi = q_wide(arl, w.ih, mi);
     mr = q_wide(nh, w.il, mr);
     mi = q_wide(aih, w.rl, mi);
     mr = q_wide(nl, w.ih, mr);
     mi = q_wide(ail, w.rh, mi);
-    return {{q_wide(nh, w.ih, q_wide(arh, w.rh, mr >> 30))}, {q_wide(aih, w.rh, q_wide(arh, w.ih, mi >> 30))}};
+    return {{q_wide(nh, w.ih, q_wide(arh, w.rh, q_sar30(mr)))}, {q_wide(aih, w.rh, q_wide(arh, w.ih, q_sar30(mi)))}};
 }
 
 // a / 2^s rounded half to even, s < 32
@@ -139,14 +174,12 @@ __device__ __forceinline__ long long q_shift_even(long long a, int s)
     return (a + h) >> s;
 }
 
-// (a + rd) / 2^s, s < 32: with rd = 2^(s-1) unbiased for the floors of numbers
-// whose fractions are spread evenly
-__device__ __forceinline__ cx<q64> q_shift(cx<q64> a, int s, long long rd)
+// a >> s, s < 32
+__device__ __forceinline__ cx<q64> q_shift(cx<q64> a, int s)
 {
-    const long long r = a.re.v + rd, i = a.im.v + rd;
-    const unsigned rl = __funnelshift_r((unsigned)r, (unsigned)(r >> 32), s), il = __funnelshift_r((unsigned)i, (unsigned)(i >> 32), s);
-    const int rh = (int)(r >> 32) >> s, ih = (int)(i >> 32) >> s;
-    return {{((long long)rh << 32) | rl}, {((long long)ih << 32) | il}};
+    const int rl = (int)__funnelshift_r((unsigned)q_lo(a.re.v), (unsigned)q_hi(a.re.v), s), rh = q_hi(a.re.v) >> s;
+    const int il = (int)__funnelshift_r((unsigned)q_lo(a.im.v), (unsigned)q_hi(a.im.v), s), ih = q_hi(a.im.v) >> s;
+    return {{q_join(rl, rh)}, {q_join(il, ih)}};
 }
 
 // the magnitude bits of a value's high word
@@ -233,7 +266,7 @@ __device__ __forceinline__ void q_split(cx<double> za, cx<double> zb, qtw w, int
 __device__ __forceinline__ unsigned q_magnitude(double x) { return (unsigned)__double2hiint(x) & 0x7fffffffu; }
 __device__ __forceinline__ int q_align(unsigned m)
 {
-    const int ex = max(1, (int)((m + 0x8000u) >> 20));
+    const int ex = max(Q_EXMIN, (int)((m + 0x8000u) >> 20));
     return ex >= 2047 ? Q_NONFINITE : ex;
 }
 
