@@ -127,6 +127,9 @@ mrc_status ensure_tw(mrc_ctx *c, int prec, cudaStream_t st)
     void *p = nullptr;
     if (cudaMalloc(&p, OPS[prec].cxb << MRC_TW_LOG) != cudaSuccess) return MRC_ERR_NO_MEMORY;
     CK(OPS[prec].twiddles(p, MRC_TW_LOG, st));
+    // a kernel that reads the table beside its predecessor's end must not have
+    // the kernel that writes it for that predecessor
+    CK(mrc_order(st));
     c->tw[prec] = p;
     return MRC_OK;
 }
@@ -854,7 +857,7 @@ mrc_status fft_stage(mrc_ctx *c, int prec, int64_t M, int dir, const std::vector
             for (size_t i = i0; i < i1; ++i) {
                 P->first[i - i0] = total;
                 P->a[i - i0] = ps[i].a[k];
-                total += ps[i].nchunk * ps[i].nrow[k];
+                total += ps[i].nchunk[k] * ps[i].nrow[k];
                 by += ps[i].bytes[k];
                 fl += ps[i].flops[k];
             }

@@ -467,7 +467,30 @@ __device__ __forceinline__ void fft_pass_body(const FftArgs &a, int64_t j, int e
     const int tid = threadIdx.x;
     const int ecount = min(EC, a.E - e0);
     const int64_t jm = j & (a.Ns - 1);
-    // first-stage global loads before the twiddle tables are filled (both latencies overlap)
+    // table entry of w (fixed point: divided by 2^s, the radix of the stage that applies it)
+    auto table = [&](cx<T> w, [[maybe_unused]] int s) -> W {
+        if constexpr (QF) return q_twiddle(w, s, INV);
+        else return INV ? c_conj(w) : w;
+    };
+    auto fill = [&]() {
+        if constexpr (P::NSTAGE > 1)
+            for (int t = tid; t < R; t += P::NT) stw[t] = table(tw[(int64_t)t << (a.tw_log - LOGR)], 0);
+        if (a.Ns > 1) {
+            const int sh = a.tw_log - (a.logNs + LOGR);
+            for (int t = tid; t < R; t += P::NT) spt[t] = table(tw[(jm * t) << sh], P::FIRST);
+        }
+    };
+    // beside its predecessor's end a small FP64 launch fills its twiddle tables;
+    // otherwise the first-stage global loads go first (both latencies overlap).
+    // (The FP32 and double-float passes have no such branch: it cost the large
+    // ones 0.5 %.)
+    if constexpr (QF) {
+        if (a.pdl) {
+            overlap_release();
+            fill();
+        }
+        overlap_wait();
+    }
     cx<T> pre[P::EPT];
     if (a.src_mode == SRC_CPLX) fft_gather_any<T, LOGR, EC, SRC_CPLX>(a, pre, j, e0, ecount);
     else if (a.src_mode == SRC_REAL32) fft_gather_any<T, LOGR, EC, SRC_REAL32>(a, pre, j, e0, ecount);
@@ -477,17 +500,7 @@ __device__ __forceinline__ void fft_pass_body(const FftArgs &a, int64_t j, int e
             sor[t] = 0u;
             if (t < EC) sexp[t] = Q_EXMIN;
         }
-    // table entry of w (fixed point: divided by 2^s, the radix of the stage that applies it)
-    auto table = [&](cx<T> w, [[maybe_unused]] int s) -> W {
-        if constexpr (QF) return q_twiddle(w, s, INV);
-        else return INV ? c_conj(w) : w;
-    };
-    if constexpr (P::NSTAGE > 1)
-        for (int t = tid; t < R; t += P::NT) stw[t] = table(tw[(int64_t)t << (a.tw_log - LOGR)], 0);
-    if (a.Ns > 1) {
-        const int sh = a.tw_log - (a.logNs + LOGR);
-        for (int t = tid; t < R; t += P::NT) spt[t] = table(tw[(jm * t) << sh], P::FIRST);
-    }
+    if (!QF || !a.pdl) fill();
     __syncthreads();
     int ex = 0;
     if constexpr (QF) {
@@ -911,7 +924,7 @@ __global__ void twiddle_kernel(cx<T> *tw, int log)
 // ---------------------------------------------------------------------------
 // Launch table of the FFT pass instantiations: entry [ec_index][logR], where
 // ec_index 0 is the default entries per CTA (MRC_F32_EC for 8-byte complex
-// values, MRC_DD_EC for 16-byte ones) and 1 is 4 entries per CTA.
+// values, MRC_DD_EC for 16-byte ones), 1 is 4 entries per CTA and 2 (FP64) one.
 using FftKernel = void (*)(FftArgs);
 struct FftEntry {
     FftKernel fn;
@@ -938,6 +951,14 @@ constexpr FftKernel fft_pass_ec4()
     else return fft_pass_kernel<T, L, 4>;
 }
 
+// one entry per CTA, for the radices that pick_ec takes it for
+template <class T, int L>
+constexpr FftKernel fft_pass_ec1()
+{
+    if constexpr (L >= 8) return fft_pass_or_mb<T, L, 1>();
+    else return nullptr;
+}
+
 template <class T, int L, int EC>
 constexpr FftSegKernel fft_seg_or_mb()
 {
@@ -953,5 +974,7 @@ void fft_fill_shifted(FftEntry (*t)[11], FftSegEntry *ts, std::integer_sequence<
     constexpr int ECD = fft_default_ec<T>();
     ((t[0][OFF + L] = FftEntry{fft_pass_or_mb<T, OFF + L, ECD>(), FftPlan<T, OFF + L, ECD>::NT}), ...);
     ((t[1][OFF + L] = FftEntry{fft_pass_ec4<T, OFF + L>(), FftPlan<T, OFF + L, 4>::NT}), ...);
+    if constexpr (FftC<T>::Q)
+        ((t[2][OFF + L] = FftEntry{fft_pass_ec1<T, OFF + L>(), FftPlan<T, OFF + L, 1>::NT}), ...);
     ((ts[OFF + L] = FftSegEntry{fft_seg_or_mb<T, OFF + L, ECD>(), FftPlan<T, OFF + L, ECD>::NT}), ...);
 }

@@ -8,11 +8,11 @@
 #include <utility>
 #include "kernels.cuh"
 
-// table[ec_index][logR] (ec_index 0: default entries per CTA, 1: 4), filled by
+// table[ec_index][logR] (ec_index 0: default entries per CTA, 1: 4, 2: 1 (FP64)), filled by
 // the two FFT translation units of this precision (low and high radices);
 // specialised once per precision by MRC_DEFINE_PREC.
 template <class T>
-const FftEntry (&fft_table())[2][11];
+const FftEntry (&fft_table())[3][11];
 template <class T>
 const FftSegEntry (&fft_seg_table())[11];
 
@@ -35,9 +35,22 @@ template <class T>
 constexpr int default_ec() { return fft_default_ec<T>(); }
 
 // entries per CTA: the full default when E allows, else 4 (>= 32-byte row
-// segments; lanes beyond E idle)
+// segments; lanes beyond E idle).  FP64 passes are bound by instructions, and a
+// CTA of 8 entries of a radix-2^10 pass holds an SM for 20 us: where 8 entries
+// leave SMs without a CTA, 4 or (from radix 2^8, whose CTAs still have a warp) 1
+// spread the same work (d = 16, M = 1024: 32 CTAs of 8 entries 32 us, whole call
+// 1.30 -> @@ ms).
 template <class T>
-int pick_ec(int E) { return E >= default_ec<T>() ? default_ec<T>() : 4; }
+int pick_ec(int E, int logR, int64_t nrow)
+{
+    if (std::is_same<T, double>::value) {
+        for (int ec = 8; ec > 1; ec >>= 1)
+            if (ec != 2 && ((E + ec - 1) / ec) * nrow >= 152 && (E >= ec || ec == 4)) return ec;
+        if (logR >= 8) return 1;
+        return 4;
+    }
+    return E >= default_ec<T>() ? default_ec<T>() : 4;
+}
 
 template <class T>
 size_t fft_smem_bytes(int logR, int ec)
@@ -47,7 +60,7 @@ size_t fft_smem_bytes(int logR, int ec)
 }
 
 template <class T>
-int ec_index(int ec) { return ec == default_ec<T>() ? 0 : 1; }
+int ec_index(int ec) { return ec == default_ec<T>() ? 0 : (ec == 4 ? 1 : 2); }
 
 // Radix plan: one pass up to 2^10, else two passes of sizes 2^ceil(l/2), 2^floor(l/2).
 inline int fft_plan(int logM, int *logRs)
@@ -86,13 +99,13 @@ cudaError_t fft_build(const FftSrc &src, const FftDst &dst, int64_t M, int E, in
     if (((int64_t)1 << logM) != M || logM > 20 || logM + 1 > tw_log) return cudaErrorInvalidValue;
     bool ec4 = false;
     ps.np = fft_plan_apply(logM, seg ? -1 : plan, ps.logR, &ec4);
-    const int ec = seg ? default_ec<T>() : (ec4 ? 4 : pick_ec<T>(E));
-    ps.ec = ec;
     const int sld = E;  // scratch row length (complex elements)
     int logNs = 0;
     for (int k = 0; k < ps.np; ++k) {
         FftArgs &a = ps.a[k];
         a = FftArgs{};
+        const int ec = seg ? default_ec<T>() : (ec4 ? 4 : pick_ec<T>(E, ps.logR[k], M >> ps.logR[k]));
+        ps.ec[k] = ec;
         a.M = M;
         a.logR = ps.logR[k];
         a.logNs = logNs;
@@ -133,7 +146,7 @@ cudaError_t fft_build(const FftSrc &src, const FftDst &dst, int64_t M, int E, in
         // FFT 67.9 -> 66.6 ms against the other order, FP32 unchanged);
         // nrow = M / R <= 2^10 in every plan
         ps.nrow[k] = (unsigned)(M >> a.logR);
-        ps.nchunk = (unsigned)((E + ec - 1) / ec);
+        ps.nchunk[k] = (unsigned)((E + ec - 1) / ec);
         double rd, wr;
         if (a.src_mode == SRC_REAL64) rd = (double)std::min<int64_t>(a.src_nvalid, 2 * M) * E * 8.0;
         else if (a.src_mode == SRC_REAL32) rd = (double)std::min<int64_t>(a.src_nvalid, 2 * M) * E * 4.0;
@@ -158,9 +171,16 @@ cudaError_t fft_run(const FftSrc &src, const FftDst &dst, int64_t M, int E, int 
     cudaError_t e = fft_build<T>(src, dst, M, E, dir, scratch, tw, tw_log, plan, false, ps);
     if (e != cudaSuccess) return e;
     for (int k = 0; k < ps.np; ++k) {
-        const FftEntry &kn = fft_table<T>()[ec_index<T>(ps.ec)][ps.logR[k]];
+        const FftEntry &kn = fft_table<T>()[ec_index<T>(ps.ec[k])][ps.logR[k]];
+        const dim3 grid(ps.nchunk[k], ps.nrow[k]);
+        const size_t smem = fft_smem_bytes<T>(ps.logR[k], ps.ec[k]);
         mrc_prof_pre(kclass_fft<T>(), st);
-        kn.fn<<<dim3(ps.nchunk, ps.nrow[k]), kn.nt, fft_smem_bytes<T>(ps.logR[k], ps.ec), st>>>(ps.a[k]);
+        if (std::is_same<T, double>::value && grid.x * grid.y <= MRC_OVERLAP_CTAS) {
+            ps.a[k].pdl = 1;
+            if ((e = mrc_launch_overlapped(kn.fn, grid, kn.nt, smem, st, ps.a[k])) != cudaSuccess) return e;
+        } else {
+            kn.fn<<<grid, kn.nt, smem, st>>>(ps.a[k]);
+        }
         mrc_prof_post(kclass_fft<T>(), st, ps.bytes[k], ps.flops[k]);
     }
     return cudaGetLastError();
@@ -303,8 +323,9 @@ template <class T>
 cudaError_t init_run()
 {
     const auto &t = fft_table<T>();
-    for (int i = 0; i < 2; ++i)
+    for (int i = 0; i < 3; ++i)
         for (int l = 0; l < 11; ++l) {
+            if (!t[i][l].fn) continue;
             cudaError_t e = cudaFuncSetAttribute(t[i][l].fn, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
             if (e != cudaSuccess) return e;
         }
@@ -326,7 +347,7 @@ cudaError_t init_run()
     void mrc_fft_fill_##SUF##_lo(FftEntry (*t)[11], FftSegEntry *ts);                                       \
     void mrc_fft_fill_##SUF##_hi(FftEntry (*t)[11], FftSegEntry *ts);                                       \
     struct FftTables_##SUF {                                                                                \
-        FftEntry t[2][11];                                                                                  \
+        FftEntry t[3][11] = {};                                                                                \
         FftSegEntry ts[11];                                                                                 \
         FftTables_##SUF()                                                                                   \
         {                                                                                                   \
@@ -340,7 +361,7 @@ cudaError_t init_run()
         return tb;                                                                                          \
     }                                                                                                       \
     template <>                                                                                             \
-    const FftEntry (&fft_table<T>())[2][11] { return fft_tables_##SUF().t; }                                \
+    const FftEntry (&fft_table<T>())[3][11] { return fft_tables_##SUF().t; }                                \
     template <>                                                                                             \
     const FftSegEntry (&fft_seg_table<T>())[11] { return fft_tables_##SUF().ts; }                           \
     cudaError_t mrc_fft_build_##SUF(const FftSrc &src, const FftDst &dst, int64_t M, int E, int dir,          \

@@ -40,6 +40,7 @@ struct FftArgs {
     int dst_eye_d;          // REAL64*: if > 0 add 1 to the diagonal of real row 0 (d = this)
     void *dst2;             // double-float DST_CPLX only: also write the hi parts here as FP32 complex (or null)
     const void *dst_base;   // DST_REAL64_BASE32: binary32 rows added to the result
+    int pdl;            // launched beside its predecessor's end (launch_overlapped)
     int src_off32, dst_off32; // every source / destination element offset of the pass fits 32 bits
 };
 
@@ -122,6 +123,34 @@ struct CvtArgs {
 };
 #define MRC_CVT_CHUNK 8192  // elements per CTA of the segmented conversion
 
+// Programmatic dependent launch: a kernel launched with mrc_launch_overlapped
+// may start while its predecessor in the stream ends; overlap_wait() returns
+// once the predecessor is complete and its writes are visible (at once in a
+// kernel launched normally), overlap_release() lets the successor start.
+#ifdef __CUDACC__
+__device__ __forceinline__ void overlap_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void overlap_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+template <class K, class A>
+cudaError_t mrc_launch_overlapped(K kernel, dim3 grid, unsigned block, size_t smem, cudaStream_t st, const A &args)
+{
+    cudaLaunchConfig_t cfg{};
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, args);
+}
+#endif
+// CTAs of a launch up to which it is worth it: above two CTAs per SM the launch
+// gap is lost in the kernel, and CTAs that wait would hold the SMs of other
+// streams' kernels
+#define MRC_OVERLAP_CTAS 304
+
 // The passes of one transform (at most two): argument blocks, radices, the
 // algorithmic charge of each, and the launch shape (nchunk entry chunks of ec
 // entries x nrow rows per pass)
@@ -130,8 +159,8 @@ struct FftPasses {
     int logR[2];
     FftArgs a[2];
     double bytes[2], flops[2];
-    unsigned nchunk, nrow[2];
-    int ec;
+    unsigned nchunk[2], nrow[2];
+    int ec[2];
 };
 
 // elements of FFT scratch a transform of M points over E entries needs
@@ -280,6 +309,8 @@ cudaError_t mrc_seed(const SegParams<SeedArgs> &P, cudaStream_t st);
 
 // misc.cu
 cudaError_t mrc_base_case(const double *A, double *psi, int d, int64_t m0, cudaStream_t st);
+// an empty kernel, launched normally
+cudaError_t mrc_order(cudaStream_t st);
 cudaError_t mrc_row_sums(const double *q, double *rs, int d, int64_t N, cudaStream_t st);
 // x(k) <- offset + scale sum_{l <= k} x(l) down the rows (scale = +-1);
 // work: mrc_scan_bytes(N, ncol)

@@ -36,6 +36,14 @@ constexpr int NT = 128;
 __device__ __forceinline__ int top_for(int m) { return m <= 4 ? 58 : (m <= 31 ? 57 : 56); }
 constexpr int SMEM_MAX = 200 * 1024;
 
+// t / d for t, d < 2^16 by a multiplication (a division by a run-time number
+// takes some 25 instructions, and every entry and output is indexed by three)
+struct FastDiv {
+    unsigned m, d;
+    __device__ __forceinline__ explicit FastDiv(int d_) : m(0xffffffffu / (unsigned)d_ + 1u), d((unsigned)d_) {}
+    __device__ __forceinline__ int div(int t) const { return d == 1u ? t : (int)__umulhi((unsigned)t, m); }
+};
+
 // accumulators of one complex sum: 2^60 h + 2^30 m + l
 struct acc {
     long long hr, hi, mr, mi, lr, li;
@@ -83,12 +91,16 @@ __device__ __forceinline__ void pairq_body(const PairArgs &a, int64_t p0)
     const int64_t M = a.M;
     const int tws = a.tw_log - a.logM - 1;
     const int tid = threadIdx.x, top = top_for(m);
+    const FastDiv dex2(ex2), dm(m), dc(c), dEC(EC);
 
     for (int t = tid; t < np * (r + c); t += NT) bnd[t] = 0u;
+    for (int t = tid; t < np; t += NT) stw[t] = q_twiddle(tw[(p0 + t) << tws], 0, false);
+    overlap_release();
+    overlap_wait();
     __syncthreads();
     // raw spectra of both rows of every pair, and the row and column bounds
     for (int t = tid; t < np * ex2; t += NT) {
-        const int q = t / ex2, e = t - q * ex2;
+        const int q = dex2.div(t), e = t - q * ex2;
         const int64_t f = p0 + q, g = (M - f) & (M - 1);
         const bool x = e < EX;
         const int ee = x ? e : e - EX;
@@ -96,24 +108,23 @@ __device__ __forceinline__ void pairq_body(const PairArgs &a, int64_t p0)
         reinterpret_cast<cx<double> *>(sf)[t] = za;
         reinterpret_cast<cx<double> *>(sg)[t] = zb;
         const unsigned b = max(max(q_magnitude(za.re), q_magnitude(za.im)), max(q_magnitude(zb.re), q_magnitude(zb.im)));
-        atomicMax(&bnd[q * (r + c) + (x ? ee / m : r + ee % c)], b);
+        atomicMax(&bnd[q * (r + c) + (x ? dm.div(ee) : r + ee - dc.div(ee) * c)], b);
     }
-    for (int t = tid; t < np; t += NT) stw[t] = q_twiddle(tw[(p0 + t) << tws], 0, false);
     __syncthreads();
     // the split of both frequencies, in place (every thread its own entries)
     for (int t = tid; t < np * ex2; t += NT) {
-        const int q = t / ex2, e = t - q * ex2;
+        const int q = dex2.div(t), e = t - q * ex2;
         const bool x = e < EX;
         const int ee = x ? e : e - EX;
         cx<q64> s, u;
         q_split(reinterpret_cast<cx<double> *>(sf)[t], reinterpret_cast<cx<double> *>(sg)[t], stw[q],
-                q_align(bnd[q * (r + c) + (x ? ee / m : r + ee % c)]), top, s, u);
+                q_align(bnd[q * (r + c) + (x ? dm.div(ee) : r + ee - dc.div(ee) * c)]), top, s, u);
         sf[t] = q_limbs(c_add(s, u));
         sg[t] = q_limbs({{s.re.v - u.re.v}, {u.im.v - s.im.v}});
     }
     __syncthreads();
     for (int t = tid; t < np * EC; t += NT) {
-        const int q = t / EC, e = t - q * EC, i = e / c, j = e - i * c;
+        const int q = dEC.div(t), e = t - q * EC, i = dc.div(e), j = e - i * c;
         const int xo = q * ex2 + i * m, yo = q * ex2 + EX + j;
         acc af{}, ag{};
         for (int k0 = 0; k0 < m; k0 += 8) {
@@ -236,7 +247,14 @@ cudaError_t mrc_pairq(const PairArgs &a0, int kclass, cudaStream_t st)
     a.pp = mrc_pairq_pp(a.npairs, a.r, a.m, a.c);
     const double by = (double)a.M * ((double)a.r * a.m + (double)a.m * a.c + (double)a.r * a.c) * 16.0;
     mrc_prof_pre(kclass, st);
-    pairq_kernel<<<(unsigned)((a.npairs + a.pp - 1) / a.pp), NT, a.pp * pair_bytes(a.r, a.m, a.c), st>>>(a);
+    const unsigned grid = (unsigned)((a.npairs + a.pp - 1) / a.pp);
+    const size_t smem = a.pp * pair_bytes(a.r, a.m, a.c);
+    if (grid <= MRC_OVERLAP_CTAS) {
+        const cudaError_t e = mrc_launch_overlapped(pairq_kernel, dim3(grid), NT, smem, st, a);
+        if (e != cudaSuccess) return e;
+    } else {
+        pairq_kernel<<<grid, NT, smem, st>>>(a);
+    }
     mrc_prof_post(kclass, st, by, 8.0 * a.r * a.m * a.c * (double)(a.M + 1));
     return cudaGetLastError();
 }

@@ -331,8 +331,8 @@ int cluster_size()
 } // namespace
 
 // The first coefficients, by powers of two: while a level's direct sums (1.5
-// m^2 d^3 multiply-adds, 1.9 per clock and SM, 16 SMs) take less than the seven
-// launches of a level by FFT (about 30 us); two for d > 32 (psi(1) by
+// m^2 d^3 multiply-adds, 1.9 per clock and SM, 16 SMs: 13 us for 8e5) take less
+// than the seven launches of a level by FFT (about 30 us); two for d > 32 (psi(1) by
 // base_case_kernel).  The mixed path's FP32 levels start after 32, 8 or 2: their
 // rounding decides its last digits, and stays what it was.
 int64_t mrc_base_size(int d, int64_t N, bool f32)
@@ -340,7 +340,7 @@ int64_t mrc_base_size(int d, int64_t N, bool f32)
     int64_t m0 = 2;
     if (f32) m0 = d <= 8 ? 32 : (d <= 32 ? 8 : 2);
     else if (d <= DSMALL)
-        while (m0 < 256 && 1.5 * (double)(m0 * m0) * d * d * d <= 1.6e6) m0 *= 2;
+        while (m0 < 256 && 1.5 * (double)(m0 * m0) * d * d * d <= 8e5) m0 *= 2;
     return std::min<int64_t>(m0, N);
 }
 
