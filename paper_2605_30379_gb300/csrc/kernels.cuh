@@ -21,7 +21,6 @@
 
 #include "arith.cuh"
 #include "mrc_internal.h"
-#include "q64.cuh"
 
 // ---------------------------------------------------------------------------
 // FFT pass: one radix-R Stockham step of a length-M transform (R = 2^logR,
@@ -34,27 +33,11 @@
 // natural frequency order.  The global loads and stores of a pass are in
 // fft_gather and fft_stage's store_global below.
 
-// The in-CTA arithmetic of a pass: FP64 points are transformed as 64-bit
-// fixed-point numbers (q64.cuh), the others in their own precision.
-template <class T>
-struct FftC {
-    using C = T;
-    using W = cx<T>;
-    static constexpr bool Q = false;
-};
-template <>
-struct FftC<double> {
-    using C = q64;
-    using W = qtw;
-    static constexpr bool Q = true;
-};
-
 // multiply by the (signed power of two) output scale in the working precision
-// (FP64: the scale is already in the exponent the fixed-point result got)
 template <class T>
 __device__ __forceinline__ cx<T> scale_out(const FftArgs &a, cx<T> v)
 {
-    if constexpr (FftC<T>::Q) return v;
+    if constexpr (sizeof(T) == 8 && sizeof(cx<T>) == 16 && !__is_same(T, dd)) return c_scal(v, a.dst_scale);
     else return {Ar<T>::scal_f(v.re, a.dst_scale_f), Ar<T>::scal_f(v.im, a.dst_scale_f)};
 }
 
@@ -163,19 +146,6 @@ constexpr int fft_default_ec() { return sizeof(cx<T>) == 8 ? MRC_F32_EC : MRC_DD
 #define MRC_FFT32_NTMAX 1024
 #endif
 
-// Resident threads per SM that the passes of at most 8 points per thread are
-// compiled for (0: off).  FP32: 2048 (32 registers, a 40-byte spill): the
-// passes are latency-bound at full occupancy instead of 75 %, FP32 FFT
-// 89.5 -> 83.5 ms at d = 64, N = 2^18.  FP64 (fixed-point stages): 1024 (64
-// registers).  Not for the double-float passes: there an explicit minimum,
-// even of 1, raised ptxas's register choice from 64 to 96-109.
-#ifndef MRC_FFT32_MINB
-#define MRC_FFT32_MINB 4  // x 512 threads
-#endif
-#ifndef MRC_FFT64_MINT
-#define MRC_FFT64_MINT 1024
-#endif
-
 // Compile-time plan of one pass: R = 2^LOGR points split into in-CTA stages
 // of radix 2^FIRST then 8, 8, ...; EC entries per CTA; NT threads, each
 // holding EPT points in registers.
@@ -186,13 +156,10 @@ struct FftPlan {
     static constexpr int NSTAGE = (LOGR < 3) ? 1 : 1 + (LOGR - FIRST) / 3;
     static constexpr int LRMAX = (LOGR < 3) ? LOGR : 3;
     static constexpr int UNITS = (R >> LRMAX) * EC;        // butterflies in a max-radix stage
-    static constexpr int NTMAX = (sizeof(cx<T>) == 8) ? MRC_FFT32_NTMAX : (FftC<T>::Q ? 1024 : 512);
+    static constexpr int NTMAX = (sizeof(cx<T>) == 8) ? MRC_FFT32_NTMAX : 512;
     static constexpr int UB = UNITS > NTMAX ? UNITS / NTMAX : 1;
     static constexpr int NT = UNITS / UB;
     static constexpr int EPT = UB << LRMAX;               // points per thread
-    // resident CTAs per SM asked of the compiler (0: none), see fft_pass_kernel_mb
-    static constexpr int MINB = EPT > 8 ? 0 : (FftC<T>::Q ? MRC_FFT64_MINT / NT
-                                                          : (sizeof(cx<T>) == 8 ? MRC_FFT32_MINB * 512 / NT : 0));
     static constexpr int LEC = EC == 1 ? 0 : EC == 2 ? 1 : EC == 4 ? 2 : EC == 8 ? 3 : 4;
 };
 
@@ -245,8 +212,7 @@ __device__ __forceinline__ void fft_gather(const FftArgs &a, cx<T> *x, int64_t j
                 const double x1 = (live && 2 * k + 1 < nv) ? base[o + (Off)ld] : 0.0;
                 v = c_from_d<T>(x0, x1);
             }
-            if constexpr (FftC<T>::Q) x[u * r + q] = v;  // the sign joins in the decoding
-            else x[u * r + q] = a.src_neg ? c_neg(v) : v;
+            x[u * r + q] = a.src_neg ? c_neg(v) : v;
         }
     }
 }
@@ -262,18 +228,11 @@ __device__ __forceinline__ void fft_gather_any(const FftArgs &a, cx<T> *x, int64
 // global memory by fft_gather before the CTA filled its twiddle tables, so
 // that both latencies overlap) and applies the inter-pass twiddles of spt;
 // later stages read the previous stage's output from sm.
-// FP64: ex is the biased exponent this thread's entry column is aligned to, and
-// sor[S][e] the union of the magnitude bits (high words) stage S leaves in
-// column e: the next stage shifts by what its own growth needs.
 template <class T, int LOGR, int EC, int S, bool INV>
-__device__ __forceinline__ void fft_stage(const FftArgs &a, cx<typename FftC<T>::C> *sm, const typename FftC<T>::W *stw,
-                                          const typename FftC<T>::W *spt, int e0, int ecount, int64_t base_out,
-                                          const cx<T> *pre, [[maybe_unused]] int &ex,
-                                          [[maybe_unused]] unsigned *sor)
+__device__ __forceinline__ void fft_stage(const FftArgs &a, cx<T> *sm, const cx<T> *stw, const cx<T> *spt,
+                                          int e0, int ecount, int64_t base_out, const cx<T> *pre)
 {
     using P = FftPlan<T, LOGR, EC>;
-    using C = typename FftC<T>::C;
-    constexpr bool QF = FftC<T>::Q;
     constexpr int R = P::R, NT = P::NT;
     constexpr int LR = (S == 0) ? P::FIRST : 3;
     constexpr int r = 1 << LR;
@@ -282,7 +241,7 @@ __device__ __forceinline__ void fft_stage(const FftArgs &a, cx<typename FftC<T>:
     constexpr int UPT = P::EPT / r;
     constexpr bool FIRST = (S == 0), LAST = (S == P::NSTAGE - 1);
     const int tid = threadIdx.x;
-    cx<C> v[UPT][r];
+    cx<T> v[UPT][r];
 #pragma unroll
     for (int u = 0; u < UPT; ++u) {
         const int unit = tid + u * NT;
@@ -290,14 +249,7 @@ __device__ __forceinline__ void fft_stage(const FftArgs &a, cx<typename FftC<T>:
 #pragma unroll
         for (int q = 0; q < r; ++q) {
             const int rho = b + q * (R / r);
-            if constexpr (FIRST && QF) {
-                // with inter-pass twiddles (stored as w / r) the points come in at
-                // 2^60, else already divided by the first radix
-                const cx<T> x = pre[u * r + q];
-                const int top = a.Ns > 1 ? Q_TOP : Q_TOP - LR, neg = a.src_neg ? -1 : 0;
-                v[u][q] = {q_decode(x.re, ex, top, neg), q_decode(x.im, ex, top, neg)};
-                if (a.Ns > 1) v[u][q] = c_mul(v[u][q], spt[rho]);
-            } else if constexpr (FIRST) {
+            if constexpr (FIRST) {
                 cx<T> x = pre[u * r + q];
                 if (a.Ns > 1) x = c_mul(x, spt[rho]);
                 v[u][q] = x;
@@ -306,54 +258,16 @@ __device__ __forceinline__ void fft_stage(const FftArgs &a, cx<typename FftC<T>:
             }
         }
     }
-    // FP64: the shift that leaves this stage its growth (|re|, |im| of its inputs
-    // below 2^57, 2^59 in the last stage, whose outputs meet no more products)
-    [[maybe_unused]] int qs = 0;
-    [[maybe_unused]] long long qc = 0;
-    if constexpr (!FIRST && QF) {
-        qs = max(0, 64 - __clz((int)sor[(S - 1) * EC + (tid & (EC - 1))]) - (LAST ? Q_TOP - 1 : Q_TOP - 3));
-        qc = q_round_start(qs);
-        ex += qs;
-    }
     if (!FIRST) __syncthreads();  // every read of sm done before the in-place writes
 #pragma unroll
     for (int u = 0; u < UPT; ++u) {
-        [[maybe_unused]] const int b = (tid + u * NT) >> P::LEC;
+        const int b = (tid + u * NT) >> P::LEC;
         if constexpr (Ns > 1) {
             const int bm = b & (Ns - 1);
-            if constexpr (QF) {
-                v[u][0] = {{q_shift_even(v[u][0].re.v, qs)}, {q_shift_even(v[u][0].im.v, qs)}};
 #pragma unroll
-                for (int q = 1; q < r; ++q)
-                    v[u][q] = q_shift(c_mul(v[u][q], stw[(bm * q) << (LOGR - LNS - LR)], qc), qs);
-            } else {
-#pragma unroll
-                for (int q = 1; q < r; ++q) v[u][q] = c_mul(v[u][q], stw[(bm * q) << (LOGR - LNS - LR)]);
-            }
+            for (int q = 1; q < r; ++q) v[u][q] = c_mul(v[u][q], stw[(bm * q) << (LOGR - LNS - LR)]);
         }
-        dft_r<C, INV, LR, LAST>(v[u]);
-    }
-    // FP64: back to floating point; the exponent takes the alignment, the
-    // stages' divisions and the output scale (a signed power of two)
-    cx<T> y[LAST ? UPT : 1][r];
-    if constexpr (LAST && QF) {
-        const unsigned hs = (unsigned)__double2hiint(a.dst_scale), sgn = hs & 0x80000000u;
-        const int eb = ex + P::FIRST + 4 + (int)((hs >> 20) & 0x7ffu) - 1023;
-#pragma unroll
-        for (int u = 0; u < UPT; ++u)
-#pragma unroll
-            for (int q = 0; q < r; ++q) {
-                y[u][q] = {q_encode(v[u][q].re, eb, sgn), q_encode(v[u][q].im, eb, sgn)};
-                if (ex >= Q_NONFINITE) {  // an Inf or NaN among the column's points
-                    y[u][q].re = __longlong_as_double(0x7ff8000000000000ll);
-                    y[u][q].im = y[u][q].re;
-                }
-            }
-    } else if constexpr (LAST) {
-#pragma unroll
-        for (int u = 0; u < UPT; ++u)
-#pragma unroll
-            for (int q = 0; q < r; ++q) y[u][q] = v[u][q];
+        dft_r<T, INV, LR, LAST>(v[u]);
     }
     // Output point q of unit u goes to row k = k0 + q Ns a.Ns.  Complex rows
     // sit at k ld + e; the real rows 2k + h (kept in the window [lo, hi)) at
@@ -376,12 +290,12 @@ __device__ __forceinline__ void fft_stage(const FftArgs &a, cx<typename FftC<T>:
                 const Off o0 = (Off)(k0 * ld + e), dq = (Off)(kst * ld);
 #pragma unroll
                 for (int q = 0; q < r; ++q) {
-                    cx<T> z = y[u][q];
-                    if (!QF && a.dst_scaled) z = scale_out(a, z);
-                    d[o0 + (Off)q * dq] = z;
+                    cx<T> y = v[u][q];
+                    if (a.dst_scaled) y = scale_out(a, y);
+                    d[o0 + (Off)q * dq] = y;
                     if constexpr (__is_same(T, dd))
                         if (a.dst2)
-                            (reinterpret_cast<cx<float> *>(a.dst2) + e0)[o0 + (Off)q * dq] = {z.re.hi, z.im.hi};
+                            (reinterpret_cast<cx<float> *>(a.dst2) + e0)[o0 + (Off)q * dq] = {y.re.hi, y.im.hi};
                 }
             } else {
                 const int lo = (int)a.dst_lo, hi = (int)a.dst_hi;
@@ -389,8 +303,8 @@ __device__ __forceinline__ void fft_stage(const FftArgs &a, cx<typename FftC<T>:
                 const bool eye_e = a.dst_eye_d > 0 && (e0 + e) % (a.dst_eye_d + 1) == 0;
 #pragma unroll
                 for (int q = 0; q < r; ++q) {
-                    const cx<T> z2 = scale_out(a, y[u][q]);
-                    const T vals[2] = {z2.re, z2.im};
+                    const cx<T> y = scale_out(a, v[u][q]);
+                    const T vals[2] = {y.re, y.im};
                     const int r0 = (int)(k0 + q * kst) * 2;
 #pragma unroll
                     for (int h = 0; h < 2; ++h) {
@@ -434,17 +348,6 @@ __device__ __forceinline__ void fft_stage(const FftArgs &a, cx<typename FftC<T>:
 #pragma unroll
             for (int q = 0; q < r; ++q) sm[(ob + q * Ns) * EC + e] = v[u][q];
         }
-        if constexpr (QF) {  // magnitude bits of this thread's points (all of one column)
-            unsigned m = 0;
-#pragma unroll
-            for (int u = 0; u < UPT; ++u)
-#pragma unroll
-                for (int q = 0; q < r; ++q) m |= q_bits(v[u][q].re) | q_bits(v[u][q].im);
-            constexpr int NL = NT < 32 ? NT : 32;
-#pragma unroll
-            for (int o = EC; o < NL; o <<= 1) m |= __shfl_xor_sync(NL == 32 ? 0xffffffffu : (1u << (NL & 31)) - 1u, m, o);
-            if ((tid & 31) < EC) atomicOr(&sor[S * EC + (tid & (EC - 1))], m);
-        }
         __syncthreads();
     }
 }
@@ -454,75 +357,37 @@ __device__ __forceinline__ void fft_pass_body(const FftArgs &a, int64_t j, int e
 {
     using P = FftPlan<T, LOGR, EC>;
     constexpr int R = P::R;
-    using C = typename FftC<T>::C;
-    using W = typename FftC<T>::W;
-    constexpr bool QF = FftC<T>::Q;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    cx<C> *sm = reinterpret_cast<cx<C> *>(smem_raw);  // [R][EC]
-    W *stw = reinterpret_cast<W *>(sm + R * EC);      // [R]  W_R^t
-    W *spt = stw + R;                                 // [R]  inter-pass twiddles
-    __shared__ int sexp[QF ? EC : 1];                 // FP64: largest exponent per entry
-    __shared__ unsigned sor[QF ? 3 * EC : 1];         // FP64: magnitude bits per stage and entry
+    cx<T> *sm = reinterpret_cast<cx<T> *>(smem_raw);  // [R][EC]
+    cx<T> *stw = sm + R * EC;                         // [R]  W_R^t
+    cx<T> *spt = stw + R;                             // [R]  inter-pass twiddles
     const cx<T> *tw = reinterpret_cast<const cx<T> *>(a.tw);
     const int tid = threadIdx.x;
     const int ecount = min(EC, a.E - e0);
     const int64_t jm = j & (a.Ns - 1);
-    // table entry of w (fixed point: divided by 2^s, the radix of the stage that applies it)
-    auto table = [&](cx<T> w, [[maybe_unused]] int s) -> W {
-        if constexpr (QF) return q_twiddle(w, s, INV);
-        else return INV ? c_conj(w) : w;
-    };
-    auto fill = [&]() {
-        if constexpr (P::NSTAGE > 1)
-            for (int t = tid; t < R; t += P::NT) stw[t] = table(tw[(int64_t)t << (a.tw_log - LOGR)], 0);
-        if (a.Ns > 1) {
-            const int sh = a.tw_log - (a.logNs + LOGR);
-            for (int t = tid; t < R; t += P::NT) spt[t] = table(tw[(jm * t) << sh], P::FIRST);
-        }
-    };
-    // beside its predecessor's end a small FP64 launch fills its twiddle tables;
-    // otherwise the first-stage global loads go first (both latencies overlap).
-    // (The FP32 and double-float passes have no such branch: it cost the large
-    // ones 0.5 %.)
-    if constexpr (QF) {
-        if (a.pdl) {
-            overlap_release();
-            fill();
-        }
-        overlap_wait();
-    }
+    // first-stage global loads before the twiddle tables are filled (both latencies overlap)
     cx<T> pre[P::EPT];
     if (a.src_mode == SRC_CPLX) fft_gather_any<T, LOGR, EC, SRC_CPLX>(a, pre, j, e0, ecount);
     else if (a.src_mode == SRC_REAL32) fft_gather_any<T, LOGR, EC, SRC_REAL32>(a, pre, j, e0, ecount);
     else fft_gather_any<T, LOGR, EC, SRC_REAL64>(a, pre, j, e0, ecount);
-    if constexpr (QF)
-        for (int t = tid; t < 3 * EC; t += P::NT) {
-            sor[t] = 0u;
-            if (t < EC) sexp[t] = Q_EXMIN;
+    if constexpr (P::NSTAGE > 1)
+        for (int t = tid; t < R; t += P::NT) {
+            cx<T> w = tw[(int64_t)t << (a.tw_log - LOGR)];
+            stw[t] = INV ? c_conj(w) : w;
         }
-    if (!QF || !a.pdl) fill();
-    __syncthreads();
-    int ex = 0;
-    if constexpr (QF) {
-        // the entry's largest exponent over the CTA's R points (a thread's points
-        // share their entry: NT is a multiple of EC or the CTA one unit per thread)
-        int m = 0;
-#pragma unroll
-        for (int q = 0; q < P::EPT; ++q) m = max(m, max(q_exponent(pre[q].re), q_exponent(pre[q].im)));
-        constexpr int NL = P::NT < 32 ? P::NT : 32;  // lanes of a warp in use
-        constexpr unsigned mask = NL == 32 ? 0xffffffffu : (1u << (NL & 31)) - 1u;
-#pragma unroll
-        for (int o = EC; o < NL; o <<= 1) m = max(m, __shfl_xor_sync(mask, m, o));
-        if ((tid & 31) < EC) atomicMax(&sexp[tid & (EC - 1)], m);
-        __syncthreads();
-        ex = sexp[tid & (EC - 1)];
-        if (ex == 2047) ex = Q_NONFINITE;
+    if (a.Ns > 1) {
+        const int sh = a.tw_log - (a.logNs + LOGR);
+        for (int t = tid; t < R; t += P::NT) {
+            cx<T> w = tw[(jm * t) << sh];
+            spt[t] = INV ? c_conj(w) : w;
+        }
     }
+    __syncthreads();
     const int64_t base_out = (j >> a.logNs << (a.logNs + LOGR)) + jm;
-    fft_stage<T, LOGR, EC, 0, INV>(a, sm, stw, spt, e0, ecount, base_out, pre, ex, sor);
-    if constexpr (P::NSTAGE > 1) fft_stage<T, LOGR, EC, 1, INV>(a, sm, stw, spt, e0, ecount, base_out, nullptr, ex, sor);
-    if constexpr (P::NSTAGE > 2) fft_stage<T, LOGR, EC, 2, INV>(a, sm, stw, spt, e0, ecount, base_out, nullptr, ex, sor);
-    if constexpr (P::NSTAGE > 3) fft_stage<T, LOGR, EC, 3, INV>(a, sm, stw, spt, e0, ecount, base_out, nullptr, ex, sor);
+    fft_stage<T, LOGR, EC, 0, INV>(a, sm, stw, spt, e0, ecount, base_out, pre);
+    if constexpr (P::NSTAGE > 1) fft_stage<T, LOGR, EC, 1, INV>(a, sm, stw, spt, e0, ecount, base_out, nullptr);
+    if constexpr (P::NSTAGE > 2) fft_stage<T, LOGR, EC, 2, INV>(a, sm, stw, spt, e0, ecount, base_out, nullptr);
+    if constexpr (P::NSTAGE > 3) fft_stage<T, LOGR, EC, 3, INV>(a, sm, stw, spt, e0, ecount, base_out, nullptr);
 }
 
 // One Stockham pass of radix R = 2^LOGR over EC entries per CTA.
@@ -537,10 +402,19 @@ __global__ void __launch_bounds__(FftPlan<T, LOGR, EC>::NT) fft_pass_kernel(FftA
     else fft_pass_body<T, LOGR, EC, false>(a, blockIdx.y, blockIdx.x * EC);
 }
 
-// The same pass with a minimum of resident CTAs per SM (FftPlan::MINB), used
-// for the FP32 and FP64 passes of at most 8 points per thread.
+// The same pass with a minimum of resident CTAs per SM (MRC_FFT32_MINB x 512
+// threads; 0 at build time = off), used for the FP32 passes of at most 8
+// points per thread.  With 4 (2048 threads: 32 registers, a 40-byte spill)
+// the FP32 passes are latency-bound at full occupancy instead of 75 %: FP32
+// FFT 89.5 -> 83.5 ms at d = 64, N = 2^18.  Not for the double-float passes:
+// there an explicit minimum, even of 1, raised ptxas's register choice from
+// 64 to 96-109.
+#ifndef MRC_FFT32_MINB
+#define MRC_FFT32_MINB 4
+#endif
 template <class T, int LOGR, int EC>
-__global__ void __launch_bounds__(FftPlan<T, LOGR, EC>::NT, FftPlan<T, LOGR, EC>::MINB)
+__global__ void __launch_bounds__(FftPlan<T, LOGR, EC>::NT,
+                                  MRC_FFT32_MINB > 0 ? (MRC_FFT32_MINB * 512) / FftPlan<T, LOGR, EC>::NT : 1)
     fft_pass_kernel_mb(FftArgs a)
 {
     if (a.dir > 0) fft_pass_body<T, LOGR, EC, true>(a, blockIdx.y, blockIdx.x * EC);
@@ -575,7 +449,8 @@ __global__ void __launch_bounds__(FftPlan<T, LOGR, EC>::NT) fft_seg_kernel(const
 }
 
 template <class T, int LOGR, int EC>
-__global__ void __launch_bounds__(FftPlan<T, LOGR, EC>::NT, FftPlan<T, LOGR, EC>::MINB)
+__global__ void __launch_bounds__(FftPlan<T, LOGR, EC>::NT,
+                                  MRC_FFT32_MINB > 0 ? (MRC_FFT32_MINB * 512) / FftPlan<T, LOGR, EC>::NT : 1)
     fft_seg_kernel_mb(const __grid_constant__ SegParams<FftArgs> P)
 {
     fft_seg_run<T, LOGR, EC>(P);
@@ -925,6 +800,7 @@ __global__ void twiddle_kernel(cx<T> *tw, int log)
 // Launch table of the FFT pass instantiations: entry [ec_index][logR], where
 // ec_index 0 is the default entries per CTA (MRC_F32_EC for 8-byte complex
 // values, MRC_DD_EC for 16-byte ones), 1 is 4 entries per CTA and 2 (FP64) one.
+// (The FP64 passes are in fftq.cuh.)
 using FftKernel = void (*)(FftArgs);
 struct FftEntry {
     FftKernel fn;
@@ -939,30 +815,17 @@ struct FftSegEntry {
 template <class T, int L, int EC>
 constexpr FftKernel fft_pass_or_mb()
 {
-    if constexpr (FftPlan<T, L, EC>::MINB > 0)
+    if constexpr (MRC_FFT32_MINB > 0 && sizeof(cx<T>) == 8 && FftPlan<T, L, EC>::EPT <= 8 &&
+                  FftPlan<T, L, EC>::NT <= MRC_FFT32_MINB * 512)
         return fft_pass_kernel_mb<T, L, EC>;
     else return fft_pass_kernel<T, L, EC>;
-}
-
-template <class T, int L>
-constexpr FftKernel fft_pass_ec4()
-{
-    if constexpr (FftC<T>::Q) return fft_pass_or_mb<T, L, 4>();
-    else return fft_pass_kernel<T, L, 4>;
-}
-
-// one entry per CTA, for the radices that pick_ec takes it for
-template <class T, int L>
-constexpr FftKernel fft_pass_ec1()
-{
-    if constexpr (L >= 8) return fft_pass_or_mb<T, L, 1>();
-    else return nullptr;
 }
 
 template <class T, int L, int EC>
 constexpr FftSegKernel fft_seg_or_mb()
 {
-    if constexpr (FftPlan<T, L, EC>::MINB > 0)
+    if constexpr (MRC_FFT32_MINB > 0 && sizeof(cx<T>) == 8 && FftPlan<T, L, EC>::EPT <= 8 &&
+                  FftPlan<T, L, EC>::NT <= MRC_FFT32_MINB * 512)
         return fft_seg_kernel_mb<T, L, EC>;
     else return fft_seg_kernel<T, L, EC>;
 }
@@ -973,8 +836,6 @@ void fft_fill_shifted(FftEntry (*t)[11], FftSegEntry *ts, std::integer_sequence<
 {
     constexpr int ECD = fft_default_ec<T>();
     ((t[0][OFF + L] = FftEntry{fft_pass_or_mb<T, OFF + L, ECD>(), FftPlan<T, OFF + L, ECD>::NT}), ...);
-    ((t[1][OFF + L] = FftEntry{fft_pass_ec4<T, OFF + L>(), FftPlan<T, OFF + L, 4>::NT}), ...);
-    if constexpr (FftC<T>::Q)
-        ((t[2][OFF + L] = FftEntry{fft_pass_ec1<T, OFF + L>(), FftPlan<T, OFF + L, 1>::NT}), ...);
+    ((t[1][OFF + L] = FftEntry{fft_pass_kernel<T, OFF + L, 4>, FftPlan<T, OFF + L, 4>::NT}), ...);
     ((ts[OFF + L] = FftSegEntry{fft_seg_or_mb<T, OFF + L, ECD>(), FftPlan<T, OFF + L, ECD>::NT}), ...);
 }

@@ -63,6 +63,7 @@
 // status word and a shared abort flag; all roles then leave their loops, the
 // MMA thread waits (bounded) for its MMAs in flight, and the TMEM is freed.
 #include "digits.cuh"
+#include "q64.cuh"
 #include "tcgen05.cuh"
 
 namespace {
