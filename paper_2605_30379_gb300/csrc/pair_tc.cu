@@ -7,8 +7,8 @@
 //     values, pairs s + t >= 7 (36 pairs in 8 weight groups), about 2^-58
 //     relative to the row and column maxima.  The FP64 pipe gives two
 //     multiply-adds per clock and SM; at d = 64, N = 2^15 the inverse's 28
-//     products take 17 ms here against 138 ms on it (whole inverse 159.6 ->
-//     39.2 ms), with smaller errors (Weibull d = 64, N = 512 against
+//     products take 14 ms here against 138 ms on it (whole inverse 159.6 ->
+//     32.2 ms with the later steps), with smaller errors (Weibull d = 64, N = 512 against
 //     long double: 7.9e-16 -> 5.5e-16);
 
 //   double-float (the residual product of Proposition 2.6): six balanced
@@ -43,10 +43,11 @@
 //              K chunk of 16 the real-FFT split of the packed spectra (the
 //              fused split of kernels.cuh) and the digit tiles, into a ring
 //              of NSLOT chunk slots (full / empty barriers);
-//   warp 12    (MMA): one thread issues every kept digit pair's MMAs of a
+//   MMA        one thread issues every kept digit pair's MMAs of a
 //              chunk and releases the slot with tcgen05.commit; after the
 //              last chunk it signals the epilogue;
-//   warps 8-11 (epilogue): tcgen05.ld of the group accumulators and the fold
+//   epilogue   (one or two groups of four warps): tcgen05.ld of the group
+//              accumulators and the fold
 //              (a compensated double-float sum of the top three groups for
 //              the residual product, FP32 below and for FP32), then, through
 //              a shared-memory transpose, the scaling by 2^(sigma + tau), the
@@ -92,14 +93,30 @@ constexpr int NCH = 64 / KC;          // chunks per frequency
 constexpr int SBO = (KC / 8) * 128;   // bytes between 8-row groups of a tile
 constexpr int A_TILE = 192 * KC * 2;  // bytes of one [-X_i; X_r; X_i] digit tile
 constexpr int B_TILE = 64 * KC * 2;   // bytes of one Y_r or Y_i digit tile
-// 13 warps: 8 split, 4 epilogue (TMEM lane quarters 0..3), 1 MMA; at most
-// four warps per SM sub-partition leaves each thread 128 registers
-constexpr int NSPLIT = 256, NEPI = 128;
-constexpr int WEPI0 = 8, WMMA = 12;
-constexpr int NTHREADS = 13 * 32;
-constexpr int XLD = 33;               // row length (values) of the epilogue transpose
+// Warps: 8 split, EG groups of 4 epilogue warps (one per TMEM lane quarter), 1
+// MMA.  The accumulators are single buffered, so the MMAs wait while they are
+// read.  With one group the roles of the longer FP64 and double-float
+// epilogues ran one after the other (d = 64, N = 2^14, double-float 1.92 ms:
+// 1.16 without the epilogue, 1.55 without the split); two groups of 32 columns
+// take 1.82 ms, FP64 0.53 -> 0.42 at M = 2^12.  FP32's lose by it (0.75 -> 0.77 ms at
+// N = 2^14): one group.
+constexpr int NSPLIT = 256, NGRP = 128, WEPI0 = 8;
+// Registers per thread: 128 with 13 warps.  With two groups the MMA warp is one
+// of a whole warpgroup (the other three only fill it up): 96 at launch, of which
+// it gives to the split (128 (2 120 + 2 96 + 40) = 60416 within the launch's
+// 640 x 96 = 61440); without that the split's 96 spill (FP64 0.53 -> 0.57 ms
+// instead of 0.42 at d = 64, M = 2^12).
+constexpr int SPLIT_REGS = 120, MMA_REGS = 40;
+template <class T>
+struct TcR {
+    static constexpr int EG = std::is_same<T, float>::value ? 1 : 2;
+    static constexpr int NEPI = EG * NGRP, WMMA = WEPI0 + 4 * EG;
+    static constexpr int NTHREADS = EG == 1 ? (WMMA + 1) * 32 : (WMMA + 4) * 32;
+    // columns a group folds at a time, row length (values) of its transpose
+    static constexpr int XCOL = 32 / EG, XLD = XCOL + 1;
+};
 constexpr unsigned TMEM_COLS = 512;
-constexpr int BAR_SPLIT = 1, BAR_EPI = 2;
+constexpr int BAR_SPLIT = 1, BAR_EPI = 2;  // (+ the epilogue group)
 template <class T>
 constexpr unsigned IDESC = tc_q<T> ? idesc_f16<128, 64>() : idesc_bf16<128, 64>();
 
@@ -110,7 +127,8 @@ struct TcL {
     static constexpr int SUB = S * (A_TILE + 2 * B_TILE);  // digit tiles of one frequency and chunk
     static constexpr int XT = S * A_TILE;                   // the X part of them (the sub-slot's start)
     static constexpr int SLOT = NF * SUB;
-    static constexpr int XCH = 2 * NF * 64 * XLD * (int)sizeof(T);  // [NF][C_r, C_i][64][XLD]
+    static constexpr int XGRP = 2 * NF * 64 * TcR<T>::XLD;               // [NF][C_r, C_i][64][XLD] values
+    static constexpr int XCH = TcR<T>::EG * XGRP * (int)sizeof(T);  // of each epilogue group
     static constexpr int OFF_XCH = NSLOT * SLOT;
     // Per-pair scale factors scx[i] = 2^-sigma_i, scy[j] = 2^-tau_j (the
     // split) and fx[i] = 2^(sigma_i - 1), fy[j] = 2^(tau_j - 1) (the output:
@@ -716,19 +734,29 @@ __device__ __forceinline__ void st_cx<float>(cx<float> *p, cx<float> v)
     *reinterpret_cast<float2 *>(p) = make_float2(v.re, v.im);
 }
 
-// FP64 outputs of one round of 32 columns (this thread: column j, sixteen
-// rows): the exponents of the row and column alignments join (with the factor
+// Row of an epilogue group's thread ge in its output step m.  XCOL = 16: a
+// warp covers 16 columns of rows i and i + 16 (17-value rows: 32 different banks)
+template <class T>
+__device__ __forceinline__ int epi_row(int ge, int m)
+{
+    if (TcR<T>::EG == 1) return (ge >> 5) + 4 * m;
+    return (ge >> 5) + 4 * (m & 3) + (ge & 16) + 32 * (m >> 2);
+}
+
+// FP64 outputs of one round (this thread: column j, eight rows): the
+// exponents of the row and column alignments join (with the factor
 // 1/2 of the merge and the split's 2 on both operands), then C(f) / 2 is stored
 // unmerged (phase 0) or the pair merged with it.
 __device__ __forceinline__ void epi_q(cx<double> *ZC, const double *xch, const float *fx, int ey, cx<double> wf, int64_t f,
-                                      int64_t gZ, int d, int64_t E, int j, int jl, int et, int phase, bool self, bool two)
+                                      int64_t gZ, int d, int64_t E, int j, int jl, int ge, int phase, bool self, bool two)
 {
+    constexpr int XLD = TcR<double>::XLD;
 #pragma unroll 1
-    for (int m0 = 0; m0 < 16; m0 += 4) {
+    for (int m0 = 0; m0 < 8; m0 += 4) {
         cx<double> v[4], cf[4];
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
-            const int i = (et >> 5) + 4 * (m0 + u);
+            const int i = epi_row<double>(ge, m0 + u);
             const int ex = __float_as_int(fx[i]), de = ex + ey - 2113;
             v[u] = {q_scale(xch[i * XLD + jl], de), q_scale(xch[(64 + i) * XLD + jl], de)};
             if (max(ex, ey) >= Q_NONFINITE) v[u].re = v[u].im = __longlong_as_double(0x7ff8000000000000ll);
@@ -737,7 +765,7 @@ __device__ __forceinline__ void epi_q(cx<double> *ZC, const double *xch, const f
         }
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
-            const int i = (et >> 5) + 4 * (m0 + u);
+            const int i = epi_row<double>(ge, m0 + u);
             if (i >= d || j >= d) continue;
             cx<double> *zf = ZC + f * E + (int64_t)i * d + j;
             if (!self && phase == 0) {
@@ -770,12 +798,13 @@ __device__ __forceinline__ TcW<T> split_tw(cx<T> w)
 // sweep); the split warps bulk-copy them into the slot (on xfull[slot]) and
 // split only Y.
 template <class T, int NCK, bool XPRE>
-__global__ void __launch_bounds__(NTHREADS, 1) tcp_kernel(const __grid_constant__ SegParams<PairArgs> P, int *status)
+__global__ void __launch_bounds__(TcR<T>::NTHREADS, 1) tcp_kernel(const __grid_constant__ SegParams<PairArgs> P, int *status)
 {
     using L = TcL<T>;
     constexpr int S = L::S, GMIN = L::GMIN, NG = L::NG, NSLOT = L::NSLOT, NF = L::NF;
+    constexpr int EG = TcR<T>::EG, WMMA = TcR<T>::WMMA, XCOL = TcR<T>::XCOL, XLD = TcR<T>::XLD;
     extern __shared__ __align__(1024) unsigned char smem[];
-    T *xch = reinterpret_cast<T *>(smem + L::OFF_XCH);          // [NF][C_r, C_i][64][XLD]
+    T *xchs = reinterpret_cast<T *>(smem + L::OFF_XCH);         // the groups' transposes
     float *scb = reinterpret_cast<float *>(smem + L::OFF_SC);  // [NB][scx, scy, fx, fy][64]
     unsigned *bxy = reinterpret_cast<unsigned *>(scb + 4 * 64 * L::NB);  // [2][bx, by][64]
     __shared__ __align__(8) unsigned long long bar_full[NSLOT], bar_empty[NSLOT], bar_tfull, bar_tempty, bar_done;
@@ -791,7 +820,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) tcp_kernel(const __grid_constant_
             mbar_init(smem_u32(&bar_xfull[s]), 1);
         }
         mbar_init(smem_u32(&bar_tfull), 1);
-        mbar_init(smem_u32(&bar_tempty), NEPI);
+        mbar_init(smem_u32(&bar_tempty), TcR<T>::NEPI);
         mbar_init(smem_u32(&bar_done), 1);
         abort_flag = 0;
         mbar_init_fence();
@@ -830,6 +859,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) tcp_kernel(const __grid_constant_
 
     if (warp < WEPI0) {
         // ------------------------------------------------------------ split
+        if constexpr (EG == 2) asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(SPLIT_REGS));
         // The bounds of pair p + grid are gathered during pair p's chunks, in
         // slices (their loads, first touches of those spectra, overlap the
         // digit work); the first pair's before its chunks.
@@ -956,7 +986,8 @@ __global__ void __launch_bounds__(NTHREADS, 1) tcp_kernel(const __grid_constant_
         }
     } else if (warp < WMMA) {
         // --------------------------------------------------------- epilogue
-        const int et = tid - WEPI0 * 32;
+        const int grp = (warp - WEPI0) >> 2, ge = (tid - WEPI0 * 32) & (NGRP - 1);
+        T *xch = xchs + grp * L::XGRP;
         const int q = warp & 3;  // TMEM lanes 32 q .. 32 q + 31
         int fi = 0, pl = 0;      // passes drained, pairs
         for (unsigned gp = blockIdx.x; gp < total; gp += gridDim.x, ++pl) {
@@ -974,25 +1005,27 @@ __global__ void __launch_bounds__(NTHREADS, 1) tcp_kernel(const __grid_constant_
             bool stop = false;
             for (int phase = 0; phase < np; ++phase, ++fi) {
                 bool ok = !failed && !abort_flag && mbar_wait(smem_u32(&bar_tfull), fi & 1);
-                if (bar_or(BAR_EPI, NEPI, !ok)) {
+                if (bar_or(BAR_EPI + grp, NGRP, !ok)) {
                     if (!failed) give_up();
                     stop = true;
                     break;
                 }
                 fence_after();
                 const unsigned tb = tmem + ((unsigned)(32 * q) << 16);
-                // two rounds of 32 columns: fold them into the transpose (lanes
-                // along i), release the accumulators after the second fold, then
-                // lanes along j for coalesced global accesses
+                // two rounds of XCOL columns per group: fold them into the transpose
+                // (lanes along i), release the accumulators after the second fold,
+                // then lanes along j for coalesced global accesses.  (Both rounds
+                // folded first, the second one's values held in registers: they
+                // spill, 1.82 -> 2.11 ms in double-float.)
 #pragma unroll 1
                 for (int r = 0; r < 2; ++r) {
 #pragma unroll
                     for (int fq = 0; fq < NF; ++fq) {
                         T *xr = xch + ((fq * 2 + (q >> 1)) * 64 + 32 * (q & 1) + lane) * XLD;  // C_r or C_i rows
 #pragma unroll
-                        for (int m = 0; m < 4; ++m) {
+                        for (int m = 0; m < XCOL / 8; ++m) {
                             T o8[8];
-                            fold8<T, NG>(tb + (unsigned)(fq * L::TCOLS + 32 * r + 8 * m), o8);
+                            fold8<T, NG>(tb + (unsigned)(fq * L::TCOLS + 2 * XCOL * grp + XCOL * r + 8 * m), o8);
 #pragma unroll
                             for (int c = 0; c < 8; ++c) xr[8 * m + c] = o8[c];
                         }
@@ -1001,21 +1034,21 @@ __global__ void __launch_bounds__(NTHREADS, 1) tcp_kernel(const __grid_constant_
                         fence_before();
                         mbar_arrive(smem_u32(&bar_tempty));  // accumulators read: the next MMAs may overwrite them
                     }
-                    bar_sync(BAR_EPI, NEPI);
-                    const int jl = et & 31, j = 32 * r + jl;
+                    bar_sync(BAR_EPI + grp, NGRP);
+                    const int jl = ge & (XCOL - 1), j = 2 * XCOL * grp + XCOL * r + jl;
                     [[maybe_unused]] const float sj = fy[j];
                     if constexpr (tc_q<T>) {
-                        epi_q(ZC, xch, fx, __float_as_int(sj), wf, f, gZ, d, E, j, jl, et, phase, self, two);
-                        bar_sync(BAR_EPI, NEPI);
+                        epi_q(ZC, xch, fx, __float_as_int(sj), wf, f, gZ, d, E, j, jl, ge, phase, self, two);
+                        bar_sync(BAR_EPI + grp, NGRP);
                         continue;
                     }
                     // four outputs at a time, their loads first
 #pragma unroll 1
-                    for (int m0 = 0; m0 < 16; m0 += 4) {
+                    for (int m0 = 0; m0 < 16 / EG; m0 += 4) {
                         cx<T> v[4], vg[4], cf[4];
 #pragma unroll
                         for (int u = 0; u < 4; ++u) {
-                            const int i = (et >> 5) + 4 * (m0 + u);
+                            const int i = epi_row<T>(ge, m0 + u);
                             const float s_ = fx[i] * sj;  // 2^(sigma_i + tau_j - 2), exact
                             v[u] = {mul_f(xch[i * XLD + jl], s_), mul_f(xch[(64 + i) * XLD + jl], s_)};
                             if constexpr (NF == 2)
@@ -1025,7 +1058,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) tcp_kernel(const __grid_constant_
                         }
 #pragma unroll
                         for (int u = 0; u < 4; ++u) {
-                            const int i = (et >> 5) + 4 * (m0 + u);
+                            const int i = epi_row<T>(ge, m0 + u);
                             if (i >= d || j >= d) continue;
                             cx<T> *zf = ZC + f * E + (int64_t)i * d + j;
                             if constexpr (NF == 2) {
@@ -1041,12 +1074,14 @@ __global__ void __launch_bounds__(NTHREADS, 1) tcp_kernel(const __grid_constant_
                             }
                         }
                     }
-                    bar_sync(BAR_EPI, NEPI);  // transpose read before it is rewritten
+                    bar_sync(BAR_EPI + grp, NGRP);  // transpose read before it is rewritten
                 }
             }
             if (stop) break;
         }
-    } else if (lane == 0) {  // the MMA warp's other lanes go straight to the final barrier (below)
+    } else {
+      if constexpr (EG == 2) asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(MMA_REGS));
+      if (warp == WMMA && lane == 0) {  // the other lanes go straight to the final barrier (below)
         // -------------------------------------------------------------- MMA
         int it = 0, fi = 0;
         bool issued = false;
@@ -1096,6 +1131,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) tcp_kernel(const __grid_constant_
             commit(smem_u32(&bar_done));
             if (!mbar_wait(smem_u32(&bar_done), 0)) give_up();  // every MMA finished before the TMEM is freed
         }
+      }
     }
     if (warp == WMMA) __syncwarp();  // lane 0 rejoins its warp before the CTA-wide barrier
 
@@ -1144,7 +1180,7 @@ cudaError_t tcp_launch(const SegParams<PairArgs> &P, int *status, cudaStream_t s
     if constexpr (__is_same(T, dd))
         if (P.a[0].xs) k = tcp_kernel_for<T, true>(nck);
     mrc_prof_pre(kclass, st);
-    k<<<grid, NTHREADS, TcL<T>::SMEM, st>>>(P, status);
+    k<<<grid, TcR<T>::NTHREADS, TcL<T>::SMEM, st>>>(P, status);
     mrc_prof_post(kclass, st, bytes, flops);
     return cudaGetLastError();
 }
