@@ -1610,14 +1610,14 @@ mrc_status mrc_transition(mrc_ctx *c, int d, int64_t N, const double *psi, const
     mrc_status s;
     if ((s = ensure_tw(c, p, st)) != MRC_OK) return s;
     const size_t E = (size_t)d * d;
-    size_t need = align_up(sizeof(double) * N * d) + align_up(mrc_scan_bytes(N, d)) +
-                  ws_product(pow2ceil(N), E, d, E, p);
+    // (the scan's sums lie where the product's spectra come after them)
+    const size_t sb = mrc_scan_bytes(N, d);
+    size_t need = align_up(sizeof(double) * N * d) + std::max(align_up(sb), ws_product(pow2ceil(N), E, d, E, p));
     if ((s = ensure_ws(c, need)) != MRC_OK) return s;
     Arena ar{(char *)c->ws};
     double *h = (double *)ar.take(sizeof(double) * N * d);
-    void *work = ar.take(mrc_scan_bytes(N, d));
     CK(mrc_row_sums(q, h, d, N, st));
-    CK(mrc_scan_cols(h, d, N, work, -1.0, 1.0, st));  // Hbar_j(k) = 1 - sum_{l<=k} sum_j' q_jj'(l)
+    CK(mrc_scan_cols(h, d, N, ar.base + ar.off, sb, -1.0, 1.0, st));  // Hbar_j(k) = 1 - sum_{l<=k} sum_j' q_jj'(l)
     return conv_product(c, ar, p, psi, N, h, N, d, 1, d, N, P, 1.0, 0, 0, true, st);
 }
 
@@ -1645,8 +1645,9 @@ mrc_status mrc_first_entrance(mrc_ctx *c, int d, int64_t N, const double *q, con
     if ((s = ensure_tw(c, pc, st)) != MRC_OK) return s;
     const size_t ECC = (size_t)nC * nC, ECD = (size_t)nC * nD;
     size_t fixed = align_up(sizeof(double) * N * ECC) * 2 + align_up(sizeof(double) * N * ECD) * 2 +
-                   align_up(sizeof(double) * N) * 2 + align_up(mrc_scan_bytes(N, 1));
-    size_t need = fixed + std::max(ws_inverse(nC, N, prec), ws_product(pow2ceil(N), ECC, ECD, ECD, pc));
+                   align_up(sizeof(double) * N) * 2;
+    const size_t sb = mrc_scan_bytes(N, 1);  // where the inverse's and the product's buffers were
+    size_t need = fixed + std::max({ws_inverse(nC, N, prec), ws_product(pow2ceil(N), ECC, ECD, ECD, pc), align_up(sb)});
     if ((s = ensure_ws(c, need)) != MRC_OK) return s;
     Arena ar{(char *)c->ws};
     double *ACC = (double *)ar.take(sizeof(double) * N * ECC);
@@ -1655,7 +1656,6 @@ mrc_status mrc_first_entrance(mrc_ctx *c, int d, int64_t N, const double *q, con
     double *gw = (double *)ar.take(sizeof(double) * N * ECD);
     double *Fw = (double *)ar.take(sizeof(double) * N);
     double *fk = (double *)ar.take(sizeof(double) * N);
-    void *work = ar.take(mrc_scan_bytes(N, 1));
     CK(mrc_gather_blocks(q, d, N, Ci.data(), nC, Di.data(), nD, ACC, QCD, st));
     const size_t mark = ar.off;
     s = inverse_impl(c, ar, nC, N, ACC, psiC, prec, sweeps, st);
@@ -1668,7 +1668,7 @@ mrc_status mrc_first_entrance(mrc_ctx *c, int d, int64_t N, const double *q, con
         double *Fo = F ? F : Fw;
         CK(mrc_weighted_rowsum(gout, nC, nD, N, alpha_C, fk, st));
         CK(cudaMemcpyAsync(Fo, fk, sizeof(double) * N, cudaMemcpyDeviceToDevice, st));
-        CK(mrc_scan_cols(Fo, 1, N, work, 1.0, 0.0, st));
+        CK(mrc_scan_cols(Fo, 1, N, ar.base + mark, sb, 1.0, 0.0, st));
         if (S) CK(mrc_one_minus(Fo, S, N, st));
     }
     return MRC_OK;
@@ -1765,10 +1765,12 @@ mrc_status mrc_renewal_visits(mrc_ctx *c, int d, int64_t N, const double *psi, c
     cudaStream_t st = (cudaStream_t)stream;
     cudaSetDevice(c->device);
     mrc_status s;
-    if ((s = ensure_ws(c, align_up(mrc_scan_bytes(N, 1)))) != MRC_OK) return s;
+    size_t sb = align_up(mrc_scan_bytes(N, 1));
+    if (c->cap && sb > std::max(c->cap, c->ws_size)) sb = align_up(mrc_scan_bytes_min(N, 1));
+    if ((s = ensure_ws(c, sb)) != MRC_OK) return s;
     // alpha psi(k) 1_B per k, then the running sum over k (Eq. (renewal-visits))
     CK(mrc_occupation_k(psi, d, N, alpha, inB.data(), out, st));
-    CK(mrc_scan_cols(out, 1, N, c->ws, 1.0, 0.0, st));
+    CK(mrc_scan_cols(out, 1, N, c->ws, sb, 1.0, 0.0, st));
     return MRC_OK;
 }
 

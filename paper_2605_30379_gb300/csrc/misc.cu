@@ -95,22 +95,23 @@ __global__ void row_sums_kernel(const double *__restrict__ q, double *__restrict
 }
 
 // Inclusive running sums down the rows of x [N][ncol], in three launches: the
-// sum of every chunk of SCAN_CH rows, the running sums of those, and each
+// sum of every chunk of `ch` rows, the running sums of those, and each
 // chunk's rows from its start.  A CTA covers one chunk of up to 32 columns:
-// TX columns x TY threads of SCAN_CH / TY consecutive rows each, so that the
+// TX columns x TY threads of ch / TY consecutive rows each, so that the
 // loads of a warp are consecutive whatever the column count; one thread per
 // chunk and column took 430 us for N = 2^14, ncol = 32 and 90 us for ncol = 1,
-// in chains of 1024 dependent loads.
-constexpr int SCAN_CH = 256;
+// in chains of 1024 dependent loads.  Chunks of 256 rows, doubled while the
+// scratch is smaller than their sums (a context whose workspace cap is low).
+constexpr int SCAN_CH = 256, SCAN_CH_MAX = 2048;
 
 struct ScanShape {
     int tx, ty, rows;  // columns, row groups, rows per thread of a CTA of 256
 };
-__host__ __device__ inline ScanShape scan_shape(int ncol)
+__host__ __device__ inline ScanShape scan_shape(int ncol, int ch)
 {
     int tx = 1;
     while (tx < 32 && tx < ncol) tx <<= 1;
-    return {tx, 256 / tx, SCAN_CH / (256 / tx)};
+    return {tx, 256 / tx, ch / (256 / tx)};
 }
 
 // Sums as unevaluated pairs h + l (Knuth's TwoSum): the survival function 1 -
@@ -131,13 +132,13 @@ __device__ __forceinline__ Sum2 sum2(Sum2 a, Sum2 b)
     return s;
 }
 
-__global__ void __launch_bounds__(256) scan_chunk_sums(const double *__restrict__ x, int ncol, int64_t N,
+__global__ void __launch_bounds__(256) scan_chunk_sums(const double *__restrict__ x, int ncol, int64_t N, int ch,
                                                        Sum2 *__restrict__ work)
 {
     __shared__ Sum2 part[256];
-    const ScanShape sh = scan_shape(ncol);
+    const ScanShape sh = scan_shape(ncol, ch);
     const int cx = threadIdx.x % sh.tx, ry = threadIdx.x / sh.tx, c = blockIdx.y * sh.tx + cx;
-    const int64_t k0 = (int64_t)blockIdx.x * SCAN_CH + (int64_t)ry * sh.rows;
+    const int64_t k0 = (int64_t)blockIdx.x * ch + (int64_t)ry * sh.rows;
     Sum2 s = {0.0, 0.0};
     if (c < ncol)
         for (int k = 0; k < sh.rows; ++k)
@@ -170,7 +171,7 @@ __device__ __forceinline__ Sum2 scan_groups(Sum2 v, Sum2 *part, const ScanShape 
 __global__ void __launch_bounds__(256) scan_chunk_offsets(Sum2 *work, int ncol, int64_t nch)
 {
     __shared__ Sum2 part[256];
-    const ScanShape sh = scan_shape(ncol);
+    const ScanShape sh = scan_shape(ncol, SCAN_CH);
     const int cx = threadIdx.x % sh.tx, ry = threadIdx.x / sh.tx, c = blockIdx.x * sh.tx + cx;
     Sum2 run = {0.0, 0.0};
     for (int64_t c0 = 0; c0 < nch; c0 += sh.ty) {
@@ -182,13 +183,13 @@ __global__ void __launch_bounds__(256) scan_chunk_offsets(Sum2 *work, int ncol, 
     }
 }
 
-__global__ void __launch_bounds__(256) scan_apply(double *__restrict__ x, int ncol, int64_t N,
+__global__ void __launch_bounds__(256) scan_apply(double *__restrict__ x, int ncol, int64_t N, int ch,
                                                   const Sum2 *__restrict__ work, double scale, double offset)
 {
     __shared__ Sum2 part[256];
-    const ScanShape sh = scan_shape(ncol);
+    const ScanShape sh = scan_shape(ncol, ch);
     const int cx = threadIdx.x % sh.tx, ry = threadIdx.x / sh.tx, c = blockIdx.y * sh.tx + cx;
-    const int64_t k0 = (int64_t)blockIdx.x * SCAN_CH + (int64_t)ry * sh.rows;
+    const int64_t k0 = (int64_t)blockIdx.x * ch + (int64_t)ry * sh.rows;
     const bool col = c < ncol;
     Sum2 s = {0.0, 0.0};
     if (col)
@@ -461,21 +462,27 @@ cudaError_t mrc_row_sums(const double *q, double *rs, int d, int64_t N, cudaStre
     return cudaGetLastError();
 }
 
-size_t mrc_scan_bytes(int64_t N, int ncol) { return sizeof(Sum2) * (size_t)((N + SCAN_CH - 1) / SCAN_CH) * ncol; }
+static size_t scan_bytes(int64_t N, int ncol, int ch) { return sizeof(Sum2) * (size_t)((N + ch - 1) / ch) * ncol; }
+size_t mrc_scan_bytes(int64_t N, int ncol) { return scan_bytes(N, ncol, SCAN_CH); }
+size_t mrc_scan_bytes_min(int64_t N, int ncol) { return scan_bytes(N, ncol, SCAN_CH_MAX); }
 
-cudaError_t mrc_scan_cols(double *x, int ncol, int64_t N, void *wk, double scale, double offset, cudaStream_t st)
+cudaError_t mrc_scan_cols(double *x, int ncol, int64_t N, void *wk, size_t wk_bytes, double scale, double offset,
+                          cudaStream_t st)
 {
     Sum2 *work = (Sum2 *)wk;
-    const int64_t nch = (N + SCAN_CH - 1) / SCAN_CH;
+    int ch = SCAN_CH;
+    while (ch < SCAN_CH_MAX && scan_bytes(N, ncol, ch) > wk_bytes) ch *= 2;
+    if (scan_bytes(N, ncol, ch) > wk_bytes) return cudaErrorInvalidValue;
+    const int64_t nch = (N + ch - 1) / ch;
     mrc_prof_pre(7, st);
-    const int nt = (ncol + scan_shape(ncol).tx - 1) / scan_shape(ncol).tx;
-    scan_chunk_sums<<<dim3((unsigned)nch, nt), 256, 0, st>>>(x, ncol, N, work);
+    const int tx = scan_shape(ncol, ch).tx, nt = (ncol + tx - 1) / tx;
+    scan_chunk_sums<<<dim3((unsigned)nch, nt), 256, 0, st>>>(x, ncol, N, ch, work);
     mrc_prof_post(7, st, 0, 0);
     mrc_prof_pre(7, st);
     scan_chunk_offsets<<<nt, 256, 0, st>>>(work, ncol, nch);
     mrc_prof_post(7, st, 0, 0);
     mrc_prof_pre(7, st);
-    scan_apply<<<dim3((unsigned)nch, nt), 256, 0, st>>>(x, ncol, N, work, scale, offset);
+    scan_apply<<<dim3((unsigned)nch, nt), 256, 0, st>>>(x, ncol, N, ch, work, scale, offset);
     mrc_prof_post(7, st, 0, 0);
     return cudaGetLastError();
 }

@@ -313,9 +313,11 @@ cudaError_t mrc_base_case(const double *A, double *psi, int d, int64_t m0, cudaS
 cudaError_t mrc_order(cudaStream_t st);
 cudaError_t mrc_row_sums(const double *q, double *rs, int d, int64_t N, cudaStream_t st);
 // x(k) <- offset + scale sum_{l <= k} x(l) down the rows (scale = +-1);
-// work: mrc_scan_bytes(N, ncol)
+// work: mrc_scan_bytes(N, ncol), or down to mrc_scan_bytes_min with longer chains
 size_t mrc_scan_bytes(int64_t N, int ncol);
-cudaError_t mrc_scan_cols(double *x, int ncol, int64_t N, void *work, double scale, double offset, cudaStream_t st);
+size_t mrc_scan_bytes_min(int64_t N, int ncol);
+cudaError_t mrc_scan_cols(double *x, int ncol, int64_t N, void *work, size_t work_bytes, double scale, double offset,
+                          cudaStream_t st);
 cudaError_t mrc_norms(const double *rho, int E, int64_t N, double *acc, cudaStream_t st);
 cudaError_t mrc_gather_blocks(const double *q, int d, int64_t N, const int *Cidx, int nC, const int *Didx,
                               int nD, double *ACC, double *QCD, cudaStream_t st);

@@ -208,3 +208,21 @@ def test_seed_singular(mrc, d):
         mrc.sync_status()
     eye = torch.eye(d, dtype=torch.float64, device="cuda")[None]
     assert torch.equal(mrc.inverse(eye, report=True)[0], eye)
+
+
+@pytest.mark.parametrize("N", [5, 2048, 32768])
+def test_running_sums_in_small_scratch(mrc, N, monkeypatch):
+    """A workspace cap of 256 B makes the running sums' chunks longer: the same
+    sums to a rounding of each (they are kept as unevaluated pairs)."""
+    rng = np.random.default_rng(N)
+    psi, alpha = dev(rng.random((N, 3, 3))), dev(rng.random(3))
+    ref = mrc.renewal_visits(psi, alpha, [0, 2])
+    ctx = mrc.create_context(max_workspace_bytes=256)
+    try:
+        monkeypatch.setattr(mrc, "context", lambda device=None: ctx)
+        got = mrc.renewal_visits(psi, alpha, [0, 2])
+        torch.cuda.synchronize()
+    finally:
+        monkeypatch.undo()
+        mrc.destroy_context(ctx)
+    assert ((got - ref).abs() <= 2.0 ** -52 * ref.abs()).all()
