@@ -77,37 +77,31 @@ def load_peaks():
         return {"hbm_gbs": 6800.0, "bf16_tflops": 1900.0, "bf16_tflops_sustained": 1700.0}, "fallback"
 
 
-# FP64 DFMA rate measured on this machine's GB300 by a dependent-chain-free FMA
-# loop (1.19 TFLOP/s); FP32 FFMA: 152 SMs x 128 lanes x 2 flops per clock.
+# FP32 FFMA: 152 SMs x 128 lanes x 2 flops per clock.
 FP32_LANES = 152 * 128
-FP64_TFLOPS_MEASURED = 1.19
 
 
 def roofline_for(kclass, ms_total, launches, bytes_, flops, peaks, sm_mhz, d=None):
     """Roofline of one kernel class from its timed launches: achieved =
     algorithmic bytes (or flops) per launch / average launch time.  FFT
     passes, the tensor-core digit products (whose FP32 and tensor pipes are
-    not the binding resource at d <= 64) and the small kernels are reported
-    against the measured HBM copy bandwidth; FP64 products against the
-    measured DFMA rate, FP32-pipe products against the FFMA peak."""
+    not the binding resource at d <= 64), the FP64 path's products (fixed point,
+    on the integer pipes or the tensor cores) and the small kernels are reported
+    against the measured HBM copy bandwidth; FP32-pipe products against the
+    FFMA peak."""
     if not launches:
         return None
     per_ms = ms_total / launches
     name = KCLASS[kclass]
     clk = (sm_mhz or 2070.0) * 1e6
+    fixed = name == "pairmul_f64"
     on_tc = name in ("pairmul_dd", "pairmul_f32") and d is not None and 32 <= d <= (512 if name == "pairmul_dd" else 64)
-    if name.startswith("fft_") or name == "misc" or on_tc:
+    if name.startswith("fft_") or name == "misc" or on_tc or fixed:
         ach = bytes_ / launches / (per_ms * 1e-3) / 1e9
         peak = peaks["hbm_gbs"]
-        src = "MEASURED_PEAKS.json hbm_gbs (of measured)" + ("; tensor-core digit products" if on_tc else "")
+        src = "MEASURED_PEAKS.json hbm_gbs (of measured)" + ("; tensor-core digit products" if on_tc else "; fixed-point products" if fixed else "")
         return {"kernel": name, "bound": "hbm", "achieved": ach, "peak": peak, "unit": "GB/s",
                 "frac": ach / peak, "traffic": None, "launches": launches, "avg_ms": per_ms, "peak_source": src}
-    if name.endswith("_f64"):
-        ach = flops / launches / (per_ms * 1e-3) / 1e12
-        peak = FP64_TFLOPS_MEASURED
-        return {"kernel": name, "bound": "alu", "achieved": ach, "peak": peak, "unit": "TFLOP/s",
-                "frac": ach / peak, "traffic": None, "launches": launches, "avg_ms": per_ms,
-                "peak_source": "FP64 DFMA loop measured on GB300 (1.19 TFLOP/s)"}
     # FP32-pipe or double-float SIMT products: FP32 FFMA bound at d >= 16
     ach = flops / launches / (per_ms * 1e-3) / 1e12
     peak = FP32_LANES * 2 * clk / 1e12
@@ -120,7 +114,7 @@ def roofline_for(kclass, ms_total, launches, bytes_, flops, peaks, sm_mhz, d=Non
 # of a class stays valid while these files are unchanged.
 _CLASS_SOURCES = {
     "fft": ["kernels.cuh", "launchers.cuh", "arith.cuh", "mrc_internal.h"],
-    "tc": ["pair_tc.cu", "ozaki_tc.cu", "tcgen05.cuh", "digits.cuh", "kernels.cuh", "arith.cuh", "mrc_internal.h"],
+    "tc": ["pair_tc.cu", "ozaki_tc.cu", "q64.cuh", "tcgen05.cuh", "digits.cuh", "kernels.cuh", "arith.cuh", "mrc_internal.h"],
     "simt": ["kernels.cuh", "launchers.cuh", "arith.cuh", "mrc_internal.h"],
 }
 
@@ -128,10 +122,13 @@ _CLASS_SOURCES = {
 def class_sources(kernel):
     if kernel.startswith("fft_"):
         prec = kernel[4:]
-        return _CLASS_SOURCES["fft"] + [f"k_{prec}_fft_lo.cu", f"k_{prec}_fft_hi.cu", f"k_{prec}.cu"]
+        fixed = ["fftq.cuh", "q64.cuh"] if prec == "f64" else []
+        return _CLASS_SOURCES["fft"] + fixed + [f"k_{prec}_fft_lo.cu", f"k_{prec}_fft_hi.cu", f"k_{prec}.cu"]
     if kernel in ("pairmul_dd", "pairmul_f32"):
         return _CLASS_SOURCES["tc"]
-    return _CLASS_SOURCES["simt"] + ["k_f64.cu", "k_f32.cu", "k_dd.cu", "misc.cu"]
+    if kernel == "pairmul_f64":
+        return _CLASS_SOURCES["tc"] + ["pair_q.cu", "launchers.cuh", "k_f64.cu"]
+    return _CLASS_SOURCES["simt"] + ["k_f64.cu", "k_f32.cu", "k_dd.cu", "misc.cu", "seed.cu"]
 
 
 def sources_digest(kernel):

@@ -37,8 +37,7 @@
 template <class T>
 __device__ __forceinline__ cx<T> scale_out(const FftArgs &a, cx<T> v)
 {
-    if constexpr (sizeof(T) == 8 && sizeof(cx<T>) == 16 && !__is_same(T, dd)) return c_scal(v, a.dst_scale);
-    else return {Ar<T>::scal_f(v.re, a.dst_scale_f), Ar<T>::scal_f(v.im, a.dst_scale_f)};
+    return {Ar<T>::scal_f(v.re, a.dst_scale_f), Ar<T>::scal_f(v.im, a.dst_scale_f)};
 }
 
 // Small DFTs in registers, natural order in and out.  INV selects the sign
