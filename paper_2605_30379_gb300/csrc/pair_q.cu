@@ -153,7 +153,8 @@ __device__ __forceinline__ void pairq_body(const PairArgs &a, int64_t p0)
 // Product with a diagonal right factor, C(f)_ij = X(f)_ij Y(f)_j: a complex
 // product per entry, with each pair of packed values aligned by itself and
 // merged in fixed point.  The 56 FP64 operations per pair of entries were what
-// bound it (1.1 ms at d = 32, M = 2^14, where its bytes take 0.08 ms).  CTA:
+// bound it (1.1 ms at d = 32, M = 2^14, where its bytes take 0.08 ms; now
+// 0.21).  CTA:
 // the pairs p0 .. p0 + pp - 1; Y's factors once per column.
 __global__ void __launch_bounds__(NT) pairdiagq_kernel(const PairArgs a)
 {

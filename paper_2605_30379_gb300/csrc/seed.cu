@@ -10,7 +10,8 @@
 // other).  Here the data live in shared memory; for d > 32 the CTAs own the rows
 // i = rank mod CL and exchange pivots and pivot rows through distributed shared
 // memory with one cluster barrier per column, and a level m -> 2m takes two
-// barriers, its sums spread over all threads of the cluster.
+// barriers, its sums spread over all threads of the cluster (whole inverse d = 3,
+// N = 128 in FP64 262 -> 37 us, mixed d = 256, N = 4096 183 -> 172 ms).
 #include <cooperative_groups.h>
 
 #include <float.h>
