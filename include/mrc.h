@@ -300,7 +300,7 @@ mrc_status mrc_renewal_visits(mrc_ctx *ctx, int d, int64_t N, const double *psi,
  * agree with mrc_inverse's to rounding.
  *   d, N, A, psi, stream : as mrc_inverse with prec = MRC_FP64.
  * Scratch: one fixed 64 MiB device array inside the library.  The call uses
- * 256 B + 512 KiB (twiddles) + 4 * 16 d^2 * M bytes of it, M being
+ * 256 B + 512 KiB (twiddles) + 8.25 KiB + 4 * 16 d^2 * M bytes of it, M being
  * the largest Newton level (< N); N must be <= 2^14.  Larger requests return
  * MRC_ERR_NO_MEMORY at once, with the limit printed to stderr.
  * No cudaMalloc/cudaFree or allocating library routine is called.

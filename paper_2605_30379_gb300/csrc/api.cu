@@ -31,6 +31,8 @@ struct BatchGraph {
 };
 
 #define MRC_BATCH_STREAMS 8
+// pairs of the largest FP64 product (N = 2^20: transforms of 2^20 points)
+#define MARK_PAIRS (((int64_t)1 << 19) + 1)
 
 struct mrc_ctx {
     int device = 0;
@@ -39,6 +41,7 @@ struct mrc_ctx {
     size_t ws_size = 0;
     void *tw[3] = {nullptr, nullptr, nullptr};
     int *d_status = nullptr;
+    void *marks = nullptr;  // of an FP64 digit product: MRC_MARK_BYTES(MARK_PAIRS)
     double *d_acc = nullptr;  // [4] norm accumulators
     cudaEvent_t ev0 = nullptr, ev1 = nullptr;
     // streams of the single-model mixed inverse, created on first use: the
@@ -231,7 +234,7 @@ bool tensor_default(int prec, int64_t M, int r, int m, int c)
 cudaError_t launch_tensor(mrc_ctx *cx, int prec, const void *zx, const void *zy, void *zc, int64_t M, int d,
                           const void *tw, cudaStream_t st)
 {
-    if (prec == PREC_F64) return mrc_pairmul_f64_tcp(zx, zy, zc, M, d, tw, MRC_TW_LOG, cx->cur_status, st);
+    if (prec == PREC_F64) return mrc_pairmul_f64_tcp(zx, zy, zc, M, d, tw, MRC_TW_LOG, cx->cur_status, cx->marks, st);
     if (prec == PREC_F32) return mrc_pairmul_f32_tcp(zx, zy, zc, M, d, tw, MRC_TW_LOG, cx->cur_status, st);
     if (d <= 64) return mrc_pairmul_dd_tcp(zx, zy, zc, M, d, tw, MRC_TW_LOG, cx->cur_status, st);
     return mrc_pairmul_dd_tc(zx, zy, zc, M, d, tw, MRC_TW_LOG, cx->cur_status, st);
@@ -910,9 +913,11 @@ mrc_status product_stage(mrc_ctx *c, int prec, int64_t M, const std::vector<Pair
         }
     }
     auto P = std::make_unique<SegParams<PairArgs>>();
+    // products per launch: FP64's pairs also by the room for their marks
+    const size_t nmax = prec == PREC_F64 ? std::min<size_t>(MRC_SEG_MAX, (size_t)(MARK_PAIRS / (M / 2 + 1))) : MRC_SEG_MAX;
     for (int g = 0; g < 10; ++g)
-        for (size_t i0 = 0; i0 < tcp[g].size(); i0 += MRC_SEG_MAX) {
-            const size_t i1 = std::min(tcp[g].size(), i0 + (size_t)MRC_SEG_MAX);
+        for (size_t i0 = 0; i0 < tcp[g].size(); i0 += nmax) {
+            const size_t i1 = std::min(tcp[g].size(), i0 + nmax);
             P->nseg = (int)(i1 - i0);
             for (size_t q = i0; q < i1; ++q) {
                 const PairJob &j = jobs[tcp[g][q]];
@@ -920,6 +925,7 @@ mrc_status product_stage(mrc_ctx *c, int prec, int64_t M, const std::vector<Pair
                 P->a[q - i0] = mrc_tcp_args(j.zx, j.zy, j.zc, M, j.d, c->tw[prec], MRC_TW_LOG);
                 P->a[q - i0].xs = j.xs;
             }
+            P->a[0].marks = (unsigned char *)c->marks;
             CK(mrc_tcp_seg(prec, *P, jobs[tcp[g][i0]].status, st));
         }
     const int bsz[5] = {16, 32, 64, 0, 24};
@@ -1208,7 +1214,11 @@ mrc_status mrc_create(mrc_ctx **out, int device, size_t max_workspace_bytes)
     mrc_ctx *c = new mrc_ctx();
     c->device = device;
     c->cap = max_workspace_bytes;
-    if (cudaMalloc(&c->d_status, sizeof(int)) != cudaSuccess || cudaMalloc(&c->d_acc, 4 * sizeof(double)) != cudaSuccess) {
+    if (cudaMalloc(&c->d_status, sizeof(int)) != cudaSuccess || cudaMalloc(&c->d_acc, 4 * sizeof(double)) != cudaSuccess ||
+        cudaMalloc(&c->marks, MRC_MARK_BYTES(MARK_PAIRS)) != cudaSuccess) {
+        cudaGetLastError();
+        cudaFree(c->d_status);
+        cudaFree(c->d_acc);
         delete c;
         return MRC_ERR_NO_MEMORY;
     }
@@ -1231,6 +1241,7 @@ mrc_status mrc_destroy(mrc_ctx *c)
     for (int p = 0; p < 3; ++p) cudaFree(c->tw[p]);
     cudaFree(c->d_status);
     cudaFree(c->d_acc);
+    cudaFree(c->marks);
     cudaEventDestroy(c->ev0);
     cudaEventDestroy(c->ev1);
     if (c->aux) {

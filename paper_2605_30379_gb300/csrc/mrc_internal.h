@@ -57,6 +57,7 @@ struct PairArgs {
     // tensor-core double-float product with X prepared (mrc_tcp_prep): zx
     // holds X's digit tiles, xs its per-pair scale factors; else null
     const void *xs;
+    unsigned char *marks;  // FP64 digit product, a launch's first product: blocks to sum again (graded.cuh)
 };
 
 // Source / destination descriptors used by the host-side FFT driver.
@@ -226,11 +227,17 @@ cudaError_t mrc_pairmul_f32_tcp(const void *zx, const void *zy, void *zc, int64_
 // every M, and at d = 36 they tie from M = 512 on).
 bool mrc_tcp64_supported(int r, int m, int c);
 bool mrc_tcp64_default(int64_t M, int d);
+// marks: MRC_MARK_BYTES(M / 2 + 1) of scratch
 cudaError_t mrc_pairmul_f64_tcp(const void *zx, const void *zy, void *zc, int64_t M, int d, const void *tw, int tw_log,
-                                int *status, cudaStream_t st);
+                                int *status, void *marks, cudaStream_t st);
+#define MRC_MARK_BYTES(pairs) (2 * (size_t)(pairs))
 // the same over the products of one segmented launch (all of the same
 // precision, M and ceil(d / 16)); a timeout is reported in *status
 cudaError_t mrc_tcp_seg(int prec, const SegParams<PairArgs> &P, int *status, cudaStream_t st);
+// the outputs of the marked blocks that are not sound, in floating FP64 (graded.cuh);
+// launched after every FP64 digit product (P.a[0].marks: of all the launch's pairs)
+cudaError_t mrc_redo_init(void);
+cudaError_t mrc_pair_redo(const SegParams<PairArgs> &P, int kclass, cudaStream_t st);
 PairArgs mrc_tcp_args(const void *zx, const void *zy, void *zc, int64_t M, int d, const void *tw, int tw_log);
 // The double-float product with X prepared once (X is the spectrum of A,
 // the same in every residual sweep): mrc_tcp_prep writes, for every product

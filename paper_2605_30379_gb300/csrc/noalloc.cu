@@ -8,7 +8,7 @@
 // host that hands its plugins fixed buffers only.  For them this entry point
 // runs the FP64 FFT-Newton schedule of mrc_inverse (the same level loop, FFT
 // kernels and default FP64 product kernel), but its scratch (the spectra of
-// the Newton levels, the Gauss-Jordan work area, the twiddle table and the
+// the Newton levels, the twiddle table, the products' marks and the
 // status word) lives in one file-scope __device__ array of fixed size, so
 // nothing is allocated at call time.  The caller still passes A and psi.
 //
@@ -42,11 +42,13 @@ unsigned char *g_addr[kMaxDevices] = {};
 
 size_t up256(size_t x) { return (x + 255) & ~(size_t)255; }
 
-// Scratch layout: [status int | twiddles | Gauss-Jordan work | 4 spectra]
+// Scratch layout: [status int | twiddles | marks of the FP64 digit product | 4 spectra]
 constexpr size_t kStatusOff = 0;
 constexpr size_t kTwOff = 256;
 constexpr size_t kTwBytes = (size_t)16 << kTwLog;
-constexpr size_t kWorkOff = kTwOff + kTwBytes;
+constexpr size_t kMarkOff = kTwOff + kTwBytes;
+constexpr size_t kMarkBytes = MRC_MARK_BYTES((1 << (kTwLog - 3)) + 128);  // levels below N: at most 2^13 points
+constexpr size_t kWorkOff = kMarkOff + kMarkBytes;
 
 int64_t max_level(int d, int64_t N) { return mrc_newton_maxM(d, N, false); }
 
@@ -59,11 +61,12 @@ cudaError_t fft_f64(void *, int, const FftSrc &sx, const FftDst &dx, int64_t M, 
 }
 
 // the level product: the default FP64 product kernels (no autotuning here);
-// status: the word a tensor-core product's bounded wait reports to
-cudaError_t product_f64(void *status, int, const void *zx, const void *zy, void *zc, int64_t M, int d, const void *tw,
+// scratch: the array, with the word a tensor-core product's bounded wait reports to
+cudaError_t product_f64(void *scratch, int, const void *zx, const void *zy, void *zc, int64_t M, int d, const void *tw,
                         int tw_log, cudaStream_t st)
 {
-    if (mrc_tcp64_default(M, d)) return mrc_pairmul_f64_tcp(zx, zy, zc, M, d, tw, tw_log, (int *)status, st);
+    if (mrc_tcp64_default(M, d)) return mrc_pairmul_f64_tcp(zx, zy, zc, M, d, tw, tw_log, (int *)((char *)scratch + kStatusOff),
+                                                               (char *)scratch + kMarkOff, st);
     return mrc_pairmul_f64(zx, zy, zc, M, d, d, d, tw, tw_log, st);
 }
 
@@ -146,7 +149,7 @@ extern "C" mrc_status mrc_inverse_noalloc(int d, int64_t N, const double *A, dou
     CKN(mrc_seed(sp, st));
     if (d > MRC_SEED_DMAX) CKN(mrc_base_case(A, psi, d, m0, st));
     const NewtonBufs nb{b0, b1, b2, bt};
-    if (mrc_newton_levels(PREC_F64, d, N, A, psi, m0, nb, tw, kTwLog, fft_f64, product_f64, status, st, nullptr,
+    if (mrc_newton_levels(PREC_F64, d, N, A, psi, m0, nb, tw, kTwLog, fft_f64, product_f64, base, st, nullptr,
                           nullptr, nullptr) != 0)
         return MRC_ERR_CUDA;
     CKN(cudaStreamSynchronize(st));

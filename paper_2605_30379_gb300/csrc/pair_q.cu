@@ -13,7 +13,8 @@
 // every eight terms), and each sum is rounded once to FP64.  (Without the low
 // products, a quarter of the work, the error of a Weibull d = 16, N = 2048
 // inverse rises from FP64's 1.2e-15 to 9e-15: e0 - q is singular at frequency
-// zero.)
+// zero.)  Outputs whose terms lie far below their row and column bounds are summed
+// again by the same CTA (graded.cuh).
 //
 // One CTA takes the pairs p0 .. p0 + pp - 1 (pp so that its outputs fill the
 // threads once, fewer when there are fewer pairs than SMs): it loads their
@@ -25,7 +26,7 @@
 // entrance with 18 x 18 blocks, N = 10000, 6.4 -> 1.2 ms.
 #include <algorithm>
 
-#include "q64.cuh"
+#include "graded.cuh"
 #include "mrc_internal.h"
 
 namespace {
@@ -34,7 +35,7 @@ constexpr int NT = 128;
 // raw values below 2^top, 2 Xh below 2^(top + 2), so that m products of two
 // numbers of such moduli stay below 2^63 with their 2^60 taken off
 __device__ __forceinline__ int top_for(int m) { return m <= 4 ? 58 : (m <= 31 ? 57 : 56); }
-constexpr int SMEM_MAX = 200 * 1024;
+constexpr int SMEM_MAX = 212 * 1024;
 
 // t / d for t, d < 2^16 by a multiplication (a division by a run-time number
 // takes some 25 instructions, and every entry and output is indexed by three)
@@ -76,15 +77,143 @@ size_t pair_bytes(int r, int m, int c)
 {
     return 2 * sizeof(qtw) * ((size_t)r * m + (size_t)m * c) + sizeof(qtw) + sizeof(int) * ((size_t)r + c);
 }
+// shared memory of a CTA of pp pairs: theirs and the logarithms at frequency 0 of
+// X's diagonal and Y
+size_t cta_bytes(int pp, int r, int m, int c) { return pp * pair_bytes(r, m, c) + sizeof(short) * ((size_t)r + (size_t)m * c); }
+
+// The CTA's shared memory
+struct Smem {
+    qtw *sf, *sg, *stw;  // per pair: X then Y entries at f and g, twiddle
+    unsigned *bnd;       // per pair: r row and c column bounds
+    short *x0, *y0;      // logarithms at frequency 0: X_ii (column 0 where X has one), Y
+    __device__ __forceinline__ Smem(unsigned char *p, int pp, int ex2, int r, int c)
+        : sf(reinterpret_cast<qtw *>(p)), sg(sf + pp * ex2), stw(sg + pp * ex2),
+          bnd(reinterpret_cast<unsigned *>(stw + pp)), x0(reinterpret_cast<short *>(bnd + pp * (r + c))), y0(x0 + r)
+    {
+    }
+};
+
+// A lower bound of a term's size from the limbs' high parts (2 Xh and 2 Yh: at most
+// four times the packed values that gr_sound compares), over 2^60
+__device__ __forceinline__ float term_size(const qtw &a, const qtw &b, const qtw &u, const qtw &v)
+{
+    return (float)max(max(abs(a.rh), abs(a.ih)), max(abs(b.rh), abs(b.ih))) *
+           (float)max(max(abs(u.rh), abs(u.ih)), max(abs(v.rh), abs(v.ih)));
+}
+
+// The logarithm of the largest term of an output from its row of X and its column of Y
+// in global memory: packed values at rows f and g
+__device__ __forceinline__ int largest_term(const cx<double> *xf, const cx<double> *xg, const cx<double> *yf,
+                                            const cx<double> *yg, int m, int c)
+{
+    int l = 2 * GR_ZERO;
+    for (int k = 0; k < m; ++k)
+        l = max(l, gr_log(max(gr_magnitude(xf[k]), gr_magnitude(xg[k]))) +
+                       gr_log(max(gr_magnitude(yf[k * c]), gr_magnitude(yg[k * c]))));
+    return l;
+}
+
+// One unsound output by one warp, with every entry aligned by itself, its terms
+// across the lanes: for CTAs with a few of them (one output in a thousand of an
+// entrance with 18 x 18 blocks, N = 10000, is 2^-14 below its bounds; splitting the whole
+// pairs again for it took the call from 2.86 to 3.02 ms)
+__device__ __forceinline__ void redo_one(const PairArgs &a, int64_t f, int i, int j, qtw w)
+{
+    const int r = a.r, m = a.m, c = a.c, lane = threadIdx.x & 31;
+    const int64_t g = (a.M - f) & (a.M - 1), EX = (int64_t)r * m, EY = (int64_t)m * c, EC = (int64_t)r * c;
+    const cx<double> *X = reinterpret_cast<const cx<double> *>(a.zx) + i * m;
+    const cx<double> *Y = reinterpret_cast<const cx<double> *>(a.zy) + j;
+    int G = 2 * GR_ZERO;
+    for (int k = lane; k < m; k += 32) {
+        cx<double> xf = X[f * EX + k], xg = X[g * EX + k], yf = Y[f * EY + k * c], yg = Y[g * EY + k * c];
+        G = max(G, (gr_scaled(xf, xg) >> 4) + (gr_scaled(yf, yg) >> 4));
+    }
+    G = __reduce_max_sync(0xffffffffu, G);
+    long long v[4] = {0, 0, 0, 0};
+    for (int k = lane; k < m; k += 32) {
+        short lx, ly;
+        qtw xf, xg, yf, yg;
+        gr_split(X[f * EX + k], X[g * EX + k], w, lx, xf, xg);
+        gr_split(Y[f * EY + k * c], Y[g * EY + k * c], w, ly, yf, yg);
+        const int s = G - (lx >> 4) - (ly >> 4);
+        if (s > 61) continue;
+        gr_mac(v[0], v[1], xf, yf, s);
+        gr_mac(v[2], v[3], xg, yg, s);
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+        for (int u = 0; u < 4; ++u) v[u] += __shfl_xor_sync(0xffffffffu, v[u], o);
+    if (lane != 0) return;
+    cx<double> *ZC = reinterpret_cast<cx<double> *>(a.zc) + (int64_t)i * c + j;
+    const cx<double> *tw = reinterpret_cast<const cx<double> *>(a.tw);
+    cx<double> zf, zg;
+    q_merge(gr_value(v[0], v[1], G), gr_value(v[2], v[3], G), tw[f << (a.tw_log - a.logM - 1)], zf, zg);
+    ZC[f * EC] = zf;
+    if (g != f) ZC[g * EC] = zg;
+}
+
+// All unsound outputs of the CTA's pairs.  One frequency after the other, so that
+// the limbs of the first sum leave room for the entries' logarithms; C(f) waits in
+// the output.
+__device__ __forceinline__ void pairq_redo(const PairArgs *ap, int64_t p0)
+{
+    extern __shared__ __align__(16) unsigned char smem[];
+    const PairArgs &a = *ap;
+    const int r = a.r, m = a.m, c = a.c, EX = r * m, EC = r * c, ex2 = EX + m * c;
+    const int np = (int)min((int64_t)a.pp, a.npairs - p0);
+    const Smem s(smem, a.pp, ex2, r, c);
+    short *const lp = reinterpret_cast<short *>(s.sg), *const l0 = lp + np * ex2;  // of the pairs' entries, of those at frequency 0
+    const cx<double> *ZX = reinterpret_cast<const cx<double> *>(a.zx), *ZY = reinterpret_cast<const cx<double> *>(a.zy);
+    cx<double> *ZC = reinterpret_cast<cx<double> *>(a.zc);
+    const cx<double> *tw = reinterpret_cast<const cx<double> *>(a.tw);
+    auto packed = [&](int64_t row, int e) { return e < EX ? ZX[row * EX + e] : ZY[row * (ex2 - EX) + e - EX]; };
+    for (int t = threadIdx.x; t < np * ex2; t += NT) {
+        const int q = t / ex2, e = t - q * ex2;
+        const int64_t f = p0 + q, g = (a.M - f) & (a.M - 1);
+        lp[t] = gr_log(max(gr_magnitude(packed(f, e)), gr_magnitude(packed(g, e))));
+        if (q == 0) l0[e] = gr_log(gr_magnitude(packed(0, e)));
+    }
+    __syncthreads();
+    for (int phase = 0; phase < 2; ++phase) {
+        for (int t = threadIdx.x; t < np * ex2; t += NT) {
+            const int q = t / ex2, e = t - q * ex2;
+            const int64_t f = p0 + q, g = (a.M - f) & (a.M - 1);
+            qtw vf, vg;
+            gr_split(packed(f, e), packed(g, e), s.stw[q], lp[t], vf, vg);
+            s.sf[t] = phase == 0 ? vf : vg;
+        }
+        __syncthreads();
+        for (int t = threadIdx.x; t < np * EC; t += NT) {
+            const int q = t / EC, e = t - q * EC, i = e / c, j = e - i * c, xo = q * ex2 + i * m, yo = q * ex2 + EX + j;
+            const unsigned *b = s.bnd + q * (r + c);
+            if (gr_sound(l0 + i * m, l0 + EX + j, lp + xo, lp + yo, m, c, q_align(b[i]), q_align(b[r + j]), a.logM)) continue;
+            const cx<double> v = gr_sum(s.sf + xo, s.sf + yo, lp + xo, lp + yo, m, c);
+            const int64_t f = p0 + q, g = (a.M - f) & (a.M - 1);
+            if (phase == 0) {
+                ZC[f * EC + e] = v;
+                continue;
+            }
+            cx<double> zf, zg;
+            q_merge(ZC[f * EC + e], v, tw[f << (a.tw_log - a.logM - 1)], zf, zg);
+            ZC[f * EC + e] = zf;
+            if (g != f) ZC[g * EC + e] = zg;
+        }
+        __syncthreads();
+    }
+}
 
 __device__ __forceinline__ void pairq_body(const PairArgs &a, int64_t p0)
 {
     extern __shared__ __align__(16) unsigned char smem[];
+    constexpr int LIST = 64;
+    __shared__ int nredo;  // unsound outputs, the first of them
+    __shared__ unsigned short redo[LIST];
     const int r = a.r, m = a.m, c = a.c, EX = r * m, EY = m * c, EC = r * c, ex2 = EX + EY;
     const int np = (int)min((int64_t)a.pp, a.npairs - p0);
-    qtw *sf = reinterpret_cast<qtw *>(smem), *sg = sf + a.pp * ex2;  // per pair: X then Y entries, f and g
-    qtw *stw = reinterpret_cast<qtw *>(sg + a.pp * ex2);
-    unsigned *bnd = reinterpret_cast<unsigned *>(stw + a.pp);            // per pair: r row and c column bounds
+    const Smem sm(smem, a.pp, ex2, r, c);
+    qtw *sf = sm.sf, *sg = sm.sg, *stw = sm.stw;
+    unsigned *bnd = sm.bnd;
     const cx<double> *ZX = reinterpret_cast<const cx<double> *>(a.zx), *ZY = reinterpret_cast<const cx<double> *>(a.zy);
     cx<double> *ZC = reinterpret_cast<cx<double> *>(a.zc);
     const cx<double> *tw = reinterpret_cast<const cx<double> *>(a.tw);
@@ -93,6 +222,7 @@ __device__ __forceinline__ void pairq_body(const PairArgs &a, int64_t p0)
     const int tid = threadIdx.x, top = top_for(m);
     const FastDiv dex2(ex2), dm(m), dc(c), dEC(EC);
 
+    if (tid == 0) nredo = 0;
     for (int t = tid; t < np * (r + c); t += NT) bnd[t] = 0u;
     for (int t = tid; t < np; t += NT) stw[t] = q_twiddle(tw[(p0 + t) << tws], 0, false);
     overlap_release();
@@ -107,8 +237,10 @@ __device__ __forceinline__ void pairq_body(const PairArgs &a, int64_t p0)
         const cx<double> za = x ? ZX[f * EX + ee] : ZY[f * EY + ee], zb = x ? ZX[g * EX + ee] : ZY[g * EY + ee];
         reinterpret_cast<cx<double> *>(sf)[t] = za;
         reinterpret_cast<cx<double> *>(sg)[t] = zb;
-        const unsigned b = max(max(q_magnitude(za.re), q_magnitude(za.im)), max(q_magnitude(zb.re), q_magnitude(zb.im)));
-        atomicMax(&bnd[q * (r + c) + (x ? dm.div(ee) : r + ee - dc.div(ee) * c)], b);
+        const int rc = x ? dm.div(ee) : ee - dc.div(ee) * c;
+        if (q == 0 && !x) sm.y0[ee] = gr_log(gr_magnitude(ZY[ee]));
+        if (q == 0 && x && ee == rc * m + min(rc, m - 1)) sm.x0[rc] = gr_log(gr_magnitude(ZX[ee]));
+        atomicMax(&bnd[q * (r + c) + (x ? rc : r + rc)], max(gr_magnitude(za), gr_magnitude(zb)));
     }
     __syncthreads();
     // the split of both frequencies, in place (every thread its own entries)
@@ -123,6 +255,7 @@ __device__ __forceinline__ void pairq_body(const PairArgs &a, int64_t p0)
         sg[t] = q_limbs({{s.re.v - u.re.v}, {u.im.v - s.im.v}});
     }
     __syncthreads();
+    const float own_min = exp2f((float)(2 * top - 60 - GR_GUARD + 4));  // term_size of an output sound by its own terms
     for (int t = tid; t < np * EC; t += NT) {
         const int q = dEC.div(t), e = t - q * EC, i = dc.div(e), j = e - i * c;
         const int xo = q * ex2 + i * m, yo = q * ex2 + EX + j;
@@ -138,6 +271,25 @@ __device__ __forceinline__ void pairq_body(const PairArgs &a, int64_t p0)
             fold(ag);
         }
         const int ax = q_align(bnd[q * (r + c) + i]), ay = q_align(bnd[q * (r + c) + r + j]);
+        // gr_sound, the likely reasons first: the term k = i at frequency 0, the terms k = i
+        // and k = j of the pair itself, all terms at frequency 0
+        const int ki = min(i, m - 1), kj = min(j, m - 1);
+        if (!gr_sound_by(ax, ay, sm.x0[i] + sm.y0[ki * c + j], a.logM)) {
+            const float s = fmaxf(term_size(sf[xo + ki], sg[xo + ki], sf[yo + ki * c], sg[yo + ki * c]),
+                                  term_size(sf[xo + kj], sg[xo + kj], sf[yo + kj * c], sg[yo + kj * c]));
+            if (!gr_in_range(ax, ay) || s < own_min) {
+                int g0 = 2 * GR_ZERO;
+                for (int k = 0; k < m; ++k) g0 = max(g0, gr_log(gr_magnitude(ZX[i * m + k])) + sm.y0[k * c + j]);
+                if (!gr_sound_by(ax, ay, g0, a.logM) && max(ax, ay) < Q_NONFINITE) {
+                    const int64_t f = p0 + q, g = (M - f) & (M - 1);
+                    const int gp = largest_term(ZX + f * EX + i * m, ZX + g * EX + i * m, ZY + f * EY + j, ZY + g * EY + j, m, c);
+                    if (gp >= 0 && !gr_sound_by(ax, ay, gp, 0)) {
+                        const int n = atomicAdd(&nredo, 1);
+                        if (n < LIST) redo[n] = (unsigned short)t;
+                    }
+                }
+            }
+        }
         const int de = ax + ay - 2017 - 2 * top;  // the alignments, the limbs, the split's factors 2 and the merge's 1/2
         cx<double> cf = {q_scale(q94_to_double(af.hr, (int)af.mr), de), q_scale(q94_to_double(af.hi, (int)af.mi), de)};
         cx<double> cg = {q_scale(q94_to_double(ag.hr, (int)ag.mr), de), q_scale(q94_to_double(ag.hi, (int)ag.mi), de)};
@@ -148,6 +300,13 @@ __device__ __forceinline__ void pairq_body(const PairArgs &a, int64_t p0)
         ZC[f * EC + e] = zf;
         if (g != f) ZC[g * EC + e] = zg;
     }
+    __syncthreads();
+    if (nredo > LIST) pairq_redo(&a, p0);
+    else
+        for (int n = tid >> 5; n < nredo; n += NT / 32) {
+            const int t = redo[n], q = dEC.div(t), e = t - q * EC, i = dc.div(e);
+            redo_one(a, p0 + q, i, e - i * c, stw[q]);
+        }
 }
 
 // Product with a diagonal right factor, C(f)_ij = X(f)_ij Y(f)_j: a complex
@@ -213,7 +372,7 @@ __global__ void __launch_bounds__(NT) pairdiagq_kernel(const PairArgs a)
     }
 }
 
-__global__ void __launch_bounds__(NT) pairq_kernel(const PairArgs a) { pairq_body(a, (int64_t)blockIdx.x * a.pp); }
+__global__ void __launch_bounds__(NT) pairq_kernel(const __grid_constant__ PairArgs a) { pairq_body(a, (int64_t)blockIdx.x * a.pp); }
 
 __global__ void __launch_bounds__(NT) pairq_seg_kernel(const __grid_constant__ SegParams<PairArgs> P)
 {
@@ -223,7 +382,7 @@ __global__ void __launch_bounds__(NT) pairq_seg_kernel(const __grid_constant__ S
 
 } // namespace
 
-bool mrc_pairq_supported(int r, int m, int c) { return pair_bytes(r, m, c) <= (size_t)SMEM_MAX; }
+bool mrc_pairq_supported(int r, int m, int c) { return cta_bytes(1, r, m, c) <= (size_t)SMEM_MAX; }
 
 // Pairs per CTA: outputs for every thread, but no fewer CTAs than SMs where the
 // pairs allow, and at most 48 KB of shared memory when one pair needs less
@@ -249,7 +408,7 @@ cudaError_t mrc_pairq(const PairArgs &a0, int kclass, cudaStream_t st)
     const double by = (double)a.M * ((double)a.r * a.m + (double)a.m * a.c + (double)a.r * a.c) * 16.0;
     mrc_prof_pre(kclass, st);
     const unsigned grid = (unsigned)((a.npairs + a.pp - 1) / a.pp);
-    const size_t smem = a.pp * pair_bytes(a.r, a.m, a.c);
+    const size_t smem = cta_bytes(a.pp, a.r, a.m, a.c);
     if (grid <= MRC_OVERLAP_CTAS) {
         const cudaError_t e = mrc_launch_overlapped(pairq_kernel, dim3(grid), NT, smem, st, a);
         if (e != cudaSuccess) return e;
@@ -277,7 +436,7 @@ cudaError_t mrc_pairq_seg(const SegParams<PairArgs> &P, unsigned nctas, double b
 {
     if (P.nseg <= 0 || nctas == 0) return cudaSuccess;
     size_t sm = 0;
-    for (int s = 0; s < P.nseg; ++s) sm = std::max(sm, P.a[s].pp * pair_bytes(P.a[s].r, P.a[s].m, P.a[s].c));
+    for (int s = 0; s < P.nseg; ++s) sm = std::max(sm, cta_bytes(P.a[s].pp, P.a[s].r, P.a[s].m, P.a[s].c));
     mrc_prof_pre(kclass, st);
     pairq_seg_kernel<<<nctas, NT, sm, st>>>(P);
     mrc_prof_post(kclass, st, bytes, flops);

@@ -9,8 +9,8 @@
 //     multiply-adds per clock and SM; at d = 64, N = 2^15 the inverse's 28
 //     products take 14 ms here against 138 ms on it (whole inverse 159.6 ->
 //     32.2 ms with the later steps), with smaller errors (Weibull d = 64, N = 512 against
-//     long double: 7.9e-16 -> 5.5e-16);
-
+//     long double: 7.9e-16 -> 5.5e-16).  The epilogue marks blocks with outputs far
+//     below their bounds, which mrc_pair_redo sums again (graded.cuh);
 //   double-float (the residual product of Proposition 2.6): six balanced
 //     base-256 digits per value, digit pairs of weight s + t >= 5 (21 pairs
 //     in 6 weight groups), about 2^-41 relative to the row and column bounds;
@@ -64,7 +64,7 @@
 // status word and a shared abort flag; all roles then leave their loops, the
 // MMA thread waits (bounded) for its MMAs in flight, and the TMEM is freed.
 #include "digits.cuh"
-#include "q64.cuh"
+#include "graded.cuh"
 #include "tcgen05.cuh"
 
 namespace {
@@ -140,7 +140,9 @@ struct TcL {
     // NB pairs behind the split.
     static constexpr int NB = 8;
     static constexpr int OFF_SC = OFF_XCH + XCH;
-    static constexpr int SMEM = OFF_SC + (4 * NB + 4) * 64 * 4;
+    // FP64: the epilogue groups' exponents at frequency 0 (epi_table)
+    static constexpr int OFF_G0 = OFF_SC + (4 * NB + 4) * 64 * 4;
+    static constexpr int SMEM = OFF_G0 + (tc_q<T> ? 2 * 64 * GR_BJ * (int)sizeof(short) : 0);
     static constexpr int TCOLS = NG * 64;  // TMEM columns of one frequency's groups
     static_assert(NF * TCOLS <= (int)TMEM_COLS, "accumulators fit in TMEM");
     static_assert(SMEM <= 227 * 1024, "shared memory");
@@ -273,12 +275,18 @@ __device__ __forceinline__ void bnd_reduce(const BndIn &b, unsigned *bx, float &
 
 // The pair's scale factors from its bounds (2 Xh and 2 Yh are split: bound
 // 2 |.|, scaled values <= 1/2)
+constexpr int EXP_NONE = -14000;
 template <class T>
 __device__ __forceinline__ void bnd_scales(const unsigned *bx, const unsigned *by, float *sc, int d, int t)
 {
     if constexpr (tc_q<T>) {
-        sc[t] = sc[128 + t] = __int_as_float(t < d ? q_align(bx[t]) : 1);
-        sc[64 + t] = sc[192 + t] = __int_as_float(t < d ? q_align(by[t]) : 1);
+        const int ax = q_align(bx[t]), ay = q_align(by[t]);
+        sc[t] = __int_as_float(t < d ? ax : 1);
+        sc[64 + t] = __int_as_float(t < d ? ay : 1);
+        // for the output: EXP_NONE where the row or column is out of the aligned
+        // range (or zero), 1023 (which epi_table lets pass) beyond the matrix
+        sc[128 + t] = __int_as_float(t < d ? (ax > Q_EXMIN ? ax : EXP_NONE) : 1023);
+        sc[192 + t] = __int_as_float(t < d ? (ay > Q_EXMIN ? ay : EXP_NONE) : 1023);
         return;
     }
     const int sx = t < d ? scale_exp(2.0f * __uint_as_float(bx[t])) : 0;
@@ -743,26 +751,67 @@ __device__ __forceinline__ int epi_row(int ge, int m)
     return (ge >> 5) + 4 * (m & 3) + (ge & 16) + 32 * (m >> 2);
 }
 
+// The sums of alignments up to which output (i, j) is sound (gr_sound_by the
+// terms at frequency 0), counted from GR_LOW (0: none): gt[i][jj], j = GR_BJ grp + jj, for
+// an epilogue group's columns, by the group; tmp: its transpose buffer (12.4 KB
+// of 17 KB)
+__device__ __forceinline__ void epi_table(unsigned short *gt, short *tmp, const cx<double> *ZX, const cx<double> *ZY, int d,
+                                          int log_m, int grp, int ge)
+{
+    short *tx = tmp, *ty = tmp + 64 * 65;
+    for (int i = ge >> 6; i < 64; i += 2) {
+        const int k = ge & 63;
+        tx[i * 65 + k] = (short)(i < d && k < d ? gr_log(gr_magnitude(ZX[i * d + k])) : GR_ZERO);
+    }
+    const int jj = ge & 31, j = GR_BJ * grp + jj;
+    for (int k = ge >> 5; k < d; k += 4)
+        ty[k * GR_BJ + jj] = (short)(j < d ? gr_log(gr_magnitude(ZY[k * d + j])) : GR_ZERO);
+    bar_sync(BAR_EPI + grp, NGRP);
+    for (int i0 = ge >> 5; i0 < 64; i0 += 32) {
+        int g[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) g[u] = 2 * GR_ZERO;
+        for (int k = 0; k < d; ++k) {
+            const int y = ty[k * GR_BJ + jj];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) g[u] = max(g[u], tx[(i0 + 4 * u) * 65 + k] + y);
+        }
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            const int i = i0 + 4 * u;
+            gt[i * GR_BJ + jj] = i < d && j < d ? (unsigned short)max(0, ((g[u] - 8 * log_m) >> 4) - 2 + GR_GUARD - GR_LOW)
+                                               : (unsigned short)0xffff;
+        }
+    }
+    bar_sync(BAR_EPI + grp, NGRP);
+}
+
 // FP64 outputs of one round (this thread: column j, eight rows): the
 // exponents of the row and column alignments join (with the factor
 // 1/2 of the merge and the split's 2 on both operands), then C(f) / 2 is stored
-// unmerged (phase 0) or the pair merged with it.
-__device__ __forceinline__ void epi_q(cx<double> *ZC, const double *xch, const float *fx, int ey, cx<double> wf, int64_t f,
-                                      int64_t gZ, int d, int64_t E, int j, int jl, int ge, int phase, bool self, bool two)
+// unmerged (phase 0) or the pair merged with it.  gt: column j of epi_table's;
+// returns the blocks of GR_BI rows that hold outputs not shown to be sound.
+__device__ __forceinline__ unsigned epi_q(cx<double> *ZC, const double *xch, const float *fx, int ey, cx<double> wf, int64_t f,
+                                          int64_t gZ, int d, int64_t E, int j, int jl, int ge, int phase, bool self, bool two,
+                                          const unsigned short *gt)
 {
+    unsigned mark = 0;
     constexpr int XLD = TcR<double>::XLD;
 #pragma unroll 1
     for (int m0 = 0; m0 < 8; m0 += 4) {
         cx<double> v[4], cf[4];
+        bool bad = false;
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
             const int i = epi_row<double>(ge, m0 + u);
             const int ex = __float_as_int(fx[i]), de = ex + ey - 2113;
             v[u] = {q_scale(xch[i * XLD + jl], de), q_scale(xch[(64 + i) * XLD + jl], de)};
             if (max(ex, ey) >= Q_NONFINITE) v[u].re = v[u].im = __longlong_as_double(0x7ff8000000000000ll);
+            if (self || phase == 1) bad = bad || (unsigned)(ex + ey - GR_LOW - 1) >= gt[i * GR_BJ];
             if (self) cf[u] = v[u];
             else if (phase == 1 && i < d && j < d) cf[u] = ZC[f * E + (int64_t)i * d + j];  // stored by this thread
         }
+        if (bad) mark |= 1u << (epi_row<double>(ge, m0) / GR_BI);  // (the four rows are of one block)
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
             const int i = epi_row<double>(ge, m0 + u);
@@ -778,6 +827,7 @@ __device__ __forceinline__ void epi_q(cx<double> *ZC, const double *xch, const f
             if (two) st_cx(ZC + gZ * E + (int64_t)i * d + j, zq);
         }
     }
+    return mark;
 }
 
 template <class T>
@@ -811,9 +861,11 @@ __global__ void __launch_bounds__(TcR<T>::NTHREADS, 1) tcp_kernel(const __grid_c
     __shared__ __align__(8) unsigned long long bar_xfull[NSLOT];  // XPRE: the slot's X tiles landed
     __shared__ unsigned tslot;
     __shared__ volatile int abort_flag;
+    [[maybe_unused]] __shared__ unsigned marks[2];  // FP64: blocks of the pair with unsound outputs, by epilogue group
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     if (tid == 0) {
+        if constexpr (tc_q<T>) marks[0] = marks[1] = 0u;
         for (int s = 0; s < NSLOT; ++s) {
             mbar_init(smem_u32(&bar_full[s]), NSPLIT);
             mbar_init(smem_u32(&bar_empty[s]), 1);
@@ -989,12 +1041,19 @@ __global__ void __launch_bounds__(TcR<T>::NTHREADS, 1) tcp_kernel(const __grid_c
         const int grp = (warp - WEPI0) >> 2, ge = (tid - WEPI0 * 32) & (NGRP - 1);
         T *xch = xchs + grp * L::XGRP;
         const int q = warp & 3;  // TMEM lanes 32 q .. 32 q + 31
+        [[maybe_unused]] unsigned short *const g0 = reinterpret_cast<unsigned short *>(smem + L::OFF_G0) + grp * 64 * GR_BJ;
+        [[maybe_unused]] int sg0 = -1;  // the product of the table
         int fi = 0, pl = 0;      // passes drained, pairs
         for (unsigned gp = blockIdx.x; gp < total; gp += gridDim.x, ++pl) {
             const int sg = (int)(gp / npairs);
             const int64_t p = gp - (unsigned)sg * npairs, f = p, gZ = (M - p) & (M - 1);
             cx<T> *ZC = zc_of(sg);
             const int d = d_of(sg);
+            if constexpr (tc_q<T>)
+                if (sg != sg0) {  // (while the split warps work on the CTA's first chunks)
+                    epi_table(g0, reinterpret_cast<short *>(xch), zx_of(sg), zy_of(sg), d, a.logM, grp, ge);
+                    sg0 = sg;
+                }
             const int64_t E = (int64_t)d * d;
             const int np = npass(p);
             const bool self = (M - p) == p;  // p = M/2 pairs with itself
@@ -1003,6 +1062,7 @@ __global__ void __launch_bounds__(TcR<T>::NTHREADS, 1) tcp_kernel(const __grid_c
             const cx<T> wg = c_neg(c_conj(wf));
             const float *fx = scb + 4 * 64 * (pl % L::NB) + 128, *fy = fx + 64;
             bool stop = false;
+            [[maybe_unused]] unsigned mark = 0;
             for (int phase = 0; phase < np; ++phase, ++fi) {
                 bool ok = !failed && !abort_flag && mbar_wait(smem_u32(&bar_tfull), fi & 1);
                 if (bar_or(BAR_EPI + grp, NGRP, !ok)) {
@@ -1038,7 +1098,9 @@ __global__ void __launch_bounds__(TcR<T>::NTHREADS, 1) tcp_kernel(const __grid_c
                     const int jl = ge & (XCOL - 1), j = 2 * XCOL * grp + XCOL * r + jl;
                     [[maybe_unused]] const float sj = fy[j];
                     if constexpr (tc_q<T>) {
-                        epi_q(ZC, xch, fx, __float_as_int(sj), wf, f, gZ, d, E, j, jl, ge, phase, self, two);
+                        mark |= epi_q(ZC, xch, fx, __float_as_int(sj), wf, f, gZ, d, E, j, jl, ge, phase, self, two,
+                                      g0 + (j & (GR_BJ - 1)));
+                        if (mark && r == 1) atomicOr(&marks[grp], mark);
                         bar_sync(BAR_EPI + grp, NGRP);
                         continue;
                     }
@@ -1078,6 +1140,11 @@ __global__ void __launch_bounds__(TcR<T>::NTHREADS, 1) tcp_kernel(const __grid_c
                 }
             }
             if (stop) break;
+            if constexpr (tc_q<T>)
+                if (ge == 0) {  // (the group's last barrier is behind)
+                    a.marks[2 * (int64_t)gp + grp] = (unsigned char)marks[grp];
+                    marks[grp] = 0u;
+                }
         }
     } else {
       if constexpr (EG == 2) asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(MMA_REGS));
@@ -1182,7 +1249,9 @@ cudaError_t tcp_launch(const SegParams<PairArgs> &P, int *status, cudaStream_t s
     mrc_prof_pre(kclass, st);
     k<<<grid, TcR<T>::NTHREADS, TcL<T>::SMEM, st>>>(P, status);
     mrc_prof_post(kclass, st, bytes, flops);
-    return cudaGetLastError();
+    const cudaError_t e = cudaGetLastError();
+    if (tc_q<T> && e == cudaSuccess) return mrc_pair_redo(P, kclass, st);
+    return e;
 }
 
 // The double-float X operand prepared once: for every pair of every product
@@ -1264,12 +1333,13 @@ PairArgs tcp_args(const void *zx, const void *zy, void *zc, int64_t M, int d, co
 
 template <class T>
 cudaError_t tcp_run(const void *zx, const void *zy, void *zc, int64_t M, int d, const void *tw, int tw_log,
-                    int *status, cudaStream_t st, int kclass)
+                    int *status, cudaStream_t st, int kclass, void *marks = nullptr)
 {
     SegParams<PairArgs> P{};  // the launch's parameter block (one product)
     P.nseg = 1;
     P.first[0] = 0;
     P.a[0] = tcp_args(zx, zy, zc, M, d, tw, tw_log);
+    P.a[0].marks = (unsigned char *)marks;
     return tcp_launch<T>(P, status, st, kclass);
 }
 
@@ -1299,7 +1369,7 @@ cudaError_t mrc_tcp_init(void)
                                              TcL<double>::SMEM);
         if (e != cudaSuccess) return e;
     }
-    return cudaSuccess;
+    return mrc_redo_init();
 }
 
 size_t mrc_tcp_prep_bytes(int64_t M, int d)
@@ -1343,9 +1413,9 @@ cudaError_t mrc_pairmul_f32_tcp(const void *zx, const void *zy, void *zc, int64_
 }
 
 cudaError_t mrc_pairmul_f64_tcp(const void *zx, const void *zy, void *zc, int64_t M, int d, const void *tw, int tw_log,
-                                int *status, cudaStream_t st)
+                                int *status, void *marks, cudaStream_t st)
 {
-    return tcp_run<double>(zx, zy, zc, M, d, tw, tw_log, status, st, 4);
+    return tcp_run<double>(zx, zy, zc, M, d, tw, tw_log, status, st, 4, marks);
 }
 
 cudaError_t mrc_tcp_seg(int prec, const SegParams<PairArgs> &P, int *status, cudaStream_t st)
