@@ -17,6 +17,7 @@
 #include <float.h>
 
 #include <algorithm>
+#include <atomic>
 
 #include "mrc_internal.h"
 
@@ -300,32 +301,42 @@ size_t seed_smem(int d, int m0, int CL)
     return sizeof(double) * E * (2 + 2 * (size_t)m0 + std::max(1, m0 / 2));
 }
 
+// 16 CTAs where the current device can place such a cluster, else the portable 8.
+// Function attributes and the answer belong to a device: every one is set up and
+// asked by itself (mrc_seed_init, or the first launch there).
+int query_cluster()
+{
+    if (cudaFuncSetAttribute(seed_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_MAX) != cudaSuccess ||
+        cudaFuncSetAttribute(seed_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) {
+        cudaGetLastError();
+        return 8;
+    }
+    cudaLaunchConfig_t cfg{};
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = CLMAX;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    cfg.gridDim = dim3(CLMAX);
+    cfg.blockDim = dim3(NT);
+    cfg.dynamicSmemBytes = SMEM_MAX;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    int nc = 0;
+    if (cudaOccupancyMaxActiveClusters(&nc, seed_kernel, &cfg) != cudaSuccess || nc < 1) {
+        cudaGetLastError();
+        return 8;
+    }
+    return CLMAX;
+}
+
+std::atomic<int> device_cluster[64];  // by device, 0: not asked yet
+
 int cluster_size()
 {
-    static const int n = [] {
-        // 16 CTAs where the device can place such a cluster, else the portable 8
-        if (cudaFuncSetAttribute(seed_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_MAX) != cudaSuccess ||
-            cudaFuncSetAttribute(seed_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) {
-            cudaGetLastError();
-            return 8;
-        }
-        cudaLaunchConfig_t cfg{};
-        cudaLaunchAttribute at[1];
-        at[0].id = cudaLaunchAttributeClusterDimension;
-        at[0].val.clusterDim.x = CLMAX;
-        at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
-        cfg.gridDim = dim3(CLMAX);
-        cfg.blockDim = dim3(NT);
-        cfg.dynamicSmemBytes = SMEM_MAX;
-        cfg.attrs = at;
-        cfg.numAttrs = 1;
-        int nc = 0;
-        if (cudaOccupancyMaxActiveClusters(&nc, seed_kernel, &cfg) != cudaSuccess || nc < 1) {
-            cudaGetLastError();
-            return 8;
-        }
-        return CLMAX;
-    }();
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return query_cluster();
+    int n = device_cluster[dev].load();
+    if (n == 0) device_cluster[dev].store(n = query_cluster());
     return n;
 }
 
@@ -347,7 +358,9 @@ int64_t mrc_base_size(int d, int64_t N, bool f32)
 
 cudaError_t mrc_seed_init(void)
 {
-    cluster_size();
+    int dev = 0;
+    const int n = query_cluster();
+    if (cudaGetDevice(&dev) == cudaSuccess && dev >= 0 && dev < 64) device_cluster[dev].store(n);
     return cudaFuncSetAttribute(seed_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_MAX);
 }
 
