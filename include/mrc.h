@@ -334,6 +334,17 @@ mrc_status mrc_inverse_noalloc(int d, int64_t N, const double *A, double *psi, v
 mrc_status mrc_selftest_timeout(mrc_ctx *ctx, int spins, void *stream);
 
 /*
+ * mrc_selftest_gauss_jordan -- A0^(-1) of one matrix by the kernel every inverse
+ * starts with (psi(0) = A(0)^(-1)), on a thread-block cluster of 8 or 16 CTAs
+ * instead of the size chosen for the device (16 where it can place such a
+ * cluster, else 8, which keeps the rows of d > 460 in device memory).
+ *   d : 1 <= d <= 512; A0, out : [d][d] row-major on the device, not the same
+ *       array; out is NaN where A0 is singular (and the context's status word
+ *       MRC_ERR_SINGULAR_A0)
+ */
+mrc_status mrc_selftest_gauss_jordan(mrc_ctx *ctx, int d, const double *A0, double *out, int cluster, void *stream);
+
+/*
  * Instrumentation (no counterpart in the paper; used to report the roofline
  * of one kernel class measured inside a timed region).
  *

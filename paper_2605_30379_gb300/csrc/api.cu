@@ -1764,6 +1764,17 @@ mrc_status mrc_selftest_timeout(mrc_ctx *c, int spins, void *stream)
     return MRC_OK;
 }
 
+mrc_status mrc_selftest_gauss_jordan(mrc_ctx *c, int d, const double *A0, double *out, int cluster, void *stream)
+{
+    if (!c || !A0 || !out || A0 == out || !valid_dN(d, 1) || (cluster != 8 && cluster != 16)) return MRC_ERR_INVALID_ARG;
+    cudaSetDevice(c->device);
+    auto P = std::make_unique<SegParams<SeedArgs>>();
+    P->nseg = 1;
+    P->a[0] = SeedArgs{A0, out, d, 1, c->d_status};
+    CK(mrc_seed(*P, (cudaStream_t)stream, cluster));
+    return MRC_OK;
+}
+
 mrc_status mrc_renewal_visits(mrc_ctx *c, int d, int64_t N, const double *psi, const double *alpha, const int *B,
                               int nB, double *out, void *stream)
 {

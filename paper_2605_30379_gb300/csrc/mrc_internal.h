@@ -312,7 +312,8 @@ int mrc_newton_levels(int prec, int d, int64_t N, const double *A, double *psi, 
 // psi(1) from mrc_base_case
 #define MRC_SEED_DMAX 32
 cudaError_t mrc_seed_init(void);
-cudaError_t mrc_seed(const SegParams<SeedArgs> &P, cudaStream_t st);
+// cluster: CTAs per model, 0 as the device allows (16, else 8)
+cudaError_t mrc_seed(const SegParams<SeedArgs> &P, cudaStream_t st, int cluster = 0);
 
 // misc.cu
 cudaError_t mrc_base_case(const double *A, double *psi, int d, int64_t m0, cudaStream_t st);

@@ -18,6 +18,7 @@
 
 #include <algorithm>
 #include <atomic>
+#include <initializer_list>
 
 #include "mrc_internal.h"
 
@@ -121,19 +122,24 @@ __device__ bool gj_small(const double *__restrict__ A0, double *W, int d, double
 // place: a finished column of the left block keeps the column of the right
 // block that its pivot row started, so that after the last step
 // A0^(-1)[c][perm[c']] = S[perm[c]][c'], perm[c] the pivot row of column c (rows
-// are not moved).  S: this CTA's rows rank + t CL.
-__device__ bool gj_cluster(cg::cluster_group &cl, const double *__restrict__ A0, double *__restrict__ out, double *S,
-                           int d, double tol, int CL, int rank)
+// are not moved).  S: this CTA's rows rank + t CL.  GLOBAL: the rows are those of
+// `out` instead, for matrices whose rows do not fit the cluster's shared memory (8
+// CTAs: d > 460), and S holds only the pivot rows; the cluster barriers order
+// those accesses too.
+template <bool GLOBAL>
+__device__ bool gj_cluster(cg::cluster_group &cl, const double *__restrict__ A0, double *out, double *S, int d, double tol,
+                           int CL, int rank)
 {
     __shared__ Pivot slot[2][CLMAX];
     __shared__ int perm[512];
     __shared__ double pr[2];
     __shared__ unsigned char used[512 / 8];  // of this CTA's rows (d / CL <= 64)
     const int nr = (d - rank + CL - 1) / CL, tid = threadIdx.x;
-    double *buf = S + (size_t)((d + CL - 1) / CL) * d;  // [2][d] normalised pivot rows
+    double *buf = S + (GLOBAL ? 0 : (size_t)((d + CL - 1) / CL) * d);  // [2][d] normalised pivot rows
+    auto row = [&](int r) { return GLOBAL ? out + (size_t)(rank + r * CL) * d : S + (size_t)r * d; };
     for (int t = tid; t < nr * d; t += NT) {
         const int r = t / d;
-        S[t] = A0[(size_t)(rank + r * CL) * d + (t - r * d)];
+        row(r)[t - r * d] = A0[(size_t)(rank + r * CL) * d + (t - r * d)];
     }
     if (tid < 64) used[tid] = 0;
     __syncthreads();
@@ -143,7 +149,7 @@ __device__ bool gj_cluster(cg::cluster_group &cl, const double *__restrict__ A0,
         if (tid < 32) {
             Pivot p = {-1.0, 0x7fffffff};
             for (int r = tid; r < nr; r += 32)
-                if (!used[r] && better(fabs(S[r * d + col]), rank + r * CL, p)) p = {fabs(S[r * d + col]), rank + r * CL};
+                if (!used[r] && better(fabs(row(r)[col]), rank + r * CL, p)) p = {fabs(row(r)[col]), rank + r * CL};
             p = warp_pivot(p);
             if (tid < CL) cl.map_shared_rank(&slot[0][0], tid)[b * CLMAX + rank] = p;
         }
@@ -154,9 +160,9 @@ __device__ bool gj_cluster(cg::cluster_group &cl, const double *__restrict__ A0,
         if (!(p.v > tol)) return false;
         // every CTA has read the last pivot row: its owner may now replace it
         if (prow >= 0)
-            for (int j = tid; j < d; j += NT) S[prow * d + j] = buf[(b ^ 1) * d + j];
+            for (int j = tid; j < d; j += NT) row(prow)[j] = buf[(b ^ 1) * d + j];
         const int owner = p.i % CL, lr = p.i / CL;
-        const double *src = cl.map_shared_rank(S, owner) + (size_t)lr * d;
+        const double *src = GLOBAL ? out + (size_t)p.i * d : cl.map_shared_rank(S, owner) + (size_t)lr * d;
         if (tid == 0) {
             pr[0] = src[col];
             pr[1] = 1.0 / pr[0];
@@ -177,21 +183,40 @@ __device__ bool gj_cluster(cg::cluster_group &cl, const double *__restrict__ A0,
         // one warp per row: f is read before any lane changes it
         for (int r = tid >> 5; r < nr; r += NT / 32) {
             if (r == prow) continue;
-            const double f = S[r * d + col];
+            double *s = row(r);
+            const double f = s[col];
             __syncwarp();
-            for (int j = tid & 31; j < d; j += 32) S[r * d + j] = fma(-f, buf[b * d + j], j == col ? 0.0 : S[r * d + j]);
+            for (int j = tid & 31; j < d; j += 32) s[j] = fma(-f, buf[b * d + j], j == col ? 0.0 : s[j]);
         }
         __syncthreads();
     }
     cl.sync();  // no CTA leaves while its rows are still read
     if (prow >= 0)
-        for (int j = tid; j < d; j += NT) S[prow * d + j] = buf[((d - 1) & 1) * d + j];
+        for (int j = tid; j < d; j += NT) row(prow)[j] = buf[((d - 1) & 1) * d + j];
     __syncthreads();
-    for (int c = 0; c < d; ++c)
-        if (perm[c] % CL == rank) {
-            const double *row = S + (size_t)(perm[c] / CL) * d;
-            for (int j = tid; j < d; j += NT) out[(size_t)c * d + perm[j]] = row[j];
-        }
+    if (!GLOBAL) {
+        for (int c = 0; c < d; ++c)
+            if (perm[c] % CL == rank) {
+                const double *s = row(perm[c] / CL);
+                for (int j = tid; j < d; j += NT) out[(size_t)c * d + perm[j]] = s[j];
+            }
+        return true;
+    }
+    // the columns of the own rows, then the rows column by column, in place
+    for (int r = 0; r < nr; ++r) {
+        double *s = row(r);
+        for (int j = tid; j < d; j += NT) buf[j] = s[j];
+        __syncthreads();
+        for (int j = tid; j < d; j += NT) s[perm[j]] = buf[j];
+        __syncthreads();
+    }
+    cl.sync();
+    for (int j = rank; j < d; j += CL) {
+        for (int i = tid; i < d; i += NT) buf[i] = out[(size_t)i * d + j];
+        __syncthreads();
+        for (int c = tid; c < d; c += NT) out[(size_t)c * d + j] = buf[perm[c]];
+        __syncthreads();
+    }
     return true;
 }
 
@@ -256,6 +281,11 @@ __device__ void levels(cg::cluster_group &cl, const double *As, double *Bs, doub
     }
 }
 
+// shared memory of a CTA's rows and two pivot rows (d > DSMALL), and whether a CTA has it
+__host__ __device__ inline size_t cluster_smem(int d, int CL) { return sizeof(double) * ((size_t)((d + CL - 1) / CL) * d + 2 * d); }
+__host__ __device__ inline bool cluster_fits(int d, int CL) { return cluster_smem(d, CL) <= (size_t)SMEM_MAX; }
+
+template <bool GLOBAL>
 __device__ __forceinline__ void seed_run(const SeedArgs &g)
 {
     extern __shared__ __align__(16) unsigned char smem[];
@@ -266,7 +296,10 @@ __device__ __forceinline__ void seed_run(const SeedArgs &g)
     const double nan = __longlong_as_double(0x7ff8000000000000ll);
     if (d > DSMALL) {
         cl.sync();  // every CTA of the cluster runs before any writes to another's shared memory
-        if (!gj_cluster(cl, g.A, g.psi, S, d, tol, CL, rank)) {
+        bool ok;
+        if (GLOBAL && !cluster_fits(d, CL)) ok = gj_cluster<true>(cl, g.A, g.psi, S, d, tol, CL, rank);
+        else ok = gj_cluster<false>(cl, g.A, g.psi, S, d, tol, CL, rank);
+        if (!ok) {
             if (rank == 0 && tid == 0) atomicExch(g.status, 2);
             for (int t = rank * NT + tid; t < E; t += CL * NT) g.psi[t] = nan;
             cl.sync();
@@ -289,15 +322,17 @@ __device__ __forceinline__ void seed_run(const SeedArgs &g)
     cl.sync();  // no CTA leaves while others still write to its shared memory
 }
 
+// GLOBAL: a model of the launch does not fit
+template <bool GLOBAL>
 __global__ void __launch_bounds__(NT) seed_kernel(const __grid_constant__ SegParams<SeedArgs> P, int CL)
 {
-    seed_run(P.a[blockIdx.x / CL]);
+    seed_run<GLOBAL>(P.a[blockIdx.x / CL]);
 }
 
 size_t seed_smem(int d, int m0, int CL)
 {
     const size_t E = (size_t)d * d;
-    if (d > DSMALL) return sizeof(double) * ((size_t)((d + CL - 1) / CL) * d + 2 * d);
+    if (d > DSMALL) return cluster_fits(d, CL) ? cluster_smem(d, CL) : sizeof(double) * 2 * d;
     return sizeof(double) * E * (2 + 2 * (size_t)m0 + std::max(1, m0 / 2));
 }
 
@@ -306,11 +341,12 @@ size_t seed_smem(int d, int m0, int CL)
 // asked by itself (mrc_seed_init, or the first launch there).
 int query_cluster()
 {
-    if (cudaFuncSetAttribute(seed_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_MAX) != cudaSuccess ||
-        cudaFuncSetAttribute(seed_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) {
-        cudaGetLastError();
-        return 8;
-    }
+    for (auto k : {seed_kernel<false>, seed_kernel<true>})
+        if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_MAX) != cudaSuccess ||
+            cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) {
+            cudaGetLastError();
+            return 8;
+        }
     cudaLaunchConfig_t cfg{};
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeClusterDimension;
@@ -322,7 +358,7 @@ int query_cluster()
     cfg.attrs = at;
     cfg.numAttrs = 1;
     int nc = 0;
-    if (cudaOccupancyMaxActiveClusters(&nc, seed_kernel, &cfg) != cudaSuccess || nc < 1) {
+    if (cudaOccupancyMaxActiveClusters(&nc, seed_kernel<false>, &cfg) != cudaSuccess || nc < 1) {
         cudaGetLastError();
         return 8;
     }
@@ -361,15 +397,21 @@ cudaError_t mrc_seed_init(void)
     int dev = 0;
     const int n = query_cluster();
     if (cudaGetDevice(&dev) == cudaSuccess && dev >= 0 && dev < 64) device_cluster[dev].store(n);
-    return cudaFuncSetAttribute(seed_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_MAX);
+    const cudaError_t e = cudaFuncSetAttribute(seed_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_MAX);
+    if (e != cudaSuccess) return e;
+    return cudaFuncSetAttribute(seed_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_MAX);
 }
 
-cudaError_t mrc_seed(const SegParams<SeedArgs> &P, cudaStream_t st)
+cudaError_t mrc_seed(const SegParams<SeedArgs> &P, cudaStream_t st, int cluster)
 {
     if (P.nseg <= 0) return cudaSuccess;
-    const int CL = cluster_size();
+    const int CL = cluster ? cluster : cluster_size();
     size_t sm = 0;
-    for (int s = 0; s < P.nseg; ++s) sm = std::max(sm, seed_smem(P.a[s].d, P.a[s].m0, CL));
+    bool fits = true;
+    for (int s = 0; s < P.nseg; ++s) {
+        sm = std::max(sm, seed_smem(P.a[s].d, P.a[s].m0, CL));
+        fits = fits && (P.a[s].d <= DSMALL || cluster_fits(P.a[s].d, CL));
+    }
     cudaLaunchConfig_t cfg{};
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeClusterDimension;
@@ -382,7 +424,7 @@ cudaError_t mrc_seed(const SegParams<SeedArgs> &P, cudaStream_t st)
     cfg.attrs = at;
     cfg.numAttrs = 1;
     mrc_prof_pre(7, st);
-    cudaError_t e = cudaLaunchKernelEx(&cfg, seed_kernel, P, CL);
+    cudaError_t e = cudaLaunchKernelEx(&cfg, fits ? seed_kernel<false> : seed_kernel<true>, P, CL);
     mrc_prof_post(7, st, 0, 0);
     return e != cudaSuccess ? e : cudaGetLastError();
 }

@@ -82,9 +82,10 @@ def load():
         lib.mrc_reward.argtypes = [P, I, I, I64, P, P, P, I, P]
         lib.mrc_renewal_visits.argtypes = [P, I, I64, P, P, P, I, P, P]
         lib.mrc_selftest_timeout.argtypes = [P, I, P]
+        lib.mrc_selftest_gauss_jordan.argtypes = [P, I, P, P, I, P]
         for name in ("mrc_create", "mrc_destroy", "mrc_sync_status", "mrc_inverse", "mrc_inverse_gj", "mrc_inverse_batched",
                      "mrc_residual", "mrc_transition", "mrc_first_entrance", "mrc_occupation", "mrc_reward",
-                     "mrc_renewal_visits", "mrc_selftest_timeout"):
+                     "mrc_renewal_visits", "mrc_selftest_timeout", "mrc_selftest_gauss_jordan"):
             getattr(lib, name).restype = I
         _lib = lib
         return lib
@@ -331,6 +332,16 @@ def selftest_timeout(spins=256, stream=None):
     wait on a barrier nothing arrives on gives up after `spins` rounds and
     leaves MRC_ERR_TIMEOUT in the context's status word."""
     _check(load().mrc_selftest_timeout(context(), int(spins), _stream(stream)), "mrc_selftest_timeout")
+
+
+def selftest_gauss_jordan(A0, cluster, stream=None):
+    """A0^(-1) of a [d][d] device tensor on a cluster of 8 or 16 CTAs
+    (mrc_selftest_gauss_jordan)."""
+    A0 = A0.contiguous()
+    out = torch.empty_like(A0)
+    _check(load().mrc_selftest_gauss_jordan(context(A0.device.index), A0.shape[0], _ptr(A0), _ptr(out), int(cluster),
+                                            _stream(stream)), "mrc_selftest_gauss_jordan")
+    return out
 
 
 def sync_status(stream=None):

@@ -15,38 +15,46 @@ FAKE = r"""
 #include <stddef.h>
 #include <map>
 static int dev, max_clusters[4];
-static std::map<int, int> attr[4];  // by device: attribute -> value (one kernel)
+static std::map<int, int> attrs_[4][2];  // by device and kernel: attribute -> value
+static const void *kernels[2];
+static std::map<int, int> &attr_of(const void *f)
+{
+    const int k = kernels[0] == nullptr || kernels[0] == f ? 0 : 1;
+    kernels[k] = f;
+    return attrs_[dev][k];
+}
 unsigned last_grid, last_cluster;
 size_t last_smem;
 extern "C" {
 void fake_device(int d, int clusters) { dev = d; max_clusters[d] = clusters; }
 cudaError_t cudaGetDevice(int *d) { *d = dev; return cudaSuccess; }
 cudaError_t cudaGetLastError(void) { return cudaSuccess; }
-cudaError_t cudaFuncSetAttribute(const void *, cudaFuncAttribute a, int v)
+cudaError_t cudaFuncSetAttribute(const void *f, cudaFuncAttribute a, int v)
 {
     if (a == cudaFuncAttributeMaxDynamicSharedMemorySize && v > 227 * 1024) return cudaErrorInvalidValue;
-    attr[dev][a] = v;
+    attr_of(f)[a] = v;
     return cudaSuccess;
 }
-static cudaError_t check(const cudaLaunchConfig_t *c)
+static cudaError_t check(const cudaLaunchConfig_t *c, const void *f)
 {
+    std::map<int, int> &attr = attr_of(f);
     unsigned cl = 1;
     for (unsigned i = 0; i < c->numAttrs; ++i)
         if (c->attrs[i].id == cudaLaunchAttributeClusterDimension) cl = c->attrs[i].val.clusterDim.x;
-    const size_t room = attr[dev].count(cudaFuncAttributeMaxDynamicSharedMemorySize)
-                            ? attr[dev][cudaFuncAttributeMaxDynamicSharedMemorySize] : 48 * 1024;
-    if (cl > 8 && !attr[dev][cudaFuncAttributeNonPortableClusterSizeAllowed]) return cudaErrorInvalidClusterSize;
+    const size_t room = attr.count(cudaFuncAttributeMaxDynamicSharedMemorySize)
+                            ? attr[cudaFuncAttributeMaxDynamicSharedMemorySize] : 48 * 1024;
+    if (cl > 8 && !attr[cudaFuncAttributeNonPortableClusterSizeAllowed]) return cudaErrorInvalidClusterSize;
     if (c->dynamicSmemBytes > room || c->gridDim.x % cl) return cudaErrorInvalidValue;
     last_grid = c->gridDim.x, last_cluster = cl, last_smem = c->dynamicSmemBytes;
     return cudaSuccess;
 }
-cudaError_t cudaOccupancyMaxActiveClusters(int *n, const void *, const cudaLaunchConfig_t *c)
+cudaError_t cudaOccupancyMaxActiveClusters(int *n, const void *f, const cudaLaunchConfig_t *c)
 {
-    const cudaError_t e = check(c);
+    const cudaError_t e = check(c, f);
     *n = e == cudaSuccess ? max_clusters[dev] : 0;
     return e;
 }
-cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t *c, const void *, void **) { return check(c); }
+cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t *c, const void *f, void **) { return check(c, f); }
 cudaError_t cudaLaunchKernel(const void *, dim3, dim3, void **, size_t, cudaStream_t) { return cudaErrorUnknown; }
 cudaError_t __cudaLaunchKernel(void *, dim3, dim3, void **, size_t, cudaStream_t) { return cudaErrorUnknown; }
 cudaError_t __cudaGetKernel(void **k, const void *f) { *k = (void *)f; return cudaSuccess; }
@@ -114,3 +122,13 @@ def test_every_device_gets_its_own_attributes(seed, d, init):
     assert [(g[0], g[1]) for g in got] == [(0, 0)] * 5
     assert [g[2] for g in got] == [16, 16, 8, 16, 16]
     assert all(g[3] == g[2] for g in got)
+
+
+@pytest.mark.parametrize("clusters", [0, 1])
+@pytest.mark.parametrize("d", [1, 32, 33, 460, 461, 512])
+def test_every_dimension_fits_either_cluster(seed, d, clusters):
+    """d <= 512 starts on clusters of 8 CTAs (a device that places no larger one) as
+    on 16, within the shared memory of a CTA."""
+    (init, err, cluster, grid, smem), = seed((0, clusters, 1, d, 2))
+    assert (init, err, cluster, grid) == (0, 0, 16 if clusters else 8, 16 if clusters else 8)
+    assert smem <= 216 * 1024
