@@ -2,6 +2,7 @@
 // the first coefficients of large matrices, survival
 // diagonal scans, residual norms, block gathers for first-entrance kernels and
 // the occupation / first-entrance reductions.
+#include <float.h>
 #include <math.h>
 #include "arith.cuh"
 #include "mrc_internal.h"
@@ -132,6 +133,8 @@ __device__ __forceinline__ Sum2 sum2(Sum2 a, Sum2 b)
     s.l += b.l;
     return s;
 }
+// the sum; the correction of an infinite one is a NaN (Inf - Inf)
+__device__ __forceinline__ double sum2_value(Sum2 s) { return fabs(s.h) <= DBL_MAX ? s.h + s.l : s.h; }
 
 __global__ void __launch_bounds__(256) scan_chunk_sums(const double *__restrict__ x, int ncol, int64_t N, int ch,
                                                        Sum2 *__restrict__ work)
@@ -203,8 +206,7 @@ __global__ void __launch_bounds__(256) scan_apply(double *__restrict__ x, int nc
         if (k0 + k < N) {
             run = sum2(run, x[(k0 + k) * ncol + c]);
             // offset + scale (h + l), scale = +-1
-            const Sum2 y = sum2(Sum2{scale * run.h, scale * run.l}, offset);
-            x[(k0 + k) * ncol + c] = y.h + y.l;
+            x[(k0 + k) * ncol + c] = sum2_value(sum2(Sum2{scale * run.h, scale * run.l}, offset));
         }
 }
 
