@@ -63,7 +63,7 @@ __device__ __forceinline__ void fftq_body(const FftArgs &a, int64_t j, int e0)
     cx<q64> *sm = reinterpret_cast<cx<q64> *>(smem_raw);  // [R][EC]: point rho, entry e at rho EC + e
     qtw *stw = reinterpret_cast<qtw *>(sm + R * EC);      // [R]  W_R^t
     qtw *spt = stw + R;                                   // [R]  inter-pass twiddles / 2^FIRST
-    __shared__ unsigned sexp[EC];                         // largest exponent per entry
+    __shared__ unsigned smax[EC];                         // largest magnitude (high word) per entry
     __shared__ unsigned sor[3 * EC];                      // magnitude bits after each stage but the last
     const cx<double> *tw = reinterpret_cast<const cx<double> *>(a.tw);
     const int tid = threadIdx.x, e = tid & (EC - 1);
@@ -71,7 +71,7 @@ __device__ __forceinline__ void fftq_body(const FftArgs &a, int64_t j, int e0)
     const int64_t jm = j & (a.Ns - 1);
     for (int t = tid; t < 3 * EC; t += NT) {
         sor[t] = 0u;
-        if (t < EC) sexp[t] = Q_EXMIN;
+        if (t < EC) smax[t] = 0u;
     }
     auto fill = [&]() {
         if constexpr (P::NSTAGE > 1)
@@ -119,7 +119,7 @@ __device__ __forceinline__ void fftq_body(const FftArgs &a, int64_t j, int e0)
     asm volatile("cp.async.wait_all;" ::: "memory");
     __syncthreads();
 
-    // the entry's largest exponent over the CTA's R points, and the conversion
+    // the entry's largest magnitude over the CTA's R points, and the conversion
     auto raw = [&](int i) -> cx<double> {
         return {__longlong_as_double(sm[i].re.v), __longlong_as_double(sm[i].im.v)};
     };
@@ -128,13 +128,24 @@ __device__ __forceinline__ void fftq_body(const FftArgs &a, int64_t j, int e0)
 #pragma unroll 2
         for (int i = 0; i < EPT; ++i) {
             const cx<double> x = raw(tid + i * NT);
-            m = max(m, (unsigned)max(q_exponent(x.re), q_exponent(x.im)));
+            m = max(m, max(q_magnitude(x.re), q_magnitude(x.im)));
         }
-        q_column<EC, NT, true>(m, sexp, tid);
+        q_column<EC, NT, true>(m, smax, tid);
     }
     __syncthreads();
-    int ex = (int)sexp[e];
-    if (ex == 2047) ex = Q_NONFINITE;
+    int ex = (int)(smax[e] >> 20);
+    // columns below 2^-895 (not zero) are scaled up first, where their zeros and
+    // subnormals would not shift out of the alignment
+    const bool tiny = ex < Q_TINY && smax[e] != 0u;
+    if (tiny) {
+#pragma unroll 1
+        for (int i = tid; i < R * EC; i += NT) {
+            const cx<double> x = raw(i);
+            sm[i] = {{__double_as_longlong(x.re * Q_SCALE)}, {__double_as_longlong(x.im * Q_SCALE)}};
+        }
+        ex = max(ex, 1) + Q_UP;
+    }
+    ex = ex == 2047 ? Q_NONFINITE : max(ex, Q_EXMIN);
     {
         // with inter-pass twiddles (stored as w / 2^FIRST) the points come in at
         // 2^60, else already divided by the first radix
@@ -147,6 +158,7 @@ __device__ __forceinline__ void fftq_body(const FftArgs &a, int64_t j, int e0)
             sm[tid + i * NT] = v;
         }
     }
+    if (tiny) ex -= Q_UP;
     // first stage (radix 2^FIRST, no twiddles)
     {
         constexpr int r = 1 << P::FIRST, UPT = EPT / r;

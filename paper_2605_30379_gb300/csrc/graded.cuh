@@ -72,15 +72,15 @@ __device__ __forceinline__ bool gr_sound(const short *x0, const short *y0, const
 // exponent l >> 4 (|re|, |im| of the packed values < 2^((l >> 4) - 1022)) at 2^GR_TOP; tiny
 // values are scaled up first (exact), where their zero or subnormal parts would not
 // shift out of the alignment
-constexpr int GR_TOP = 56, GR_UP = 200;
+constexpr int GR_TOP = 56;
 __device__ __forceinline__ short gr_scaled(cx<double> &za, cx<double> &zb)
 {
     unsigned b = max(gr_magnitude(za), gr_magnitude(zb));
-    if (b >= (128u << 20)) return (short)(b >> 16);
-    za = c_scal(za, 0x1p200);
-    zb = c_scal(zb, 0x1p200);
+    if (b >= ((unsigned)Q_TINY << 20)) return (short)(b >> 16);
+    za = c_scal(za, Q_SCALE);
+    zb = c_scal(zb, Q_SCALE);
     b = max(gr_magnitude(za), gr_magnitude(zb));
-    return (short)(b == 0u ? GR_ZERO : (int)(b >> 16) - 16 * GR_UP);
+    return (short)(b == 0u ? GR_ZERO : (int)(b >> 16) - 16 * Q_UP);
 }
 __device__ __forceinline__ void gr_split(cx<double> za, cx<double> zb, qtw w, short &l, qtw &f, qtw &g)
 {
@@ -109,7 +109,7 @@ __device__ __forceinline__ void gr_mac(long long &re, long long &im, const qtw &
 __device__ __forceinline__ double gr_scale(double x, int de)
 {
     const int e = ((__double2hiint(x) >> 20) & 0x7ff) + de;
-    return x == 0.0 || e >= 1 ? q_scale(x, de) : (e > -120 ? q_scale(x, de + 200) * 0x1p-200 : 0.0);
+    return x == 0.0 || e >= 1 ? q_scale(x, de) : (e > -120 ? q_scale(x, de + Q_UP) * (1.0 / Q_SCALE) : 0.0);
 }
 
 // An output's sum at one frequency, halved for q_merge, from gr_mac's sums with the

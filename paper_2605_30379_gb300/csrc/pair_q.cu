@@ -238,6 +238,7 @@ __device__ __forceinline__ void pairq_body(const PairArgs &a, int64_t p0)
         reinterpret_cast<cx<double> *>(sf)[t] = za;
         reinterpret_cast<cx<double> *>(sg)[t] = zb;
         const int rc = x ? dm.div(ee) : ee - dc.div(ee) * c;
+        // frequency 0: Y and X's diagonal
         if (q == 0 && !x) sm.y0[ee] = gr_log(gr_magnitude(ZY[ee]));
         if (q == 0 && x && ee == rc * m + min(rc, m - 1)) sm.x0[rc] = gr_log(gr_magnitude(ZX[ee]));
         atomicMax(&bnd[q * (r + c) + (x ? rc : r + rc)], max(gr_magnitude(za), gr_magnitude(zb)));
@@ -326,8 +327,17 @@ __global__ void __launch_bounds__(NT) pairdiagq_kernel(const PairArgs a)
     const cx<double> *ZX = reinterpret_cast<const cx<double> *>(a.zx), *ZY = reinterpret_cast<const cx<double> *>(a.zy);
     cx<double> *ZC = reinterpret_cast<cx<double> *>(a.zc);
     const cx<double> *tw = reinterpret_cast<const cx<double> *>(a.tw);
-    auto align = [](cx<double> za, cx<double> zb) {
-        return q_align(max(max(q_magnitude(za.re), q_magnitude(za.im)), max(q_magnitude(zb.re), q_magnitude(zb.im))));
+    // the alignment; tiny values are scaled up by 2^up for it
+    auto align = [](cx<double> &za, cx<double> &zb, int &up) {
+        unsigned b = max(gr_magnitude(za), gr_magnitude(zb));
+        up = 0;
+        if (b < ((unsigned)Q_TINY << 20) && b != 0u) {
+            up = Q_UP;
+            za = c_scal(za, Q_SCALE);
+            zb = c_scal(zb, Q_SCALE);
+            b = max(gr_magnitude(za), gr_magnitude(zb));
+        }
+        return q_align(b);
     };
     // 2 Xh(f) and 2 Xh(M - f), moduli below 2^60
     auto split = [](cx<double> za, cx<double> zb, qtw w, int ex, cx<q64> &xf, cx<q64> &xg) {
@@ -341,20 +351,22 @@ __global__ void __launch_bounds__(NT) pairdiagq_kernel(const PairArgs a)
         const int64_t f = p0 + q, g = (M - f) & (M - 1);
         const qtw w = q_twiddle(tw[f << tws], 0, false);
         if (j == 0) stw[q] = q_twiddle(c_conj(tw[f << tws]), 0, false);
-        const cx<double> za = ZY[f * c + j], zb = ZY[g * c + j];
-        const int ex = align(za, zb);
+        cx<double> za = ZY[f * c + j], zb = ZY[g * c + j];
+        int up;
+        const int ex = align(za, zb, up);
         cx<q64> vf, vg;
         split(za, zb, w, ex, vf, vg);
         yf[t] = q_limbs(vf);
         yg[t] = q_limbs(vg);
-        yex[t] = ex;
+        yex[t] = ex - up;
     }
     __syncthreads();
     for (int t = tid; t < np * E; t += NT) {
         const int q = t / E, e = t - q * E, j = e % c;
         const int64_t f = p0 + q, g = (M - f) & (M - 1);
-        const cx<double> za = ZX[f * E + e], zb = ZX[g * E + e];
-        const int ex = align(za, zb), ey = yex[q * c + j];
+        cx<double> za = ZX[f * E + e], zb = ZX[g * E + e];
+        int up;
+        const int ex = align(za, zb, up), ey = yex[q * c + j];
         const qtw wc = stw[q];  // conj w
         cx<q64> xf, xg;
         split(za, zb, qtw{wc.rh, wc.rl, -wc.ih, -wc.il}, ex, xf, xg);
@@ -363,7 +375,7 @@ __global__ void __launch_bounds__(NT) pairdiagq_kernel(const PairArgs a)
         const cx<q64> s = {{cf.re.v + cg.re.v}, {cf.im.v - cg.im.v}};
         const cx<q64> p = c_mul(cx<q64>{{cf.re.v - cg.re.v}, {cf.im.v + cg.im.v}}, wc);
         // cf = 4 C(f) 2^(2 1080 - 60 - ex - ey); the merge halves
-        const int eb = ex + ey - 2 * (Q_TOP - 2 + 1022) + Q_TOP - 3 + 1086;
+        const int eb = ex - up + ey - 2 * (Q_TOP - 2 + 1022) + Q_TOP - 3 + 1086;
         cx<double> zf = {q_encode({s.re.v - p.im.v}, eb, 0u), q_encode({s.im.v + p.re.v}, eb, 0u)};
         cx<double> zg = {q_encode({s.re.v + p.im.v}, eb, 0u), q_encode({p.re.v - s.im.v}, eb, 0u)};
         if (max(ex, ey) >= Q_NONFINITE) zf.re = zf.im = zg.re = zg.im = __longlong_as_double(0x7ff8000000000000ll);

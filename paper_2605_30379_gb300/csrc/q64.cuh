@@ -67,15 +67,15 @@ __device__ __forceinline__ int q_top30(long long a)
 }
 __device__ __forceinline__ long long q_sar30(long long a) { return q_join(q_top30(a), q_hi(a) >> 30); }
 
-// biased exponent of a double (0 for zero and subnormals, 2047 for Inf / NaN)
-__device__ __forceinline__ int q_exponent(double x) { return (__double2hiint(x) >> 20) & 0x7ff; }
-
 // x 2^(top + 1022 - ex) rounded to an integer, for |x| < 2^(ex - 1022), ex >=
 // Q_EXMIN and top <= 60: the magnitude is rounded (symmetric in the sign, so that
 // a column of one sign is not shortened; a tie, frequent where few bits are
 // dropped, goes by a mantissa bit that is kept); neg (0 or -1) flips the sign.
 // Q_EXMIN shifts zeros (and subnormals) out altogether.
 constexpr int Q_EXMIN = 64;
+// Values whose alignment would be near it are scaled up first (exact): below 2^-895 by 2^256
+constexpr int Q_TINY = 128, Q_UP = 256;
+constexpr double Q_SCALE = 0x1p256;
 __device__ __forceinline__ q64 q_decode(double x, int ex, int top, int neg = 0)
 {
     const unsigned hw = (unsigned)__double2hiint(x), lw = (unsigned)__double2loint(x);
@@ -95,32 +95,37 @@ __device__ __forceinline__ unsigned long long q_round11(unsigned long long n)
     return m + (((unsigned)n & 0x7ffu) + ((unsigned)m & 1u) > 0x400u ? 1ull : 0ull);
 }
 
-// v 2^(eb - 1086) rounded to a double (flushed to zero below the normal
-// range, infinity above it), |v| < 2^63: a value with leading bit 63 - lz gets
-// the biased exponent eb - lz.
+// The rest of q_encode, of a magnitude (out of line: one copy of the code)
+static __device__ __noinline__ double q_encode_rest(long long a, int eb)
+{
+    const int lz = __clzll(a);
+    const int e = eb - lz, u = min(max(1 - e, 0), 54);  // a subnormal drops u bits more; what falls out is kept as one bit
+    unsigned long long n = (unsigned long long)a << (lz & 63);
+    n = (n >> u) | ((n & ((1ull << u) - 1ull)) != 0ull ? 1ull : 0ull);
+    const unsigned long long m = q_round11(n);
+    if (a == 0) return 0.0;
+    if (e >= 2047) return __longlong_as_double(0x7ff0000000000000ll);
+    return __hiloint2double((int)((unsigned)(m >> 32) + ((unsigned)max(e - 1, 0) << 20)), (int)(unsigned)m);
+}
+
+// v 2^(eb - 1086) rounded to a double (gradual underflow, infinity above the
+// range), |v| < 2^63: a value with leading bit 63 - lz gets the biased exponent
+// eb - lz.
 __device__ __forceinline__ double q_encode(q64 x, int eb, unsigned sgn)
 {
     const int s = q_hi(x.v) >> 31;
     const long long a = q_join(q_lo(x.v) ^ s, q_hi(x.v) ^ s) - (long long)s;
     const unsigned sg = ((unsigned)s ^ sgn) & 0x80000000u;
-    int lz = __clz(q_hi(a)) - 1;  // leading bit to 62
     // the common case: the value's high word is not zero and no exponent between
     // eb - 63 and eb leaves the range
     if (q_hi(a) != 0 && (unsigned)(eb - 64) < 2047u - 64u) {
+        const int lz = __clz(q_hi(a)) - 1;  // leading bit to 62
         const unsigned hi = __funnelshift_l((unsigned)q_lo(a), (unsigned)q_hi(a), lz);
         const unsigned long long n = (unsigned long long)q_join(q_lo(a) << lz, (int)hi) + 0x200ull;
         return __hiloint2double((int)((unsigned)(n >> 42) + ((unsigned)(eb - 2 - lz) << 20) | sg), (int)(n >> 10));
     }
-    lz = __clzll(a);
-    const unsigned long long m = q_round11((unsigned long long)a << (lz & 63));
-    const int e = eb - lz;
-    unsigned hi = (unsigned)(m >> 32) + ((unsigned)(e - 1) << 20), lo = (unsigned)m;
-    if (e < 1 || a == 0) hi = lo = 0u;
-    if (e >= 2047) {
-        hi = a == 0 ? 0u : 0x7ff00000u;
-        lo = 0u;
-    }
-    return __hiloint2double((int)(hi | sg), (int)lo);
+    const double y = q_encode_rest(a, eb);
+    return __hiloint2double(__double2hiint(y) | (int)sg, __double2loint(y));
 }
 
 // a w for a real factor w <= 2^60 (Q60)
