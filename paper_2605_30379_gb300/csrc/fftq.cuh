@@ -133,7 +133,9 @@ __device__ __forceinline__ void fftq_body(const FftArgs &a, int64_t j, int e0)
         q_column<EC, NT, true>(m, smax, tid);
     }
     __syncthreads();
-    int ex = (int)(smax[e] >> 20);
+    // |re|, |im| <= 2^(ex - 1022) (1 + 2^-20): a largest value of one, the diagonal of e0 - q and
+    // of its inverse, does not cost its columns a bit
+    int ex = (int)((smax[e] - min(smax[e], 1u)) >> 20);
     // columns below 2^-895 (not zero) are scaled up first, where their zeros and
     // subnormals would not shift out of the alignment
     const bool tiny = ex < Q_TINY && smax[e] != 0u;
@@ -145,16 +147,16 @@ __device__ __forceinline__ void fftq_body(const FftArgs &a, int64_t j, int e0)
         }
         ex = max(ex, 1) + Q_UP;
     }
-    ex = ex == 2047 ? Q_NONFINITE : max(ex, Q_EXMIN);
+    ex = smax[e] >= 0x7ff00000u ? Q_NONFINITE : max(ex, Q_EXMIN);
     {
         // with inter-pass twiddles (stored as w / 2^FIRST) the points come in at
         // 2^60, else already divided by the first radix
-        const int top = a.Ns > 1 ? Q_TOP : Q_TOP - P::FIRST, neg = a.src_neg ? -1 : 0;
+        const int top = a.Ns > 1 ? Q_TOP : Q_TOP - P::FIRST, neg = a.src_neg ? -1 : 0, odd = tid >> P::LEC & 1;
 #pragma unroll 2
         for (int i = 0; i < EPT; ++i) {
             const cx<double> x = raw(tid + i * NT);
             cx<q64> v = {q_decode(swap ? x.im : x.re, ex, top, neg), q_decode(swap ? x.re : x.im, ex, top, neg)};
-            if (a.Ns > 1) v = c_mul(v, spt[(tid + i * NT) >> P::LEC]);
+            if (a.Ns > 1) v = c_mul(v, spt[(tid + i * NT) >> P::LEC], (1ll << 29) - (NT >> P::LEC & i ? odd ^ 1 : odd));
             sm[tid + i * NT] = v;
         }
     }
@@ -191,7 +193,9 @@ __device__ __forceinline__ void fftq_body(const FftArgs &a, int64_t j, int e0)
         const bool last = S == P::NSTAGE - 1;
         const int b = tid >> P::LEC, bm = b & ((1 << lns) - 1);
         const int qs = max(0, 64 - __clz((int)sor[(S - 1) * EC + e]) - (last ? Q_TOP - 1 : Q_TOP - 3));
-        const long long qc = q_round_start(qs);
+        // (unit twiddles, b = 0 mod 2^lns: see q_round_start)
+        const int odd = (b >> lns) & 1;
+        const long long qc = q_round_start(qs) - odd, qd = q_round_start(qs) - (odd ^ 1);
         ex += qs;
         cx<q64> v[8];
 #pragma unroll
@@ -199,7 +203,7 @@ __device__ __forceinline__ void fftq_body(const FftArgs &a, int64_t j, int e0)
         __syncthreads();  // every read done before the in-place writes
         v[0] = {{q_shift_even(v[0].re.v, qs)}, {q_shift_even(v[0].im.v, qs)}};
 #pragma unroll
-        for (int q = 1; q < 8; ++q) v[q] = q_shift(c_mul(v[q], stw[(bm * q) << (LOGR - lns - 3)], qc), qs);
+        for (int q = 1; q < 8; ++q) v[q] = q_shift(c_mul(v[q], stw[(bm * q) << (LOGR - lns - 3)], q & 1 ? qd : qc), qs);
         dft8<q64, false>(v);
         const int ob = ((b >> lns) << (lns + 3)) + bm;
         unsigned m = 0;

@@ -128,11 +128,13 @@ __device__ __forceinline__ double q_encode(q64 x, int eb, unsigned sgn)
     return __hiloint2double(__double2hiint(y) | (int)sg, __double2loint(y));
 }
 
-// a w for a real factor w <= 2^60 (Q60)
+// a w for a real factor w <= 2^60 (Q60).  (With the mean of the low product in its
+// place small values were off by up to half a unit, the positive ones all one way:
+// the inverse transform of a spectrum near one added -4e-17 up over 2^10 points.)
 __device__ __forceinline__ long long q_mul(long long a, long long w)
 {
     const int ah = q_top30(a), al = q_lo(a) & Q_MASK30, wh = (int)(w >> 30), wl = (int)w & Q_MASK30;
-    const long long mid = q_wide(al, wh, q_wide(ah, wl, (1ll << 29) + wl / 2));  // + the mean of al wl
+    const long long mid = q_wide(al, wh, q_wide(ah, wl, q_sar30(q_wide(al, wl, 1ll << 59))));
     return q_wide(ah, wh, q_sar30(mid));
 }
 
@@ -151,7 +153,10 @@ struct Ar<q64> {
 
 // a w / 2^s without its last shift: high + middle products as a 64-bit number
 // of weight 2^-s, to be shifted right by s.  c is the middle products' start:
-// q_round_start(s) rounds the result.  To it they add the mean of the low
+// q_round_start(s) rounds the result.  (A tie, which only twiddles that are powers
+// of two meet, but for those with one point in 2^s, goes up; with one less it goes
+// down.  The passes take the two in turn: all ties up made the zero frequency of
+// e0 plus a small tail 4e-16 too large at M = 2^10.)  To it they add the mean of the low
 // products that are left out (the low limbs of a are 2^29 in the mean): the same
 // twiddle serves every entry of a matrix, so that the offset would add up over a
 // row.
