@@ -134,7 +134,7 @@ __device__ __forceinline__ double q_encode(q64 x, int eb, unsigned sgn)
 __device__ __forceinline__ long long q_mul(long long a, long long w)
 {
     const int ah = q_top30(a), al = q_lo(a) & Q_MASK30, wh = (int)(w >> 30), wl = (int)w & Q_MASK30;
-    const long long mid = q_wide(al, wh, q_wide(ah, wl, q_sar30(q_wide(al, wl, 1ll << 59))));
+    const long long mid = q_wide(al, wh, q_wide(ah, wl, (long long)(int)__umulhi((unsigned)al << 2, (unsigned)wl) + (1ll << 29)));
     return q_wide(ah, wh, q_sar30(mid));
 }
 
