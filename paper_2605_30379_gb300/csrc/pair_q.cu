@@ -35,7 +35,7 @@ constexpr int NT = 128;
 // raw values below 2^top, 2 Xh below 2^(top + 2), so that m products of two
 // numbers of such moduli stay below 2^63 with their 2^60 taken off
 __device__ __forceinline__ int top_for(int m) { return m <= 4 ? 58 : (m <= 31 ? 57 : 56); }
-constexpr int SMEM_MAX = 212 * 1024;
+constexpr int PAIR_MAX = 200 * 1024, SMEM_MAX = 213 * 1024;  // of a pair; of a CTA, with the logarithms
 
 // t / d for t, d < 2^16 by a multiplication (a division by a run-time number
 // takes some 25 instructions, and every entry and output is indexed by three)
@@ -394,7 +394,12 @@ __global__ void __launch_bounds__(NT) pairq_seg_kernel(const __grid_constant__ S
 
 } // namespace
 
-bool mrc_pairq_supported(int r, int m, int c) { return cta_bytes(1, r, m, c) <= (size_t)SMEM_MAX; }
+// Besides the shared memory: sums of up to 79 terms stay below 2^63 (gr_sum; the limb
+// sums 127), and outputs are counted in 16 bits (FastDiv, the list of unsound ones)
+bool mrc_pairq_supported(int r, int m, int c)
+{
+    return m <= 79 && (int64_t)r * c < 65536 && pair_bytes(r, m, c) <= (size_t)PAIR_MAX;
+}
 
 // Pairs per CTA: outputs for every thread, but no fewer CTAs than SMs where the
 // pairs allow, and at most 48 KB of shared memory when one pair needs less
