@@ -86,9 +86,9 @@ def roofline_for(kclass, ms_total, launches, bytes_, flops, peaks, sm_mhz, d=Non
     algorithmic bytes (or flops) per launch / average launch time.  FFT
     passes, the tensor-core digit products (whose FP32 and tensor pipes are
     not the binding resource at d <= 64), the FP64 path's products (fixed point,
-    on the integer pipes or the tensor cores) and the small kernels are reported
-    against the measured HBM copy bandwidth; FP32-pipe products against the
-    FFMA peak."""
+    bound by instruction issue on the integer pipes or beside the tensor cores)
+    and the small kernels are reported against the measured HBM copy bandwidth;
+    FP32-pipe products against the FFMA peak."""
     if not launches:
         return None
     per_ms = ms_total / launches
@@ -100,7 +100,7 @@ def roofline_for(kclass, ms_total, launches, bytes_, flops, peaks, sm_mhz, d=Non
         ach = bytes_ / launches / (per_ms * 1e-3) / 1e9
         peak = peaks["hbm_gbs"]
         src = "MEASURED_PEAKS.json hbm_gbs (of measured)" + ("; tensor-core digit products" if on_tc else "; fixed-point products" if fixed else "")
-        return {"kernel": name, "bound": "hbm", "achieved": ach, "peak": peak, "unit": "GB/s",
+        return {"kernel": name, "bound": "issue" if fixed else "hbm", "achieved": ach, "peak": peak, "unit": "GB/s",
                 "frac": ach / peak, "traffic": None, "launches": launches, "avg_ms": per_ms, "peak_source": src}
     # FP32-pipe or double-float SIMT products: FP32 FFMA bound at d >= 16
     ach = flops / launches / (per_ms * 1e-3) / 1e12
@@ -114,7 +114,7 @@ def roofline_for(kclass, ms_total, launches, bytes_, flops, peaks, sm_mhz, d=Non
 # of a class stays valid while these files are unchanged.
 _CLASS_SOURCES = {
     "fft": ["kernels.cuh", "launchers.cuh", "arith.cuh", "mrc_internal.h"],
-    "tc": ["pair_tc.cu", "ozaki_tc.cu", "q64.cuh", "tcgen05.cuh", "digits.cuh", "kernels.cuh", "arith.cuh", "mrc_internal.h"],
+    "tc": ["pair_tc.cu", "ozaki_tc.cu", "graded.cuh", "q64.cuh", "tcgen05.cuh", "digits.cuh", "kernels.cuh", "arith.cuh", "mrc_internal.h"],
     "simt": ["kernels.cuh", "launchers.cuh", "arith.cuh", "mrc_internal.h"],
 }
 
@@ -127,7 +127,7 @@ def class_sources(kernel):
     if kernel in ("pairmul_dd", "pairmul_f32"):
         return _CLASS_SOURCES["tc"]
     if kernel == "pairmul_f64":
-        return _CLASS_SOURCES["tc"] + ["pair_q.cu", "launchers.cuh", "k_f64.cu"]
+        return _CLASS_SOURCES["tc"] + ["pair_q.cu", "pair_redo.cu", "graded.cuh", "launchers.cuh", "k_f64.cu"]
     return _CLASS_SOURCES["simt"] + ["k_f64.cu", "k_f32.cu", "k_dd.cu", "misc.cu", "seed.cu"]
 
 

@@ -52,7 +52,9 @@ typedef enum {
 } mrc_status;
 
 typedef enum {
-    MRC_FP64 = 0,  /* binary64 data and accuracy in every stage (its arithmetic partly in 64-bit fixed point) */
+    MRC_FP64 = 0,  /* binary64 data in every stage; transforms and products partly in 64-bit fixed point:
+                      every entry's series within about 6e-14 per product of that entry's own scale,
+                      most within binary64 rounding; magnitudes below 2^-1042 count as zero */
     MRC_MIXED = 1  /* FP32 Newton + double-float (FP32-pair) residual refinement */
 } mrc_precision;
 
@@ -60,10 +62,11 @@ typedef struct {
     int prec;               /* mrc_precision */
     int refine_sweeps;      /* MRC_MIXED: residual/correction sweeps (default 1, max 4) */
     double target_residual; /* MRC_MIXED with a report: max|rho_L| bound checked after refinement (0 = no check) */
-    int autotune;           /* 1: pick the per-frequency product kernel (FP32-pipe tile 16/32/64, or the
-                               tensor-core kernel for double-float) by timing each candidate once per
-                               (precision, shape, transform size) on the call's own stream; choices are
-                               kept in the context and, if MRC_AUTOTUNE_CACHE names a file, loaded at
+    int autotune;           /* 1: pick the FFT plans and the per-frequency product kernel (FP32 and
+                               double-float: tiles 16/24/32/64; FP64: the fixed-point product or tiles 32/64;
+                               each precision's tensor-core kernel where it exists) by timing each candidate
+                               once per (precision, shape, transform size) on the call's own stream; choices
+                               are kept in the context and, if MRC_AUTOTUNE_CACHE names a file, loaded at
                                mrc_create and written at mrc_destroy.  Batched calls tune before capture. */
 } mrc_options;
 
@@ -196,10 +199,11 @@ mrc_status mrc_inverse_host(mrc_ctx *ctx, int d, int64_t N, const double *A_host
  * Eq. (newton) to each model).
  * Scheduling, stage by stage: every launch covers all models of a wave at
  * one stage -- one launch per FFT pass of each Newton level size m (every
- * model with m0 <= m < N at once, whatever its d), one per FP32-pipe product
- * tile configuration, one for all Gauss-Jordan inverses of the A(0), one for
- * the direct recursions, one per conversion; the tensor-core products
- * (square 32 <= d, one CTA per SM) run model after model.  The residual and
+ * model with m0 <= m < N at once, whatever its d), one per product tile
+ * configuration (FP64: one for the fixed-point products), one for all first
+ * coefficients (Gauss-Jordan of the A(0) and, for d <= 32, direct sums), one for
+ * psi(1) of larger models, one per conversion; the tensor-core products of d <= 64
+ * one per K-chunk count ceil(d / 16), those of larger d model after model.  The residual and
  * correction stages group models by transform length pow2ceil(N).  Models
  * enter waves in decreasing cost (~ N d^2 (log2 N + d)) while the waves'
  * buffers (mrc_inverse_workspace_bytes per model) fit the budget: the

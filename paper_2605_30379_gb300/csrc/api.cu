@@ -211,10 +211,12 @@ size_t ws_inverse(int d, int64_t N, int prec)
     return ahat + xpre + psi32 + std::max(newton, refine);
 }
 
-// Product kernel choices: 0..2 and 4 the FP32-pipe tile configurations
-// 16/32/64 and 24 (pairmul_cfg), 3 the tensor-core digit kernel: for square 32 <= d <= 64
-// (FP64: 17 <= d) the pipelined one (pair_tc.cu), for double-float
-// 64 < d <= 512 the tiled one (ozaki_tc.cu).
+// Product kernel choices: 0..2 and 4 the tile configurations 16/32/64 and 24
+// (pairmul_cfg) on the FP32 pipes; FP64: 0 and 4 the fixed-point product
+// (pair_q.cu) where its shape is supported, 1 and 2 the tiles 32 and 64 on the FP64
+// pipe; 3 the tensor-core digit kernel: for square 32 <= d <= 64 (FP64: 17 <= d)
+// the pipelined one (pair_tc.cu), for double-float 64 < d <= 512 the tiled one
+// (ozaki_tc.cu).
 bool tensor_choice_exists(int prec, int r, int m, int c)
 {
     if (prec == PREC_F64) return mrc_tcp64_supported(r, m, c);
@@ -257,8 +259,9 @@ uint64_t tune_key(int prec, int r, int m, int c, int64_t M)
 // Autotuned product kernel for (precision, r, m, c, log2 M): every candidate
 // runs once to warm up and twice under CUDA events on the call's own buffers
 // and stream; the fastest is cached in the context.  Candidates compute the
-// same product (the tensor-core kernel only for double-float, where its
-// accuracy matches), so whichever ran last leaves a valid result behind.
+// same product to the accuracy of the precision, so whichever ran last leaves a
+// valid result behind.  (The time of an FP64 product also depends on how many of
+// its outputs are summed twice, graded.cuh.)
 // Returns -1 (use the built-in choice) when tuning is off or a graph is being
 // captured.
 int tuned_choice(mrc_ctx *cx, int prec, const void *zx, const void *zy, void *zc, int64_t M, int r, int m, int c,
@@ -269,11 +272,12 @@ int tuned_choice(mrc_ctx *cx, int prec, const void *zx, const void *zy, void *zc
     auto it = cx->tune.find(key);
     if (it != cx->tune.end()) return it->second;
     if (cx->capturing) return -1;
-    int cands[5] = {0, 1, 2, 4, 3};
-    const int nc = tensor_choice_exists(prec, r, m, c) ? 5 : 4;
+    std::vector<int> cands = {0, 1, 2, 4};
+    if (prec == PREC_F64) cands = mrc_pairq_supported(r, m, c) ? std::vector<int>{0, 1, 2} : std::vector<int>{1, 2};
+    if (tensor_choice_exists(prec, r, m, c)) cands.push_back(3);
     float best = 1e30f;
     int pick = -1;
-    for (int k = 0; k < nc; ++k) {
+    for (size_t k = 0; k < cands.size(); ++k) {
         if (launch_choice(cx, prec, cands[k], zx, zy, zc, M, r, m, c, tw, st) != cudaSuccess) continue;
         cudaEventRecord(cx->ev0, st);
         launch_choice(cx, prec, cands[k], zx, zy, zc, M, r, m, c, tw, st);
@@ -358,7 +362,8 @@ cudaError_t fft_any(mrc_ctx *cx, int prec, const FftSrc &sx, const FftDst &dx, i
 
 // The per-frequency product of one precision: the autotuned choice when the
 // call asked for tuning, else the tensor-core digit kernels where
-// tensor_default says so, the FP32- or FP64-pipe tiles elsewhere.
+// tensor_default says so, elsewhere the FP32-pipe tiles or, for FP64, the fixed-point
+// product where it fits and the FP64-pipe tiles.
 cudaError_t pairmul_any(mrc_ctx *cx, int prec, const void *zx, const void *zy, void *zc, int64_t M, int r, int m,
                         int c, const void *tw, cudaStream_t st)
 {

@@ -2,7 +2,7 @@
 // (Eq. (fft-convolution): C(phi) = X(phi) Y(phi) at every frequency of the
 // half spectrum) as exact digit products on the fifth-generation tensor
 // cores: tcgen05.mma, BF16 operands in shared memory, FP32 accumulators in
-// tensor memory (TMEM).  Square d x d with 32 <= d <= 512: 64 x 64 output
+// tensor memory (TMEM).  Square d x d with 64 < d <= 512 (pair_tc.cu below): 64 x 64 output
 // tiles (padded), K in chunks of 64 whose group sums are exact and are added
 // in the working precision; the row and column scalings are taken once per
 // frequency pair over whole rows and columns.
@@ -63,8 +63,6 @@ template <class T>
 __host__ __device__ constexpr size_t tc_xs_off() { return tc_tiles<T>(); }
 template <class T>
 __host__ __device__ constexpr size_t tc_small_bounds_off() { return tc_tiles<T>(); }
-template <class T>
-__host__ __device__ constexpr size_t tc_small_smem() { return tc_tiles<T>() + 4 * 64 * sizeof(int); }
 static_assert((size_t)128 * TC_XLD * sizeof(dd) <= (size_t)5 * (TC_A_TILE + 2 * TC_B_TILE), "exchange fits the tiles");
 template <class T>
 __host__ __device__ constexpr size_t tc_smem() { return tc_tiles<T>() + (size_t)128 * TC_XLD * sizeof(T) + 4 * TC_DMAX * sizeof(int); }
@@ -331,165 +329,7 @@ __device__ __forceinline__ void tc_split_y(const PairArgs &a, unsigned char *sBr
 __device__ __forceinline__ dd tc_scale(dd x, int e) { return {scale2(x.hi, e), scale2(x.lo, e)}; }
 __device__ __forceinline__ float tc_scale(float x, int e) { return scale2(x, e); }
 
-// d <= 64: one output tile and one K chunk per frequency; the exchange of
-// C_r and C_i reuses the digit tiles and the bounds sit right after them
-// (a smaller and tighter kernel than the tiled one below, which it matches
-// result for result).
-template <class T>
-__global__ void __launch_bounds__(TC_THREADS, 1) oztc_pairmul_kernel(PairArgs a, int *status)
-{
-    constexpr int S = OzP<T>::S, GMIN = OzP<T>::GMIN, NG = 2 * (S - 1) - GMIN + 1;
-    static_assert(NG * 64 <= (int)TC_TMEM_COLS, "group accumulators fit in TMEM");
-    extern __shared__ __align__(1024) unsigned char smem[];
-    unsigned char *sA = smem;                 // [S] 192 x 32 MN-major: -X_i, X_r, X_i
-    unsigned char *sBr = sA + S * TC_A_TILE;  // [S] 64 x 32 K-major (Y_r)
-    unsigned char *sBi = sBr + S * TC_B_TILE; // [S] 64 x 32 K-major (Y_i)
-    T *xs = reinterpret_cast<T *>(smem);      // C_r | C_i exchange (reuses the tiles)
-    unsigned *bx = reinterpret_cast<unsigned *>(smem + tc_small_bounds_off<T>());
-    unsigned *by = bx + 64;
-    int *sig = reinterpret_cast<int *>(by + 64);
-    int *tau = sig + 64;
-    __shared__ __align__(8) unsigned long long mbar;
-    __shared__ unsigned tslot;
-
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const unsigned mb = smem_u32(&mbar);
-    if (warp == 0) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(smem_u32(&tslot)),
-                     "r"(TC_TMEM_COLS)
-                     : "memory");
-        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n" ::: "memory");
-    }
-    if (tid == 0) {
-        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(mb) : "memory");
-        asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
-    }
-    tc_fence_before();
-    __syncthreads();
-    tc_fence_after();
-    const unsigned tmem = tslot;
-    unsigned parity = 0;
-    bool failed = false;
-
-    const cx<T> *ZX = reinterpret_cast<const cx<T> *>(a.zx);
-    const cx<T> *ZY = reinterpret_cast<const cx<T> *>(a.zy);
-    cx<T> *ZC = reinterpret_cast<cx<T> *>(a.zc);
-    const cx<T> *tw = reinterpret_cast<const cx<T> *>(a.tw);
-    const int d = a.r;
-    const int64_t E = (int64_t)d * d, M = a.M;
-    const int q = warp & 3, cb = (warp >> 2) * 16;  // TMEM lanes 32 q .., columns cb .. cb + 15
-
-    for (int64_t p = blockIdx.x; p < a.npairs && !failed; p += gridDim.x) {
-        const int64_t f = p, gL = M - p, gZ = gL & (M - 1);
-        const cx<T> wf = tw[f << (a.tw_log - a.logM - 1)];
-        const cx<T> wg = c_neg(c_conj(wf));
-        const bool two = (gZ != f);
-        const int nfreq = (gL == f) ? 1 : 2;  // p = M/2 pairs with itself
-
-        // ---- row bounds of X and column bounds of Y over both frequencies:
-        // |Xh(f)|, |Xh(g)| <= |Z(f)| + |Z(g)| entrywise
-        for (int t = tid; t < 128; t += TC_THREADS) bx[t] = 0u;
-        __syncthreads();
-        {
-            const int k = tid & 63;
-            float my = 0.0f;
-            for (int t = tid; t < 64 * 64; t += TC_THREADS) {
-                const int i = t >> 6;
-                float mx = 0.0f;
-                if (i < d && k < d) {
-                    const int64_t e = (int64_t)i * d + k;
-                    const cx<T> xa = ZX[f * E + e], xb = ZX[gZ * E + e];
-                    const cx<T> ya = ZY[f * E + e], yb = ZY[gZ * E + e];
-                    mx = fabsf(hi_part(xa.re)) + fabsf(hi_part(xa.im)) + fabsf(hi_part(xb.re)) +
-                         fabsf(hi_part(xb.im));
-                    my = fmaxf(my, fabsf(hi_part(ya.re)) + fabsf(hi_part(ya.im)) + fabsf(hi_part(yb.re)) +
-                                       fabsf(hi_part(yb.im)));
-                }
-                const unsigned wmx = __reduce_max_sync(0xffffffffu, __float_as_uint(mx));  // one row per warp
-                if (lane == 0) atomicMax(&bx[i], wmx);
-            }
-            atomicMax(&by[k], __float_as_uint(my));
-        }
-        __syncthreads();
-        if (tid < 64) {
-            sig[tid] = scale_exp(__uint_as_float(bx[tid]));
-            tau[tid] = scale_exp(__uint_as_float(by[tid]));
-        }
-        __syncthreads();
-
-        for (int phase = 0; phase < nfreq && !failed; ++phase) {
-            const int64_t ra = phase == 0 ? f : gZ, rb = phase == 0 ? gZ : f;
-            const cx<T> w = phase == 0 ? wf : wg;
-            for (int kh = 0; kh < 64 / TC_KH; ++kh) {
-                tc_split_x<T>(a, sA, sig, ra, rb, w, 0, kh * TC_KH, tid);
-                tc_split_y<T>(a, sBr, sBi, tau, ra, rb, w, 0, kh * TC_KH, tid);
-                asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");  // digit tiles visible to the MMAs
-                __syncthreads();
-                if (tid == 0) {
-                    tc_fence_after();
-                    tc_issue<S, GMIN>(tmem, smem_u32(sA), smem_u32(sBr), smem_u32(sBi), kh == 0);
-                    tc_commit(mb);
-                }
-                const bool ok = tc_wait(mb, parity);  // before the tiles are rewritten or the sums read
-                parity ^= 1u;
-                if (__syncthreads_or(!ok)) {
-                    failed = true;
-                    break;
-                }
-            }
-            if (failed) break;
-
-            // ---- fold the group sums of D = [C_r; C_i]; C_r and C_i meet in shared memory
-            T dv[16];
-            tc_fence_after();
-            tc_fold<T, NG>(tmem, q, cb, dv);
-            tc_fence_before();
-            __syncthreads();  // accumulators read before the next MMAs
-            {
-                const int row = 32 * q + lane;
-#pragma unroll
-                for (int c = 0; c < 16; ++c) xs[row * TC_XLD + cb + c] = dv[c];
-            }
-            __syncthreads();
-            {
-                const int i = tid & 63, jb = tid >> 6;
-#pragma unroll
-                for (int jj = 0; jj < 8; ++jj) {
-                    const int j = 8 * jb + jj;
-                    if (i >= d || j >= d) continue;
-                    // the fold factored out 2^(8 (NG - 1)) of the group weights 2^(8 (g - GMIN))
-                    const int ex = sig[i] + tau[j] + 8 * GMIN - 16 * S + 8 * (NG - 1);
-                    const cx<T> v = {tc_scale(xs[i * TC_XLD + j], ex), tc_scale(xs[(64 + i) * TC_XLD + j], ex)};
-                    const int64_t e = (int64_t)i * d + j;
-                    if (nfreq == 1) {
-                        ZC[f * E + e] = merge_real(v, v, c_conj(wf));  // p = M/2: C(g) = C(f)
-                    } else if (phase == 0) {
-                        ZC[f * E + e] = v;  // C(f), merged once C(g) is known (same thread)
-                    } else {
-                        const cx<T> cf = ZC[f * E + e];
-                        ZC[f * E + e] = merge_real(cf, v, c_conj(wf));
-                        if (two) ZC[gZ * E + e] = merge_real(v, cf, c_conj(wg));
-                    }
-                }
-            }
-            __syncthreads();  // exchange read before the next digit tiles
-        }
-    }
-
-    if (failed) {
-        if (tid == 0 && status) atomicExch(status, 6);
-        tc_wait(mb, parity);  // let MMAs still in flight finish before the TMEM is freed
-    }
-    tc_fence_before();
-    __syncthreads();
-    if (warp == 0) {
-        tc_fence_after();
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem), "r"(TC_TMEM_COLS)
-                     : "memory");
-    }
-}
-
-// d > 64: 64 x 64 output tiles and 64-deep K chunks.
+// 64 x 64 output tiles and 64-deep K chunks.
 template <class T>
 __global__ void __launch_bounds__(TC_THREADS, 1) oztc_tiled_kernel(PairArgs a, int *status)
 {
@@ -670,12 +510,7 @@ cudaError_t mrc_tc_wait_selftest(int *status, int spins, cudaStream_t st)
 
 cudaError_t mrc_tc_init(void)
 {
-    cudaError_t e = cudaFuncSetAttribute(oztc_pairmul_kernel<dd>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)tc_small_smem<dd>());
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(oztc_tiled_kernel<dd>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)tc_smem<dd>());
-    return e;
+    return cudaFuncSetAttribute(oztc_tiled_kernel<dd>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tc_smem<dd>());
 }
 
 cudaError_t mrc_pairmul_dd_tc(const void *zx, const void *zy, void *zc, int64_t M, int d, const void *tw, int tw_log,
@@ -700,8 +535,7 @@ cudaError_t mrc_pairmul_dd_tc(const void *zx, const void *zy, void *zc, int64_t 
     const double bytes = (double)M * 3.0 * d * d * sizeof(cx<T>);
     const double flops = 8.0 * d * d * d * (double)(M + 1);
     mrc_prof_pre(6, st);
-    if (d <= 64) oztc_pairmul_kernel<T><<<grid, TC_THREADS, tc_small_smem<T>(), st>>>(a, status);
-    else oztc_tiled_kernel<T><<<grid, TC_THREADS, tc_smem<T>(), st>>>(a, status);
+    oztc_tiled_kernel<T><<<grid, TC_THREADS, tc_smem<T>(), st>>>(a, status);
     mrc_prof_post(6, st, bytes, flops);
     return cudaGetLastError();
 }
