@@ -18,6 +18,16 @@ def mrc():
     return m
 
 
+def status(mrc, call, *args):
+    """The status a call raises (no exception kept: its frames would hold device tensors
+    until a later collection)."""
+    try:
+        call(*args)
+    except mrc.MrcError as e:
+        return e.status
+    return 0
+
+
 @pytest.mark.parametrize("cluster", [8, 16])
 @pytest.mark.parametrize("d", [1, 3, 32, 33, 100, 457, 459, 460, 461, 500, 512])
 def test_inverse(mrc, d, cluster):
@@ -35,14 +45,10 @@ def test_inverse(mrc, d, cluster):
 def test_singular(mrc, d, cluster):
     A = np.random.default_rng(d).standard_normal((d, d))
     A[:, d // 2] = 0.0
-    got = mrc.selftest_gauss_jordan(torch.from_numpy(A).cuda(), cluster)
-    with pytest.raises(mrc.MrcError) as ei:
-        mrc.sync_status()
-    assert ei.value.status == 2
-    assert torch.isnan(got).all()
+    assert torch.isnan(mrc.selftest_gauss_jordan(torch.from_numpy(A).cuda(), cluster)).all()
+    assert status(mrc, mrc.sync_status) == 2
 
 
 def test_arguments(mrc):
     A = torch.eye(4, dtype=torch.float64, device="cuda")
-    with pytest.raises(mrc.MrcError):
-        mrc.selftest_gauss_jordan(A, 4)
+    assert status(mrc, mrc.selftest_gauss_jordan, A, 4) == 1
