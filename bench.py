@@ -114,7 +114,7 @@ def roofline_for(kclass, ms_total, launches, bytes_, flops, peaks, sm_mhz, d=Non
 # of a class stays valid while these files are unchanged.
 _CLASS_SOURCES = {
     "fft": ["kernels.cuh", "launchers.cuh", "arith.cuh", "mrc_internal.h"],
-    "tc": ["pair_tc.cu", "ozaki_tc.cu", "graded.cuh", "q64.cuh", "tcgen05.cuh", "digits.cuh", "kernels.cuh", "arith.cuh", "mrc_internal.h"],
+    "tc": ["pair_tc.cu", "ozaki_tc.cu", "q64.cuh", "tcgen05.cuh", "digits.cuh", "kernels.cuh", "arith.cuh", "mrc_internal.h"],
     "simt": ["kernels.cuh", "launchers.cuh", "arith.cuh", "mrc_internal.h"],
 }
 

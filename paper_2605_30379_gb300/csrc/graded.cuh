@@ -23,17 +23,22 @@
 //   max_k |X_ik(p)| |Y_kj(p)|, its own terms;
 // the sum's error then stays below about 2^(GUARD - 58) of the entry's scale (2^-44,
 // 6e-14), and below 2^-53 for the entries within 2^5 of the bounds, which are most.
-// Against a 2^-94 reference, states entered with probability 1e-1 to 1e-8 (d = 4 to 64, N =
-// 2^12) come out within 7e-13 of their largest value, within 2e-13 with GUARD = 12, but
-// that sums one output in ten of a long entrance problem again (2.86 -> 3.75 ms; 2.90
-// with 14).  Weibull and Lognormal models of 5 to 64 states have unsound outputs in the
-// first few levels (M <= 64) alone: e0 - q has the identity on its diagonal there and
-// very small entries beside it (Lognormal d = 24, N = 2^12: 1.77 -> 2.14 ms).
+// Against references with 94-bit residuals, states entered with probability 1e-1 to
+// 1e-8 come out within 8e-13 of their largest value with GUARD = 14 (d = 4 to 64, N = 2^12; 9e-14
+// in floating FP64, whose error, like this one, grows with N) and within 2e-13 with 12.
+// Up to 16 terms 12 costs ordinary models nothing beyond their first levels (Lognormal d = 16,
+// N = 2^10: 0.46 -> 0.63 ms, 0.53 with 14), so they take it; an entrance with 18 x 18 blocks, N =
+// 10000, has one output in ten below 2^-12 there: 2.86 -> 3.75 ms, 2.95 with 14.  Weibull and
+// Lognormal models of 5 to 64 states have unsound outputs in the first few levels
+// (M <= 64) alone: e0 - q has the identity on its diagonal there and very small entries
+// beside it (Lognormal d = 24, N = 2^12: 1.77 -> 2.14 ms).
 #pragma once
 #include "kernels.cuh"
 #include "q64.cuh"
 
+// by the number of terms; the digit products have 17 or more
 constexpr int GR_GUARD = 14;
+__host__ __device__ constexpr int gr_guard(int m) { return m <= 16 ? 12 : GR_GUARD; }
 // alignments of a row and a column below which results may be subnormal
 constexpr int GR_LOW = 1150;
 // Logarithms: biased exponent and four bits of mantissa of the larger part's high
@@ -48,9 +53,9 @@ __device__ __forceinline__ short gr_log(unsigned m)
 
 // Whether terms of logarithm g, log_m / 2 below, show an output of alignments ax, ay to be sound
 __device__ __forceinline__ bool gr_in_range(int ax, int ay) { return min(ax, ay) > Q_EXMIN && ax + ay > GR_LOW; }
-__device__ __forceinline__ bool gr_sound_by(int ax, int ay, int g, int log_m)
+__device__ __forceinline__ bool gr_sound_by(int ax, int ay, int g, int log_m, int guard)
 {
-    return gr_in_range(ax, ay) && 16 * (ax + ay + 2 - GR_GUARD) + 8 * log_m <= g;
+    return gr_in_range(ax, ay) && 16 * (ax + ay + 2 - guard) + 8 * log_m <= g;
 }
 
 // The whole test of output (i, j).  x0, xp: logarithms of X's row i at frequency 0
@@ -65,7 +70,7 @@ __device__ __forceinline__ bool gr_sound(const short *x0, const short *y0, const
         gp = max(gp, xp[k] + yp[k * c]);
     }
     if (max(ax, ay) >= Q_NONFINITE || gp < 0) return true;  // NaN, or zero
-    return gr_sound_by(ax, ay, g0, log_m) || gr_sound_by(ax, ay, gp, 0);
+    return gr_sound_by(ax, ay, g0, log_m, gr_guard(m)) || gr_sound_by(ax, ay, gp, 0, gr_guard(m));
 }
 
 // 2 Xh(f) and 2 Xh(M - f) of an entry from its packed values, as limbs aligned to its own

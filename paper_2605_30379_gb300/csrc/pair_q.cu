@@ -256,7 +256,8 @@ __device__ __forceinline__ void pairq_body(const PairArgs &a, int64_t p0)
         sg[t] = q_limbs({{s.re.v - u.re.v}, {u.im.v - s.im.v}});
     }
     __syncthreads();
-    const float own_min = exp2f((float)(2 * top - 60 - GR_GUARD + 4));  // term_size of an output sound by its own terms
+    const int guard = gr_guard(m);
+    const float own_min = exp2f((float)(2 * top - 60 - guard + 4));  // term_size of an output sound by its own terms
     for (int t = tid; t < np * EC; t += NT) {
         const int q = dEC.div(t), e = t - q * EC, i = dc.div(e), j = e - i * c;
         const int xo = q * ex2 + i * m, yo = q * ex2 + EX + j;
@@ -275,16 +276,16 @@ __device__ __forceinline__ void pairq_body(const PairArgs &a, int64_t p0)
         // gr_sound, the likely reasons first: the term k = i at frequency 0, the terms k = i
         // and k = j of the pair itself, all terms at frequency 0
         const int ki = min(i, m - 1), kj = min(j, m - 1);
-        if (!gr_sound_by(ax, ay, sm.x0[i] + sm.y0[ki * c + j], a.logM)) {
+        if (!gr_sound_by(ax, ay, sm.x0[i] + sm.y0[ki * c + j], a.logM, guard)) {
             const float s = fmaxf(term_size(sf[xo + ki], sg[xo + ki], sf[yo + ki * c], sg[yo + ki * c]),
                                   term_size(sf[xo + kj], sg[xo + kj], sf[yo + kj * c], sg[yo + kj * c]));
             if (!gr_in_range(ax, ay) || s < own_min) {
                 int g0 = 2 * GR_ZERO;
                 for (int k = 0; k < m; ++k) g0 = max(g0, gr_log(gr_magnitude(ZX[i * m + k])) + sm.y0[k * c + j]);
-                if (!gr_sound_by(ax, ay, g0, a.logM) && max(ax, ay) < Q_NONFINITE) {
+                if (!gr_sound_by(ax, ay, g0, a.logM, guard) && max(ax, ay) < Q_NONFINITE) {
                     const int64_t f = p0 + q, g = (M - f) & (M - 1);
                     const int gp = largest_term(ZX + f * EX + i * m, ZX + g * EX + i * m, ZY + f * EY + j, ZY + g * EY + j, m, c);
-                    if (gp >= 0 && !gr_sound_by(ax, ay, gp, 0)) {
+                    if (gp >= 0 && !gr_sound_by(ax, ay, gp, 0, guard)) {
                         const int n = atomicAdd(&nredo, 1);
                         if (n < LIST) redo[n] = (unsigned short)t;
                     }
