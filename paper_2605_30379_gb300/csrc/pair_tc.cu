@@ -8,7 +8,7 @@
 //     relative to the row and column maxima.  The FP64 pipe gives two
 //     multiply-adds per clock and SM; at d = 64, N = 2^15 the inverse's 28
 //     products take 14 ms here against 138 ms on it (whole inverse 159.6 ->
-//     32.2 ms with the later steps), with smaller errors (Weibull d = 64, N = 512 against
+//     33.5 ms with the later steps), with smaller errors (Weibull d = 64, N = 512 against
 //     long double: 7.9e-16 -> 5.5e-16).  The epilogue marks blocks with outputs far
 //     below their bounds, which mrc_pair_redo sums again (graded.cuh);
 //   double-float (the residual product of Proposition 2.6): six balanced
